@@ -8,8 +8,8 @@
 // the [eq] ancestors and the psi term of one interval from device buffers the
 // caller already owns (the interval activities in, the ancestors out).  Its scratch
 // (the fixed-point weight table, the FP64 exp/expm1 tables, the activity
-// histogram, per-tile weight sums and a few scalars) lives in one file-scope
-// static __device__ array of kScratchBytes (120 KiB), held by every GPU that loads
+// histogram, per-tile weight sums and ranges and a few scalars) lives in one file-scope
+// static __device__ array of kScratchBytes (128 KiB), held by every GPU that loads
 // the library until the process exits.  Every call shares that array: the
 // histogram and scalars are cleared at the start of each call, the tables are uploaded
 // only when the bias or the weight scale differs from the last upload on that device,
@@ -36,8 +36,8 @@ constexpr int kMaxTiles = (int)(kMaxClones / kTile);        // 1024
 constexpr int kMaxDevices = 64;
 
 struct SelState {
-  int32_t dk_min, dk_max, kref, err;
-  uint32_t U, pad;
+  int32_t kref, err;
+  uint32_t U, nbins;  // [eq] offset word; histogram bins in use
   double psi_term;
 };
 
@@ -47,7 +47,8 @@ constexpr size_t kOffQ = kOffWtab + (size_t)kKcap * 8;
 constexpr size_t kOffQm1 = kOffQ + (size_t)kKcap * 8;
 constexpr size_t kOffHist = kOffQm1 + (size_t)kKcap * 8;
 constexpr size_t kOffTileSum = kOffHist + (size_t)kKcap * 4;
-constexpr size_t kOffState = kOffTileSum + (size_t)kMaxTiles * 8;
+constexpr size_t kOffTileRange = kOffTileSum + (size_t)kMaxTiles * 8;
+constexpr size_t kOffState = kOffTileRange + (size_t)kMaxTiles * 8;
 constexpr size_t kScratchBytes = kOffState + 256;
 
 static __device__ __align__(256) unsigned char g_select_scratch[kScratchBytes];
@@ -79,6 +80,7 @@ struct SelArgs {
   double* qm1tab;
   unsigned int* hist;
   unsigned long long* tile_sum;
+  int2* tile_range;  // (min, max) activity of each tile
   SelState* st;
   uint32_t nc;
   int32_t ntiles;
@@ -88,10 +90,17 @@ struct SelArgs {
   double s;
 };
 
+// Activity range of each tile, and everything that must start at zero: the histogram
+// and the error word (kernels on the caller's stream in place of a memset and a copy
+// from host memory, each of which costs as much as a launch of this kernel).
 __global__ void __launch_bounds__(kThreads) k_sel_range(SelArgs A) {
+  __shared__ int s_mn[kWarps], s_mx[kWarps];
   const int tid = threadIdx.x;
   const int64_t base = (int64_t)blockIdx.x * kTile;
+  for (int b = (int)blockIdx.x * kThreads + tid; b < kKcap; b += A.ntiles * kThreads) A.hist[b] = 0u;
+  if (blockIdx.x == 0 && tid == 0) A.st->err = 0;
   int mn = INT_MAX, mx = INT_MIN;
+#pragma unroll
   for (int i = tid; i < kTile; i += kThreads) {
     if (base + i < (int64_t)A.nc) {
       const int v = A.dK[base + i];
@@ -101,37 +110,87 @@ __global__ void __launch_bounds__(kThreads) k_sel_range(SelArgs A) {
   }
   mn = __reduce_min_sync(0xffffffffu, mn);
   mx = __reduce_max_sync(0xffffffffu, mx);
-  if ((tid & 31) == 0 && mn != INT_MAX) {
-    atomicMin(&A.st->dk_min, mn);
-    atomicMax(&A.st->dk_max, mx);
+  if ((tid & 31) == 0) {
+    s_mn[tid >> 5] = mn;
+    s_mx[tid >> 5] = mx;
+  }
+  __syncthreads();
+  if (tid == 0) {
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) {
+      mn = min(mn, s_mn[w]);
+      mx = max(mx, s_mx[w]);
+    }
+    A.tile_range[blockIdx.x] = make_int2(mn, mx);
   }
 }
 
+// Weights, tile sums and the activity histogram.  A clone's activity is counted in
+// shared memory and each block adds its few occupied bins to the global histogram:
+// nearly all of a population's clones share a dozen activities, so a global atomic per
+// clone (2^20 of them on a dozen addresses) serialised at those addresses.  The whole call
+// at the clone limit: 255 us with those and a memset and a copy in front of three kernels,
+// 46 us now, of which more than half is the read-back of the result and its wait.
 __global__ void __launch_bounds__(kThreads) k_sel_weights(SelArgs A) {
   __shared__ unsigned long long s_red[kWarps];
+  __shared__ unsigned int s_hist[kHistSmem];
+  __shared__ int s_mn[kWarps], s_mx[kWarps];
   const int tid = threadIdx.x;
   const int tile = blockIdx.x;
   const int64_t base = (int64_t)tile * kTile;
-  const int kref = A.s_neg ? A.st->dk_max : A.st->dk_min;
+  int dk[kItems];
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    const int64_t j = base + tid + i * kThreads;
+    dk[i] = j < (int64_t)A.nc ? A.dK[j] : 0;
+  }
+  int mn = INT_MAX, mx = INT_MIN;
+  for (int t = tid; t < A.ntiles; t += kThreads) {
+    const int2 r = A.tile_range[t];
+    mn = min(mn, r.x);
+    mx = max(mx, r.y);
+  }
+  mn = __reduce_min_sync(0xffffffffu, mn);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((tid & 31) == 0) {
+    s_mn[tid >> 5] = mn;
+    s_mx[tid >> 5] = mx;
+  }
+  for (int b = tid; b < kHistSmem; b += kThreads) s_hist[b] = 0u;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    mn = min(mn, s_mn[w]);
+    mx = max(mx, s_mx[w]);
+  }
+  const int kref = A.s_neg ? mx : mn;
   unsigned long long sum = 0ull;
   bool range_err = false;
-  for (int i = tid; i < kTile; i += kThreads) {
-    if (base + i < (int64_t)A.nc) {
-      const unsigned int k = abs_diff(A.dK[base + i], kref);
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    if (base + tid + i * kThreads < (int64_t)A.nc) {
+      const unsigned int k = abs_diff(dk[i], kref);
       if (k >= (unsigned int)kKcap) {
         range_err = true;
       } else {
         sum += A.wtab[k];
-        atomicAdd(&A.hist[k], 1u);
+        if (k < (unsigned int)kHistSmem) atomicAdd(&s_hist[k], 1u);
+        else atomicAdd(&A.hist[k], 1u);
       }
     }
   }
   if (range_err) A.st->err = kErrRange;
-  const unsigned long long total = block_sum_u64(sum, s_red);
+  const unsigned long long total = block_sum_u64(sum, s_red);  // and a barrier before s_hist is read
+  const int nb = hist_bins(mn, mx, kHistSmem);
+  for (int b = tid; b < nb; b += kThreads) {
+    const unsigned int c = s_hist[b];
+    if (c) atomicAdd(&A.hist[b], c);
+  }
   if (tid == 0) {
     A.tile_sum[tile] = total;
     if (tile == 0) {
       A.st->kref = kref;
+      A.st->nbins = (uint32_t)hist_bins(mn, mx, kKcap);
       A.st->U = philox4x32_10(make_uint4(0u, A.beta, 0u, kTagResample), (uint32_t)A.seed,
                               (uint32_t)(A.seed >> 32)).x;
     }
@@ -139,7 +198,6 @@ __global__ void __launch_bounds__(kThreads) k_sel_weights(SelArgs A) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_sel_ancestors(SelArgs A) {
-  __shared__ uint32_t s_jlo[kTile + 1];
   __shared__ unsigned long long s_red[kWarps];
   __shared__ unsigned long long s_wsum[kWarps];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -180,23 +238,16 @@ __global__ void __launch_bounds__(kThreads) k_sel_ancestors(SelArgs A) {
   const float ratio = __fdiv_rn((float)nc, __uint2float_rn((uint32_t)(T >> sh)));
   unsigned long long run = excl + xs - tsum;
   for (int q = 0; q < wid; ++q) run += s_wsum[q];
+  // old clone k of this tile is the ancestor of new clones [j_lo(S_k), j_lo(S_{k+1}))
+  uint32_t jl[kItems + 1];
+  j_lo_run<kItems>(run, w, T, c, nc, sh, ratio, jl);
 #pragma unroll
-  for (int i = 0; i < kItems; ++i) {
-    s_jlo[tid * kItems + i] = j_lo(run, T, c, nc, sh, ratio);
-    run += w[i];
-  }
-  if (tid == kThreads - 1) s_jlo[kTile] = j_lo(run, T, c, nc, sh, ratio);
-  __syncthreads();
-  // old clone k of this tile is the ancestor of new clones [s_jlo[k], s_jlo[k+1])
-#pragma unroll
-  for (int i = 0; i < kItems; ++i) {
-    const int k = tid * kItems + i;
-    for (uint32_t jj = s_jlo[k]; jj < s_jlo[k + 1]; ++jj) A.anc[jj] = (int32_t)(base + k);
-  }
+  for (int i = 0; i < kItems; ++i)
+    for (uint32_t jj = jl[i]; jj < jl[i + 1]; ++jj) A.anc[jj] = (int32_t)(base + tid * kItems + i);
 
   // psi term of this interval (same arithmetic as the batch path)
   if (tile == 0 && wid == 0) {
-    const int R = hist_bins(A.st->dk_min, A.st->dk_max, kKcap);
+    const int R = (int)A.st->nbins;
     double a = 0.0, q = 0.0;
     for (int b = lane; b < R; b += 32) {
       const unsigned int cnt = A.hist[b];
@@ -258,11 +309,6 @@ extern "C" int pop_select_noalloc(const int32_t* d_dK, int64_t n_clones, double 
       t_host.qm1tab[k] = std::expm1(x);
     }
   }
-  SelState st0;
-  std::memset(&st0, 0, sizeof st0);
-  st0.dk_min = INT_MAX;
-  st0.dk_max = INT_MIN;
-
   SelArgs A;
   A.dK = d_dK;
   A.anc = d_anc;
@@ -271,6 +317,7 @@ extern "C" int pop_select_noalloc(const int32_t* d_dK, int64_t n_clones, double 
   A.qm1tab = (double*)(scratch + kOffQm1);
   A.hist = (unsigned int*)(scratch + kOffHist);
   A.tile_sum = (unsigned long long*)(scratch + kOffTileSum);
+  A.tile_range = (int2*)(scratch + kOffTileRange);
   A.st = (SelState*)(scratch + kOffState);
   A.nc = (uint32_t)n_clones;
   A.ntiles = (int32_t)((n_clones + kTile - 1) / kTile);
@@ -289,9 +336,6 @@ extern "C" int pop_select_noalloc(const int32_t* d_dK, int64_t n_clones, double 
       return POP_ERR_CUDA;
     g_tables[dev] = TableKey{true, s, F};
   }
-  if (cudaMemsetAsync(A.hist, 0, (size_t)kKcap * 4, stream) != cudaSuccess ||
-      cudaMemcpyAsync(A.st, &st0, sizeof st0, cudaMemcpyHostToDevice, stream) != cudaSuccess)
-    return POP_ERR_CUDA;
   k_sel_range<<<A.ntiles, kThreads, 0, stream>>>(A);
   k_sel_weights<<<A.ntiles, kThreads, 0, stream>>>(A);
   k_sel_ancestors<<<A.ntiles, kThreads, 0, stream>>>(A);

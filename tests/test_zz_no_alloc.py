@@ -108,3 +108,22 @@ def test_select_noalloc_reports_a_spread_beyond_the_table(pg):
     w, _ = oracle.weights(0.2, dK)
     assert np.array_equal(d_anc.cpu().numpy(), oracle.ancestors(w, 2, 1))
     assert abs(term - oracle.psi_term(0.2, dK)) <= 1e-12 * abs(oracle.psi_term(0.2, dK))
+
+
+@pytest.mark.parametrize("nc,top,s", [
+    (1, 4, 0.3),          # one clone: one block clears the whole histogram
+    (1023, 3000, 0.002),  # activities beyond the bins counted in shared memory (512)
+    (1025, 600, -0.01),   # two tiles, the reference is the maximum
+    (40 * 1024, 511, 0.01),  # the last bin counted in shared memory
+])
+def test_select_noalloc_histogram_edges_match_oracle(pg, nc, top, s):
+    import torch
+    import oracle
+    dK = np.random.default_rng(nc).integers(0, top + 1, nc).astype(np.int32)
+    d_anc = torch.full((nc,), -1, dtype=torch.int32, device="cuda")
+    for interval in (1, 2):  # the second call clears what the first one counted
+        term = pg.select_noalloc(torch.from_numpy(dK).to("cuda"), s, 9, interval, d_anc)
+        w, _ = oracle.weights(s, dK)
+        assert np.array_equal(d_anc.cpu().numpy(), oracle.ancestors(w, interval, 9))
+        want = oracle.psi_term(s, dK)
+        assert abs(term - want) <= 1e-12 * abs(want)
