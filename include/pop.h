@@ -379,7 +379,7 @@ int pop_launch_count(pop_t* pop, uint64_t* h_n);
  *   d_anc       device, n_clones int32: ancestors of the new clones (output)
  *   h_psi_term  host, may be NULL: ln((1/N_c) sum_i exp(-s K_i^beta)) (output)
  * Results equal those of pop_resample for the same activities.  Scratch lives in
- * a static device array of 120 KiB that every GPU which loads the library holds
+ * a static device array of 128 KiB that every GPU which loads the library holds
  * until the process exits; each call clears what must start at zero, the array
  * keeps the last call's contents (the weight tables are re-sent only when s or the
  * weight scale of N_c changes), and calls that overlap on the GPU race on it.  The
