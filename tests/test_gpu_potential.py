@@ -128,3 +128,34 @@ def test_learned_potential_separates_and_guides_without_bias(env):
     p, _, _ = run_batch(L, N, s, dt, 1000, 16384, 32, 8000, "plain", burn=300)
     se = np.hypot(g.std(ddof=1), p.std(ddof=1)) / np.sqrt(32)
     assert abs(g.mean() - p.mean()) < 3 * se, (g.mean(), p.mean(), se)
+
+
+@pytest.mark.parametrize("L,n,copies", [
+    (9, 1, 1), (10, 63, 1), (11, 65, 1),      # groups of four windows that wrap round the ring; L mod 4 windows left over
+    (64, 64, 1), (65, 130, 1), (127, 70, 1),  # the word boundaries of the extended configuration
+    (128, 300, 2500),                         # more than one chunk of configurations per block
+])
+def test_gradient_at_the_edges_of_the_window_groups(env, L, n, copies):
+    # the batch mean over equal copies is the mean over one, so the oracle sees n configurations
+    torch, pg, potential = env
+    theta = potential.init_params(11) + np.random.default_rng(L).normal(0, 0.05, potential.N_PARAMS).astype(np.float32)
+    words, labels = batch(n, L, 100 + L)
+    tr = potential.Trainer(theta=theta)
+    loss, grad = tr.grad(torch.from_numpy(words.view(np.int64)).cuda().repeat(copies, 1),
+                         torch.from_numpy(labels).cuda().repeat(copies), L)
+    want_loss, want_grad = mlp.loss_and_grad(theta, words, labels, L, bf=True)
+    tol_loss, tol = mlp.grad_tolerance(theta, words, labels, L)
+    assert abs(loss - want_loss) <= tol_loss
+    assert np.all(np.abs(grad - want_grad) <= tol)
+    tr.close()
+
+
+def test_gradient_of_a_network_that_is_not_finite(env):
+    torch, pg, potential = env
+    theta = potential.init_params(12)
+    theta[-1] = np.nan  # every logit
+    words, labels = batch(70, 20, 3)
+    tr = potential.Trainer(theta=theta)
+    loss, grad = tr.grad(torch.from_numpy(words.view(np.int64)).cuda(), torch.from_numpy(labels).cuda(), 20)
+    assert np.isnan(loss) and np.isnan(grad[-1]) and np.isnan(grad[128 * 9 + 128:128 * 9 + 128 + 128 * 128]).all()
+    tr.close()
