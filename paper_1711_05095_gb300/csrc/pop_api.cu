@@ -218,6 +218,7 @@ struct pop_batch {
   int evolve_grid = 0;
   int evolve_grid_cap = 0;  // persistent grid at full occupancy
   size_t evolve_smem = 0;
+  int wide_unit = 0;         // wide rings: slots per warp and pass of the dynamical stage
   bool s_fixed = false;
   std::vector<double> s;
   Phase phase = kReady;
@@ -344,6 +345,25 @@ void kernel_end(pop_t* h, cudaStream_t st) {
   if (h->timer_events != nullptr) timer_record(h, st);
 }
 
+// Lanes per clone of the wide dynamical stage: 256 sites each.
+int wide_lanes(const pop_t* h) {
+  int g = 1;
+  while (256 * g < h->max_L) g *= 2;
+  return g;
+}
+
+template <bool MOD>
+void launch_wide(pop_t* h, cudaStream_t st, float dt_f) {
+  const unsigned grid = (unsigned)h->evolve_grid;
+  switch (wide_lanes(h)) {
+    case 1: k_evolve_wide<1, MOD><<<grid, kWideThreads, 0, st>>>(h->B, dt_f, h->wide_unit); break;
+    case 2: k_evolve_wide<2, MOD><<<grid, kWideThreads, 0, st>>>(h->B, dt_f, h->wide_unit); break;
+    case 4: k_evolve_wide<4, MOD><<<grid, kWideThreads, 0, st>>>(h->B, dt_f, h->wide_unit); break;
+    case 8: k_evolve_wide<8, MOD><<<grid, kWideThreads, 0, st>>>(h->B, dt_f, h->wide_unit); break;
+    default: k_evolve_wide<16, MOD><<<grid, kWideThreads, 0, st>>>(h->B, dt_f, h->wide_unit); break;
+  }
+}
+
 int launch_evolve(pop_t* h, cudaStream_t st, float dt_f) {
   const unsigned grid = (unsigned)h->evolve_grid;
   const size_t sm = h->evolve_smem;
@@ -358,11 +378,11 @@ int launch_evolve(pop_t* h, cudaStream_t st, float dt_f) {
   } else if (h->any_mod) {
     if (h->lay.W == 1) k_evolve<1, true><<<grid, kThreads, sm, st>>>(h->B, dt_f);
     else if (h->lay.W == 2) k_evolve<2, true><<<grid, kThreads, sm, st>>>(h->B, dt_f);
-    else k_evolve_wide<true><<<grid, kThreads, 0, st>>>(h->B, dt_f);
+    else launch_wide<true>(h, st, dt_f);
   } else {
     if (h->lay.W == 1) k_evolve<1, false><<<grid, kThreads, sm, st>>>(h->B, dt_f);
     else if (h->lay.W == 2) k_evolve<2, false><<<grid, kThreads, sm, st>>>(h->B, dt_f);
-    else k_evolve_wide<false><<<grid, kThreads, 0, st>>>(h->B, dt_f);
+    else launch_wide<false>(h, st, dt_f);
   }
   kernel_end(h, st);
   return cuda_status(cudaGetLastError());
@@ -417,6 +437,11 @@ int launch_resample(pop_t* h, cudaStream_t st) {
     if (h->lay.W == 1) k_select_iid<1><<<grid, kThreads, 0, st>>>(h->B);
     else if (h->lay.W == 2) k_select_iid<2><<<grid, kThreads, 0, st>>>(h->B);
     else k_select_iid<0><<<grid, kThreads, 0, st>>>(h->B);
+    kernel_end(h, st);
+  }
+  if (h->lay.W > 2) {
+    kernel_begin(h, st, POP_K_GATHER);
+    k_copy_wide<<<dim3(grid, (unsigned)h->lay.W), kThreads, 0, st>>>(h->B);
     kernel_end(h, st);
   }
   return cuda_status(cudaGetLastError());
@@ -574,15 +599,26 @@ void set_evolve_grid(pop_t* h, int grid) {
   h->B.unit_r = h->lay.nunits % grid;
 }
 
-// Rings longer than 128 sites: one warp per clone, a grid-stride loop over slots.
+// Rings longer than 128 sites: a grid-stride loop of warps over units of slots.  A unit
+// is as large as leaves a unit to every resident warp (a longer queue per warp keeps its
+// lanes busier towards the end), between the 32 / G clones a warp holds and 256.
 template <bool MOD>
 int size_evolve_grid_wide(pop_t* h) {
+  const int g = wide_lanes(h);
+  const void* f = g == 1   ? (const void*)k_evolve_wide<1, MOD>
+                  : g == 2 ? (const void*)k_evolve_wide<2, MOD>
+                  : g == 4 ? (const void*)k_evolve_wide<4, MOD>
+                  : g == 8 ? (const void*)k_evolve_wide<8, MOD>
+                           : (const void*)k_evolve_wide<16, MOD>;
   int per_sm = 0, sms = 0;
-  POP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_evolve_wide<MOD>, kThreads, 0));
+  POP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kWideThreads, 0));
   POP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
   if (per_sm < 1) per_sm = 1;
   const long long want = (long long)per_sm * sms;
-  const long long need = (h->lay.nslots + kWarps - 1) / kWarps;
+  const long long warps = kWideThreads / 32;
+  h->wide_unit = 256;
+  while (h->wide_unit > 32 / g && h->lay.nslots / h->wide_unit < want * warps) h->wide_unit /= 2;
+  const long long need = (h->lay.nslots / h->wide_unit + warps - 1) / warps;
   h->evolve_grid = (int)(want < need ? want : need);
   h->evolve_grid_cap = h->evolve_grid;
   h->evolve_smem = 0;

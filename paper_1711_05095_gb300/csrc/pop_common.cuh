@@ -48,7 +48,7 @@ constexpr int kMap = 2048;                // new slots of one tile mapped in sha
 constexpr int kScanTiles = POP_SCAN_TILES; // fused stage: k_tile_scan when every population
                                            // of the launch has more tiles
 constexpr int kMaxL = 128;                // one clone per lane: W <= 2 words
-constexpr int kMaxLWide = 4096;           // one clone per warp: 2 words per lane
+constexpr int kMaxLWide = 4096;           // 1 to 16 lanes per clone, 256 sites each
 constexpr int kInvStride = kMaxLWide + 1; // per-population 1/r table stride
 constexpr uint32_t kStepLimit = 1u << 24; // BKL steps per clone per interval
 

@@ -1065,16 +1065,12 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
       B.anc[dst] = lt * kTile + k;
     }
   } else {
-    // one warp per new clone; its lanes copy the lattice words (coalesced)
-    for (uint32_t jj = J0 + (uint32_t)wid; jj < J1; jj += NWARP) {
+    // wide lattices: the ancestors here, their words by k_copy_wide
+    for (uint32_t jj = J0 + (uint32_t)tid; jj < J1; jj += NT) {
       const int k = source(jj);
       const int64_t dst = d.off + (int64_t)jj;
-      for (int q = lane; q < B.W; q += 32)
-        B.Y[dst * B.W + q] = Xo[(base + k) * B.W + q];
-      if (lane == 0) {
-        B.KY[dst] = s_K[k];
-        B.anc[dst] = lt * kTile + k;
-      }
+      B.KY[dst] = s_K[k];
+      B.anc[dst] = lt * kTile + k;
     }
   }
   }  // [eq]
@@ -1143,7 +1139,7 @@ constexpr int kIidSmemTiles = 2048;  // tile prefixes kept in shared memory (16 
 template <int W>
 __global__ void __launch_bounds__(kThreads) k_select_iid(Batch B) {
   __shared__ unsigned long long s_te[kIidSmemTiles];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int tid = threadIdx.x;
   const int tile = blockIdx.x;
   const int p = B.tile_pop[tile];
   const PopDesc d = B.pops[p];
@@ -1162,7 +1158,7 @@ __global__ void __launch_bounds__(kThreads) k_select_iid(Batch B) {
     const int lt = tile - d.first_tile;
     const unsigned long long* S = B.S + d.off;
     const uint32_t k0 = (uint32_t)d.seed, k1 = (uint32_t)(d.seed >> 32);
-    for (int i = (W > 0 ? tid : wid); i < kTile; i += (W > 0 ? kThreads : kWarps)) {
+    for (int i = tid; i < kTile; i += kThreads) {
       const int64_t j = (int64_t)lt * kTile + i;
       if (j >= d.nc) break;
       const uint4 r = philox4x32_10(make_uint4((uint32_t)j, beta, 0u, kTagIid), k0, k1);
@@ -1179,19 +1175,13 @@ __global__ void __launch_bounds__(kThreads) k_select_iid(Batch B) {
         if (S[mid] <= alpha) lo = mid; else hi = mid - 1;
       }
       const int64_t src = d.off + lo, dst = d.off + j;
-      if constexpr (W > 0) {
+      if constexpr (W > 0) {  // wide lattices: k_copy_wide copies the words
         unsigned long long x[W];
         load_lat<W>(Xo, src, x);
         store_lat<W>(B.Y, dst, x);
-        B.KY[dst] = KXo[src];
-        B.anc[dst] = (int32_t)lo;
-      } else {
-        for (int q = lane; q < B.W; q += 32) B.Y[dst * B.W + q] = Xo[src * B.W + q];
-        if (lane == 0) {
-          B.KY[dst] = KXo[src];
-          B.anc[dst] = (int32_t)lo;
-        }
       }
+      B.KY[dst] = KXo[src];
+      B.anc[dst] = (int32_t)lo;
     }
   }
   if (blockIdx.x == gridDim.x - 1 && tid == 0) *B.beta += 1u;
@@ -1571,119 +1561,226 @@ __global__ void __launch_bounds__(kGuideThreads, W == 1 ? POP_GUIDE1_MIN_BLOCKS 
 }
 
 // ---------------------------------------------------------------------------
-// Dynamical stage for rings longer than 128 sites: one warp per clone.  Lane l
-// holds sites [128 l, 128 l + 128) in two words.  Active bonds are x XOR rot(x),
-// where the site above a lane's top bit is bit 0 of the next lane and the site
-// above L-1 is site 0.  The escape rate is a warp sum, the k-th active bond is
-// found from an exclusive prefix of the lanes' counts, and the draw, the waiting
-// time and the bond index are the same on every lane (the same arithmetic as the
-// one-clone-per-lane kernel, so results are identical to the oracle's).
+// Dynamical stage for rings longer than 128 sites: G lanes per clone (1, 2, 4, 8 or 16:
+// the smallest power of two that holds the batch's largest ring), each with 256 sites in
+// eight 32-bit words, 32 / G clones side by side in a warp.  The site above a lane's top
+// bit is bit 0 of the group's next lane and the site above L - 1 is site 0; the escape
+// rate is a sum over the group, the k-th active bond lies in the lane whose range of an
+// exclusive prefix of the lanes' counts holds k, and the draw, the waiting time and the
+// bond are the same on every lane of the group (the same arithmetic as the one-lane
+// kernels).  Steps are predicated; a group whose clone ended takes the next clone of the
+// warp's unit of `unit` slots, so a warp needs no barrier and no shared counter.
+// Bound by ALU issue: about 250 instructions per step and warp for 32 / G clones; a
+// whole warp per clone, 128 sites to a lane, took 225 for one.  2^16 clones of L = 256,
+// dt = 0.05, with the cloning stage: 301 us per interval with a warp per clone and a
+// block's own copy of its tile, 51 us now.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void wide_active(unsigned long long xl, unsigned long long xh, int L,
-                                            int lane, unsigned long long& al,
-                                            unsigned long long& ah) {
-  const unsigned long long nb = __shfl_sync(0xffffffffu, xl, (lane + 1) & 31) & 1ull;
-  const unsigned long long b0 = __shfl_sync(0xffffffffu, xl, 0) & 1ull;
-  const int last = (L - 1) >> 7, pos = (L - 1) & 127;
-  unsigned long long rl = (xl >> 1) | (xh << 63);
-  unsigned long long rh = (xh >> 1) | (nb << 63);
-  if (lane == last) {
-    if (pos < 64) rl |= b0 << pos; else rh |= b0 << (pos - 64);
-  }
-  if (lane > last) { rl = 0ull; rh = 0ull; }
-  al = xl ^ rl;
-  ah = xh ^ rh;
-}
+constexpr int kWideWords = 8;                        // 32-bit words per lane
+constexpr int kWideThreads = 128;
 
-// One BKL step of the warp's clone; returns true if it hopped (MOD: accumulate
-// the rate integral as in bkl_step).
-template <bool MOD>
-__device__ __forceinline__ bool wide_step(unsigned long long& xl, unsigned long long& xh,
-                                          float& t, float& acc, int L, int lane, const float* inv,
-                                          const float2* tab, uint32_t wa, uint32_t wb,
-                                          float dt_f) {
-  unsigned long long al, ah;
-  wide_active(xl, xh, L, lane, al, ah);
-  const int cl = __popcll(al) + __popcll(ah);
-  const int r = __reduce_add_sync(0xffffffffu, (unsigned int)cl);
-  if (r == 0) return false;
-  const float tau = __fmul_rn(neg_ln_u(wa, tab), inv[r]);
-  const float t_new = __fadd_rn(t, tau);
-  if (t_new >= dt_f) {
-    if (MOD) acc = __fmaf_rn((float)r, __fsub_rn(dt_f, t), acc);
-    return false;
-  }
-  if (MOD) acc = __fmaf_rn((float)r, tau, acc);
-  t = t_new;
-  const uint32_t k = __umulhi(wb, (uint32_t)r);
-  int incl = cl;
+// Position of the k-th set bit of the eight-word mask a (p[j] = popc(a[j])).
+__device__ __forceinline__ uint32_t kth_bond256(const uint32_t (&a)[8], const uint32_t (&p)[8], uint32_t k,
+                                                const uint8_t* kth8) {
+  const uint32_t lo = (p[0] + p[1]) + (p[2] + p[3]);
+  const bool h = k >= lo;
+  k = h ? k - lo : k;
+  uint32_t b[4], q[4];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
+  for (int j = 0; j < 4; ++j) {
+    b[j] = h ? a[4 + j] : a[j];
+    q[j] = h ? p[4 + j] : p[j];
   }
-  const int excl = incl - cl;
-  const unsigned int owner_mask = __ballot_sync(0xffffffffu, (uint32_t)excl <= k && k < (uint32_t)incl);
-  const int owner = __ffs(owner_mask) - 1;
-  int bpos = 0;
-  if (lane == owner) {
-    const uint32_t kk = k - (uint32_t)excl;
-    const uint32_t cl0 = (uint32_t)__popcll(al);
-    bpos = (kk < cl0) ? kth_set_bit64(al, kk) : 64 + kth_set_bit64(ah, kk - cl0);
-  }
-  const int b = (owner << 7) + __shfl_sync(0xffffffffu, bpos, owner);
-  const int b1 = (b + 1 == L) ? 0 : b + 1;
-  if ((b >> 7) == lane) { const int q = b & 127; if (q < 64) xl ^= 1ull << q; else xh ^= 1ull << (q - 64); }
-  if ((b1 >> 7) == lane) { const int q = b1 & 127; if (q < 64) xl ^= 1ull << q; else xh ^= 1ull << (q - 64); }
-  return true;
+  return kth_bond32<4>(b, q, k, kth8) + (h ? 128u : 0u);
 }
 
-template <bool MOD>
-__global__ void __launch_bounds__(kThreads) k_evolve_wide(Batch B, float dt_f) {
+template <int G, bool MOD>
+__global__ void __launch_bounds__(kWideThreads) k_evolve_wide(Batch B, float dt_f, int unit) {
   __shared__ float2 s_tab[64];
+  __shared__ __align__(16) uint32_t s_kth8[512];
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid < 64) s_tab[tid] = B.logtab[tid];
+  reinterpret_cast<uint4*>(s_kth8)[tid] = reinterpret_cast<const uint4*>(g_kth8.w)[tid];
   __syncthreads();
+  const uint8_t* const kth8 = reinterpret_cast<const uint8_t*>(s_kth8);
   const uint32_t beta = *B.beta;
   const int par = (int)(beta & 1u);
-  const int64_t nwarps = (int64_t)gridDim.x * kWarps;
-  for (int64_t slot = (int64_t)blockIdx.x * kWarps + (tid >> 5); slot < B.nslots; slot += nwarps) {
-    const int p = B.tile_pop[slot / kTile];
+  const int sub = lane & (G - 1);                    // the lane's place in its group
+  const int lead = lane & ~(G - 1);                  // the group's first lane
+  const uint32_t site0 = 256u * (uint32_t)sub;       // the lane's first site
+  unsigned int leaders = 0u;                         // first lanes of all groups
+#pragma unroll
+  for (int i = 0; i < 32; i += G) leaders |= 1u << i;
+  const int W = B.W;
+  const int64_t nunits = B.nslots / unit;
+  const int64_t nwarps = (int64_t)gridDim.x * (kWideThreads / 32);
+  for (int64_t un = (int64_t)blockIdx.x * (kWideThreads / 32) + (tid >> 5); un < nunits; un += nwarps) {
+    const int64_t slot0 = un * unit;                 // a unit lies within one tile
+    const int p = B.tile_pop[slot0 / kTile];
     const PopDesc d = B.pops[p];
-    const int64_t j = slot - d.off;
-    if (j >= d.nc) continue;  // padding (warp-uniform)
-    const int W = B.W;
-    unsigned long long xl = (2 * lane < W) ? B.Y[slot * W + 2 * lane] : 0ull;
-    unsigned long long xh = (2 * lane + 1 < W) ? B.Y[slot * W + 2 * lane + 1] : 0ull;
+    const int64_t j0 = slot0 - d.off;
+    const int n = (int)max((int64_t)0, min((int64_t)unit, d.nc - j0));  // warp-uniform
     const float* inv = B.inv_rate + (size_t)p * kInvStride;
     const uint32_t k0 = (uint32_t)d.seed, k1 = (uint32_t)(d.seed >> 32);
+    const uint32_t L = (uint32_t)d.L, lm1 = L - 1u;
+    int next = 0;                                    // the unit's next clone (warp-uniform)
+    int cl = -1, h = 0;
+    uint32_t q = 0u, u[8];
     float t = 0.0f, acc = 0.0f;
-    int h = 0;
-    for (uint32_t q = 0;; ++q) {
-      if (q >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
-        if (lane == 0) B.st[p].err = kErrRange;
-        break;
+    int hmin = INT_MAX, hmax = INT_MIN, amin = INT_MAX, amax = INT_MIN;
+    unsigned int ev = 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) u[j] = 0u;
+    for (;;) {
+      const unsigned int m = __ballot_sync(0xffffffffu, cl < 0) & leaders;
+      if (m != 0u && next < n) {
+        const int idx = next + __popc(m & ((1u << lead) - 1u));
+        next += __popc(m);
+        if (cl < 0 && idx < n) {
+          cl = idx;
+          const unsigned long long* src = B.Y + (slot0 + idx) * W + 4 * sub;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const unsigned long long v = 4 * sub + j < W ? src[j] : 0ull;
+            u[2 * j] = (uint32_t)v;
+            u[2 * j + 1] = (uint32_t)(v >> 32);
+          }
+          t = acc = 0.0f;
+          h = 0;
+          q = 0u;
+        }
+      } else if (m == leaders) {
+        break;  // every group is empty and the unit has run out
       }
-      const uint4 d4 = philox4x32_10(make_uint4(q, beta, (uint32_t)j, kTagEvolve), k0, k1);
-      if (!wide_step<MOD>(xl, xh, t, acc, d.L, lane, inv, s_tab, d4.x, d4.y, dt_f)) break;
-      ++h;
-      if (!wide_step<MOD>(xl, xh, t, acc, d.L, lane, inv, s_tab, d4.z, d4.w, dt_f)) break;
-      ++h;
+      const bool live = cl >= 0;
+      const uint4 d4 = philox4x32_10(make_uint4(q, beta, (uint32_t)(j0 + cl), kTagEvolve), k0, k1);
+      bool run = live;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float E = neg_ln_u(e == 0 ? d4.x : d4.z, s_tab);
+        const uint32_t wb = e == 0 ? d4.y : d4.w;
+        uint32_t nb = 0u, c0 = u[0] & 1u;            // bit 0 of the next lane, and site 0
+        if constexpr (G > 1) {
+          nb = __shfl_sync(0xffffffffu, c0, lead | ((sub + 1) & (G - 1)));
+          c0 = __shfl_sync(0xffffffffu, c0, lead);
+          if (sub == G - 1) nb = 0u;
+        }
+        uint32_t a[8], pc[8], cnt = 0u;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t up = j < 7 ? u[(j + 1) & 7] : nb;
+          // the closing bond: site L - 1's right neighbour is site 0 (the sites above L - 1 are 0)
+          a[j] = u[j] ^ __funnelshift_r(u[j], up, 1) ^ __funnelshift_lc(0u, c0, lm1 - site0 - 32u * (uint32_t)j);
+          pc[j] = (uint32_t)__popc(a[j]);
+          cnt += pc[j];
+        }
+        uint32_t r = cnt, k;
+        if constexpr (G > 1) {
+#pragma unroll
+          for (int o = 1; o < G; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+        }
+        const float tau = __fmul_rn(E, __ldg(inv + r));
+        const float t_new = __fadd_rn(t, tau);
+        const bool moving = run && r != 0u;
+        const bool hopped = moving && t_new < dt_f;
+        if (MOD) {
+          const float seg = hopped ? tau : __fsub_rn(dt_f, t);
+          acc = moving ? __fmaf_rn((float)r, seg, acc) : acc;
+        }
+        t = hopped ? t_new : t;
+        k = __umulhi(wb, r);
+        uint32_t b;
+        if constexpr (G > 1) {
+          uint32_t incl = cnt;
+#pragma unroll
+          for (int o = 1; o < G; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o, G);
+            if (sub >= o) incl += y;
+          }
+          const uint32_t excl = incl - cnt;
+          const bool owner = excl <= k && k < incl;
+          const unsigned int om = __ballot_sync(0xffffffffu, owner);
+          // a k outside the lane's count reads the table at a place inside it
+          const uint32_t mine = site0 + kth_bond256(a, pc, owner ? k - excl : 0u, kth8);
+          const unsigned int gm = (om >> lead) & (G == 32 ? 0xffffffffu : ((1u << G) - 1u));
+          b = __shfl_sync(0xffffffffu, mine, lead + (gm ? __ffs(gm) - 1 : 0));
+        } else {
+          b = kth_bond256(a, pc, k, kth8);
+        }
+        // flip sites b and (b + 1) mod L; no hop: bond 2^30, beyond every word
+        b = hopped ? b : 1u << 30;
+        const uint32_t c = b == lm1 ? 0u : b + 1u;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          u[j] ^= __funnelshift_lc(0u, 1u, b - site0 - 32u * (uint32_t)j) ^
+                  __funnelshift_lc(0u, 1u, c - site0 - 32u * (uint32_t)j);
+        h += hopped ? 1 : 0;
+        run = hopped;
+      }
+      ++q;
+      if (run && q >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
+        B.st[p].err = kErrRange;
+        run = false;
+      }
+      if (live && !run) {
+        const int64_t slot = slot0 + cl;
+        unsigned long long* dst = B.Xb[par] + slot * W + 4 * sub;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (4 * sub + j < W) dst[j] = ((unsigned long long)u[2 * j + 1] << 32) | u[2 * j];
+        if (sub == 0) {
+          B.KXb[par][slot] = B.KY[slot] + h;
+          B.dKb[par][slot] = h;
+          if (MOD) {
+            B.Ab[par][slot] = acc;
+            amin = min(amin, __float_as_int(acc));  // A >= 0: float bits order like values
+            amax = max(amax, __float_as_int(acc));
+          }
+          hmin = min(hmin, h);
+          hmax = max(hmax, h);
+          ev += (unsigned int)h;
+        }
+        cl = -1;
+      }
     }
-    if (2 * lane < W) B.Xb[par][slot * W + 2 * lane] = xl;
-    if (2 * lane + 1 < W) B.Xb[par][slot * W + 2 * lane + 1] = xh;
-    if (lane == 0) {
-      B.KXb[par][slot] = B.KY[slot] + h;
-      B.dKb[par][slot] = h;
-      atomicMin(&B.st[p].dk_min[par], h);
-      atomicMax(&B.st[p].dk_max[par], h);
-      atomicAdd(&B.st[p].events, (unsigned long long)h);
+    hmin = __reduce_min_sync(0xffffffffu, hmin);
+    hmax = __reduce_max_sync(0xffffffffu, hmax);
+    ev = __reduce_add_sync(0xffffffffu, ev);
+    if (MOD) {
+      amin = __reduce_min_sync(0xffffffffu, amin);
+      amax = __reduce_max_sync(0xffffffffu, amax);
+    }
+    if (lane == 0 && n > 0) {
+      PopState* st = B.st + p;
+      atomicMin(&st->dk_min[par], hmin);
+      atomicMax(&st->dk_max[par], hmax);
+      atomicAdd(&st->events, (unsigned long long)ev);
       if (MOD) {
-        B.Ab[par][slot] = acc;
-        atomicMin(&B.st[p].a_min[par], __float_as_int(acc));
-        atomicMax(&B.st[p].a_max[par], __float_as_int(acc));
+        atomicMin(&st->a_min[par], amin);
+        atomicMax(&st->a_max[par], amax);
       }
     }
+  }
+}
+
+// The lattices of the new clones of a wide batch, each from the ancestor the cloning
+// stage recorded: one word per thread and pass, so neighbouring threads read and write
+// neighbouring words.  Copied by the cloning stage's own block of a tile (a warp per
+// clone, one after the other) it was 64 blocks of dependent loads for 2^16 clones of
+// four words: 176 us.
+__global__ void __launch_bounds__(kThreads) k_copy_wide(Batch B) {
+  const int tile = blockIdx.x;
+  const int p = B.tile_pop[tile];
+  const PopDesc d = B.pops[p];
+  const int par = (int)(B.st[p].beta & 1u);
+  const unsigned long long* const X = B.Xb[par] + d.off * B.W;
+  const int64_t base = (int64_t)tile * kTile;
+  const int n = (int)min((int64_t)kTile, d.nc - (base - d.off));
+  const uint32_t W = (uint32_t)B.W;
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    const uint32_t e = blockIdx.y * kTile + i * kThreads + threadIdx.x;  // word of the tile
+    const uint32_t j = e / W, q = e - j * W;
+    if ((int)j < n) B.Y[(base + j) * W + q] = X[(int64_t)B.anc[base + j] * W + q];
   }
 }
 

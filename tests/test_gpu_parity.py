@@ -658,3 +658,17 @@ def test_an_interval_that_cannot_end_stops_at_the_step_limit(pg):
         b.events()
     assert e.value.status == pg.POP_ERR_RANGE
     b.close()
+
+
+@pytest.mark.parametrize("L,nc,mode,sel", [
+    (255, 33, 0, 0), (256, 1025, MOD, IID),      # one lane per clone
+    (257, 1500, MOD, 0), (512, 65, 0, IID),      # two lanes: one site in the second, both full
+    (513, 70, 0, 0), (1024, 40, MOD, 0),         # four
+    (1025, 31, MOD, IID), (2048, 17, 0, 0),      # eight
+    (2049, 9, 0, 0),                             # sixteen
+])
+def test_parity_at_the_edges_of_the_lanes_of_a_wide_ring(pg, L, nc, mode, sel):
+    # a second, short ring shares the batch: its clones leave all but the first lane empty
+    pops = [dict(L=L, N=L // 3, n_clones=nc, seed=300 + L, weight_mode=mode, selection=sel),
+            dict(L=11, N=5, n_clones=nc + 3, seed=301 + L, selection=sel)]
+    run_parity(pg, pops, [10.0 / L ** 2, -0.1], 8.0 / L, 3)
