@@ -98,6 +98,8 @@ struct PopState {
                                // histograms do not hold every clone (set by the fused
                                // stage, cleared by k_tile_scan<true>)
   unsigned long long T;        // total weight of this interval (k_tile_scan or k_gather)
+  unsigned long long pos_m;    // PosScale of T (k_tile_scan)
+  int32_t pos_sh;
 };
 
 struct Batch {
@@ -523,6 +525,55 @@ __device__ __forceinline__ void j_lo_run(unsigned long long S0, const unsigned l
     }
     out[i + 1] = (uint32_t)j;
   }
+}
+
+// ---------------------------------------------------------------------------
+// The same j_lo from fixed-point positions.  With f = F + 1 = 62 - ceil(log2 N_c)
+// fraction bits, a weight w covers the length u = w N_c 2^f / T of the line on which the
+// new slots are the multiples of 2^f, the whole line being N_c 2^f <= 2^62; j_lo(S) is the
+// first multiple at or beyond the position of S less c 2^(f - 33).  u is formed in
+// 64 bits as w times a 53-bit factor of N_c 2^f / T, so a position is at most
+// 2^-52 2^62 + 1025 (a floor per clone of the tile and one for its prefix) < 2^12 off.
+// Where a position lies kPosMargin or more from a multiple the floor is therefore exact;
+// the others (2^14 in 2^f, 2^-28 of the clones at N_c = 2^20) are settled by the 128-bit
+// comparisons of j_lo.  A clone costs one addition and one shift, where the walk with
+// 128-bit products took about 40 instructions.
+// ---------------------------------------------------------------------------
+#ifndef POP_POS_MARGIN
+#define POP_POS_MARGIN (1ull << 13)  // 2^12 and a factor of two; at most 2^31 (pos_slot)
+#endif
+constexpr unsigned long long kPosMargin = POP_POS_MARGIN;
+
+struct PosScale {
+  unsigned long long m;  // the factor's 53 bits, leading bit at 63
+  int sh;                // u = (w << sh) m / 2^64
+};
+
+__device__ __forceinline__ PosScale pos_scale(unsigned long long T, uint32_t nc, int F) {
+  if (T == 0ull) return PosScale{0ull, 0};  // no clone has a weight: no slots
+  const double kap = __ddiv_rn(__hiloint2double((1023 + F + 1) << 20, 0) * (double)nc, (double)T);
+  const unsigned long long b = (unsigned long long)__double_as_longlong(kap);
+  return PosScale{((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << 11, (int)(b >> 52) - 1023 + 1};
+}
+
+// T 2^sh <= 2^63, so no weight or prefix sum leaves 64 bits.
+__device__ __forceinline__ unsigned long long pos_of(unsigned long long w, const PosScale& k) {
+  return __umul64hi(w << k.sh, k.m);
+}
+
+// What is added to the positions of a population: the offset of the [eq] points, one slot
+// (the ceiling) and the margin (added so that one comparison sees both sides).
+__device__ __forceinline__ unsigned long long pos_offset(unsigned long long c, int F) {
+  const int f = F + 1;
+  const unsigned long long cp = f >= 33 ? c << (f - 33) : c >> (33 - f);
+  return (1ull << f) - cp + kPosMargin;
+}
+
+// The slot of a position (offset included); near is set when it is too close to call.
+__device__ __forceinline__ uint32_t pos_slot(unsigned long long q, int F, bool& near) {
+  const uint32_t hi = (uint32_t)(q >> 32), frac = hi & ((1u << (F - 31)) - 1u);
+  near = near || (frac == 0u && (uint32_t)q < (uint32_t)(2ull * kPosMargin));
+  return hi >> (F - 31);
 }
 
 // ---------------------------------------------------------------------------

@@ -535,7 +535,12 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_scan(Batch B, int pop0) {
     run += chunk;
     __syncthreads();
   }
-  if (tid == 0) B.st[p].T = run;
+  if (tid == 0) {
+    const PosScale ps = pos_scale(run, (uint32_t)d.nc, d.F);
+    B.st[p].T = run;
+    B.st[p].pos_m = ps.m;
+    B.st[p].pos_sh = ps.sh;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -595,19 +600,19 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
   __shared__ __align__(16) uint32_t s_rng[kTile + 1];
   uint32_t* const s_jlo = s_rng;
   uint16_t* const s_src = reinterpret_cast<uint16_t*>(s_rng);
-  __shared__ uint32_t s_J[2];
-  __shared__ unsigned long long s_red[SCAN ? 1 : NWARP];
+  __shared__ uint32_t s_J0, s_J1;
   __shared__ unsigned long long s_wsum[NWARP];
+  __shared__ unsigned long long s_T, s_pos0;
+  __shared__ PosScale s_ps;
   // FUSE only: the population's waiting-time factors, the log table, the Philox key
   // schedule, the slot counter and the block's activity range of the next interval
   __shared__ float s_inv[FUSE ? kMaxL + 1 : 1];
   __shared__ float2 s_logtab[FUSE ? 64 : 1];
   __shared__ uint2 s_keys[FUSE ? 10 : 1];
-  // FUSE: the first kWStage entries of the population's weight table (the activity
-  // spreads of nearly every interval), read from shared memory instead of a dependent
-  // global load (the separate cloning stage measured faster without the extra barrier)
-  constexpr int kWStage = 64;
-  __shared__ unsigned long long s_wt[FUSE ? kWStage : 1];
+  // the lengths u of the first kUStage weights of the population's table (the activity
+  // spreads of nearly every interval)
+  constexpr int kUStage = 64;
+  __shared__ unsigned long long s_u[kUStage];
   __shared__ __align__(16) uint32_t s_kth8[FUSE ? 512 : 1];
   // FUSE, plain weights: activity histograms of the first three tiles the new clones
   // fall in (the rest go straight to global memory)
@@ -654,7 +659,6 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
   }
 
   const unsigned long long* wt = B.wtab + (size_t)p * kKcap;
-  if (FUSE && tid < kWStage) s_wt[tid] = wt[tid];
   // independent loads first: activities and the old clones of this tile
   int dkv[NI];
 #pragma unroll
@@ -689,131 +693,145 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
   const float a_ref = st->a_ref;
   const unsigned long long c = 2ull * (unsigned long long)st->U + 1ull;
 
-  // population total T and this tile's exclusive prefix
-  unsigned long long T = 0ull, excl = 0ull, tT = 0ull, tE = 0ull;
-  if constexpr (SCAN) {
-    T = st->T;
-    excl = B.tile_excl[tile];
-  } else {
-    for (int i = tid; i < d.ntiles; i += NT) {
-      const unsigned long long v = B.tile_sum[d.first_tile + i];
-      tT += v;
-      if (i < lt) tE += v;
-    }
-  }
-
-  // weights of this tile's clones and their scan within each warp
-  if constexpr (FUSE) __syncthreads();  // s_wt
-  unsigned long long w[NI];
-  unsigned long long tsum = 0ull;
-#pragma unroll
-  for (int i = 0; i < NI; ++i) {
-    w[i] = 0ull;
-    if (j0 + i < d.nc) {
-      if (FUSE && !d.modified) {  // plain: wtab[|dK - k_ref|] (0 beyond the table: k_weights reports it)
-        const unsigned int k = abs_diff(dkv[i], kref);
-        w[i] = k < (unsigned int)kWStage ? s_wt[k] : (k < (unsigned int)kKcap ? __ldg(wt + k) : 0ull);
-      } else {
-        unsigned int k;
-        clone_weight(d, dkv[i], kref, av[i], a_ref, wt, B.exp2tab, w[i], k);
+  // warp 0: the total T, this tile's exclusive prefix and position, and the lengths of
+  // the first weights, from k_tile_scan's sums or from the tile sums themselves
+  if (wid == 0) {
+    unsigned long long T, excl = 0ull;
+    PosScale ps;
+    const unsigned long long w0 = wt[lane], w1 = wt[lane + 32];
+    if constexpr (SCAN) {
+      T = st->T;
+      excl = B.tile_excl[tile];
+      ps = PosScale{st->pos_m, st->pos_sh};
+    } else {
+      T = 0ull;
+      for (int i = lane; i < d.ntiles; i += 32) {
+        const unsigned long long v = B.tile_sum[d.first_tile + i];
+        T += v;
+        if (i < lt) excl += v;
       }
+      T = warp_sum_u64(T);
+      excl = warp_sum_u64(excl);
+      ps = pos_scale(T, nc, d.F);
     }
-    tsum += w[i];
-  }
-  unsigned long long xs = tsum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long y = __shfl_up_sync(0xffffffffu, xs, o);
-    if (lane >= o) xs += y;
-  }
-  if (lane == 31) s_wsum[wid] = xs;
-  if constexpr (SCAN) {
-    __syncthreads();
-  } else {
-    T = block_sum_u64_n<NWARP>(tT, s_red);
-    excl = block_sum_u64_n<NWARP>(tE, s_red);
-  }
-
-  const int sh = max(0, 64 - __clzll((long long)T) - 24);
-  const float ratio = __fdiv_rn((float)nc, __uint2float_rn((uint32_t)(T >> sh)));
-  unsigned long long run = excl + xs - tsum;
-  for (int q = 0; q < wid; ++q) run += s_wsum[q];
-  if (d.iid) {
-    // [iid]: publish this tile's prefix sums; k_select_iid draws the points
-#pragma unroll
-    for (int i = 0; i < NI; ++i) {
-      B.S[base + (int64_t)tid * NI + i] = run;
-      run += w[i];
+    s_u[lane] = pos_of(w0, ps);
+    s_u[lane + 32] = pos_of(w1, ps);
+    if (lane == 0) {
+      s_T = T;
+      s_pos0 = pos_of(excl, ps) + pos_offset(c, d.F);
+      s_ps = ps;
     }
-    if (lt == 0 && tid == 0) st->T = T;
-  } else {
-  uint32_t jl[NI + 1];
-  j_lo_run<NI>(run, w, T, c, nc, sh, ratio, jl);
-  if (tid == 0) s_J[0] = jl[0];
-  if (tid == NT - 1) s_J[1] = jl[NI];
+  }
   __syncthreads();
 
-  const uint32_t J0 = s_J[0], J1 = s_J[1];
-  const bool mapped = (J1 - J0) <= (uint32_t)kMap;
-  if (FUSE && mapped) {
-    // the thread's old clones own the new slots [jl[0], jl[NI]): a marker at the first
-    // slot of each old clone with copies, then an inclusive max scan over the slots
-    // (markers grow with the slot, and the first slot always has one); no divergent
-    // loops, at the cost of two more barriers (the separate cloning stage, bound by
-    // memory, measured faster with the loops below)
-    constexpr int SP = kMap / NT;  // slots per thread in the scan
-    static_assert(SP % 8 == 0, "whole 16-byte words of the map per thread");
-    const int nsl = (int)(J1 - J0);
-    for (int e = tid; e < kMap / 2; e += NT) s_rng[e] = 0u;
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < NI; ++i)
-      if (jl[i + 1] > jl[i]) s_src[jl[i] - J0] = (uint16_t)(tid * NI + i);
-    __syncthreads();
-    uint4 pk[SP / 8];
-    int m = 0;
-#pragma unroll
-    for (int v = 0; v < SP / 8; ++v) {
-      pk[v] = reinterpret_cast<const uint4*>(s_src)[tid * (SP / 8) + v];
-      const uint32_t wd[4] = {pk[v].x, pk[v].y, pk[v].z, pk[v].w};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) m = max(m, (int)max(wd[q] & 0xffffu, wd[q] >> 16));
-    }
-    int inc = m;
+  // the exact weight of one of this thread's clones
+  auto weight = [&](int i) -> unsigned long long {
+    unsigned long long w = 0ull;
+    unsigned int k;
+    if (j0 + i < d.nc) clone_weight(d, dkv[i], kref, av[i], a_ref, wt, B.exp2tab, w, k);
+    return w;
+  };
+  // inclusive scan over the threads of a warp, then the sums of the earlier warps
+  auto scan_block = [&](unsigned long long v) -> unsigned long long {
+    unsigned long long xs = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc = max(inc, y);
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, xs, o);
+      if (lane >= o) xs += y;
     }
-    __shared__ int s_mx[NWARP];
-    if (lane == 31) s_mx[wid] = inc;
-    int run = __shfl_up_sync(0xffffffffu, inc, 1);
-    if (lane == 0) run = 0;
+    if (lane == 31) s_wsum[wid] = xs;
     __syncthreads();
-    for (int q = 0; q < wid; ++q) run = max(run, s_mx[q]);
+    unsigned long long before = xs - v;
+    for (int q = 0; q < wid; ++q) before += s_wsum[q];
+    return before;
+  };
+  uint32_t J0 = 0u, J1 = 0u;
+  uint32_t jl[NI + 1];
+  bool near = false;
+  // the map from new slot to old clone: the thread's old clones own the new slots
+  // [jl[0], jl[NI]), nearly always one or two each
+  auto fill_map = [&]() {
 #pragma unroll
-    for (int v = 0; v < SP / 8; ++v) {
-      uint32_t wd[4] = {pk[v].x, pk[v].y, pk[v].z, pk[v].w};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        run = max(run, (int)(wd[q] & 0xffffu));
-        const uint32_t lo = (uint32_t)run;
-        run = max(run, (int)(wd[q] >> 16));
-        wd[q] = lo | ((uint32_t)run << 16);
-      }
-      if (tid * SP + 8 * v < nsl) reinterpret_cast<uint4*>(s_src)[tid * (SP / 8) + v] = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+    for (int i = 0; i < NI; ++i) {
+      const uint32_t a = jl[i] - J0, b = min(jl[i + 1] - J0, (uint32_t)kMap);
+      const uint16_t k = (uint16_t)(tid * NI + i);
+      if (a < b) s_src[a] = k;
+      if (a + 1u < b) s_src[a + 1u] = k;
+      for (uint32_t e = a + 2u; e < b; ++e) s_src[e] = k;
     }
-  } else if (mapped) {
-    // the thread's old clones own the new slots [jl[0], jl[NI]), held in its registers
+    if (tid == NT - 1) s_J1 = jl[NI];
+  };
+  if (!d.iid) {
+    unsigned long long u[NI], sum = 0ull;
 #pragma unroll
-    for (int i = 0; i < NI; ++i)
-      for (uint32_t jj = jl[i]; jj < jl[i + 1]; ++jj) s_src[jj - J0] = (uint16_t)(tid * NI + i);
-  } else {
+    for (int i = 0; i < NI; ++i) {
+      if (d.modified) {
+        u[i] = pos_of(weight(i), s_ps);
+      } else {  // plain: wtab[|dK - k_ref|], k_ref the smallest or largest activity
+        const unsigned int k = (unsigned int)(d.s_neg ? kref - dkv[i] : dkv[i] - kref);
+        u[i] = 0ull;
+        if (j0 + i < d.nc) {
+          if (k < (unsigned int)kUStage) u[i] = s_u[k];
+          else if (k < (unsigned int)kKcap) u[i] = pos_of(__ldg(wt + k), s_ps);  // 0 beyond: k_weights reports it
+        }
+      }
+      sum += u[i];
+    }
+    unsigned long long q = scan_block(sum) + s_pos0;
+    J0 = pos_slot(s_pos0, d.F, near);
+    jl[0] = pos_slot(q, d.F, near);
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      q += u[i];
+      jl[i + 1] = pos_slot(q, d.F, near);
+    }
+    fill_map();
+    near = __syncthreads_or(near) != 0;
+  }
+  if (d.iid || near) {
+    // a position too close to a slot, or [iid]: the exact prefix sums
+    const unsigned long long T = s_T;
+    unsigned long long w[NI], sum = 0ull;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      w[i] = weight(i);
+      sum += w[i];
+    }
+    unsigned long long run = scan_block(sum);
+    if constexpr (SCAN) {
+      run += B.tile_excl[tile];
+    } else {
+      for (int i = 0; i < lt; ++i) run += B.tile_sum[d.first_tile + i];
+    }
+    if (d.iid) {
+      // publish this tile's prefix sums; k_select_iid draws the points
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        B.S[base + (int64_t)tid * NI + i] = run;
+        run += w[i];
+      }
+      if (lt == 0 && tid == 0) st->T = T;
+    } else {
+      const int sh = max(0, 64 - __clzll((long long)T) - 24);
+      const float ratio = __fdiv_rn((float)nc, __uint2float_rn((uint32_t)(T >> sh)));
+      j_lo_run<NI>(run, w, T, c, nc, sh, ratio, jl);
+      if (tid == 0) s_J0 = jl[0];
+      __syncthreads();
+      J0 = s_J0;
+      fill_map();
+      __syncthreads();
+    }
+  }
+  if (!d.iid) {
+  J1 = s_J1;
+  const bool mapped = (J1 - J0) <= (uint32_t)kMap;
+  if (!mapped) {
+    __syncthreads();
 #pragma unroll
     for (int i = 0; i < NI; ++i) s_jlo[tid * NI + i] = jl[i];
     if (tid == NT - 1) s_jlo[kTile] = jl[NI];
+    __syncthreads();
   }
-  __syncthreads();
   auto source = [&](uint32_t jj) -> int {
     if (mapped) return s_src[jj - J0];
     int lo = 0, hi = kTile - 1;  // one old clone with very many copies: search j_lo
@@ -1081,7 +1099,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
   // GUIDED: X_ref + log1p(...) with X_ref the largest log weight.
   if (d.modified && lt == 0 && tid == 0) {
     const double base_w = ldexp((double)d.nc, d.F);
-    const long long D = (long long)T - (long long)((unsigned long long)d.nc << d.F);
+    const long long D = (long long)s_T - (long long)((unsigned long long)d.nc << d.F);
     const double ref = d.guided ? (double)a_ref : -(double)d.c_f * (double)a_ref;
     st->psi_acc += ref + log1p((double)D / base_w);
     st->dk_min[par] = INT_MAX;
