@@ -188,21 +188,22 @@ __device__ __forceinline__ uint4 philox4x32_10_rk(uint4 c, const uint2* rk) {
 // (|r| <= 1/128) and ln(1+r) ~ r (1 - r/2 + r^2/3).  tab[i] = (float(1/c_i),
 // float(ln c_i)).  ln 2 is a 15-bit head (exact products with 33-p) plus a float
 // tail.  Every float step is an explicitly rounded intrinsic, so no contraction
-// can change the bits; the integer work stays in 32 bits (no 64-bit shifts or
-// conversions): the leading one of v = 2w+1 is one above that of w, and for p >= 24
-// the head of v is w >> (p - 24) (the trailing 1 of v is shifted out).
+// can change the bits.  The 24 leading bits of v come from the float unit: with f = w
+// rounded towards zero, 2f + 1 rounded towards zero is v truncated to 24 bits for every w
+// (exact below 2^23; above, the 1 falls to the rounding), so its exponent is p and its
+// fraction that of m.  Two instructions, where the leading one, two shifts and a choice
+// between them took eight.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float neg_ln_u(uint32_t w, const float2* tab) {
-  const int p = 32 - __clz((int)w);  // leading one of 2w+1: 0..32
-  const uint32_t t = (p >= 24) ? (w >> (p - 24)) : ((2u * w + 1u) << (23 - p));
-  const float m = __uint_as_float(0x3f800000u | (t & 0x007fffffu));
-  const float2 cl = tab[(t >> 17) & 63u];
+  const uint32_t b = __float_as_uint(__fmaf_rz(__uint2float_rz(w), 2.0f, 1.0f));
+  const float m = __uint_as_float(0x3f800000u | (b & 0x007fffffu));
+  const float2 cl = tab[(b >> 17) & 63u];
   const float r = __fmaf_rn(m, cl.x, -1.0f);
   float q = __fmaf_rn(r, 0x1.555556p-2f, -0.5f);
   q = __fmaf_rn(q, r, 1.0f);
   const float ln_m = __fadd_rn(cl.y, __fmul_rn(q, r));
   // float(33 - p) exactly: 1.5*2^23 + n has n in its low mantissa bits
-  const float n = __fsub_rn(__int_as_float(0x4B400000 + (33 - p)), 12582912.0f);
+  const float n = __fsub_rn(__uint_as_float(0x4B400000u + (33u + 127u) - (b >> 23)), 12582912.0f);
   const float E = __fmaf_rn(n, 0x1.7f7d1cp-20f, -ln_m);
   return __fmaf_rn(n, 0x1.62e4p-1f, E);
 }

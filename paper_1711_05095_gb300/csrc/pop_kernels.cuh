@@ -117,8 +117,8 @@ __device__ __forceinline__ bool bkl_step(uint32_t (&u)[2 * W], float& t, float& 
 // The same step without branches, for a clone that is `live` (else nothing changes):
 // the rate, waiting time and bond are computed in any case and applied under the
 // step's predicate, so the lanes of a warp stay together.  r = 0 or t_new >= dt ends
-// the interval as in bkl_step (MOD: the last segment r (dt - t) is added when r > 0;
-// for r = 0 it adds nothing).  A step that does not hop passes bond 1024, which
+// the interval as in bkl_step: inv[0] is NaN, so the comparison fails for r = 0 (MOD: the
+// last segment r (dt - t) is added; for r = 0 it adds nothing).  A step that does not hop passes bond 1024, which
 // hop32 turns into no change.  FULL: L = 64 W (see active_bonds32).
 template <int W, bool MOD, bool FULL = false>
 __device__ __forceinline__ bool bkl_step_pred(uint32_t (&u)[2 * W], float& t, float& acc, uint32_t lm1,
@@ -132,11 +132,10 @@ __device__ __forceinline__ bool bkl_step_pred(uint32_t (&u)[2 * W], float& t, fl
   for (int j = 0; j < NW; ++j) r += pc[j];
   const float tau = __fmul_rn(E, inv[r]);
   const float t_new = __fadd_rn(t, tau);
-  const bool moving = live && r != 0u;
-  const bool hopped = moving && t_new < dt_f;
+  const bool hopped = live && t_new < dt_f;
   if (MOD) {
     const float seg = hopped ? tau : __fsub_rn(dt_f, t);
-    acc = moving ? __fmaf_rn((float)r, seg, acc) : acc;
+    acc = live ? __fmaf_rn((float)r, seg, acc) : acc;
   }
   t = hopped ? t_new : t;
   const uint32_t b = kth_bond32<NW>(a, pc, __umulhi(wb, r), kth8);
@@ -638,7 +637,8 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
   const int32_t* const KXo = B.KXb[par];
   if constexpr (FUSE) {
     const float* src = B.inv_rate + (size_t)p * kInvStride;
-    for (int r = tid; r <= kMaxL; r += NT) s_inv[r] = (r <= d.L) ? src[r] : 0.0f;
+    for (int r = tid; r <= kMaxL; r += NT)  // inv[0] = NaN: see bkl_step_pred
+      s_inv[r] = r == 0 ? __int_as_float(0x7fffffff) : (r <= d.L) ? src[r] : 0.0f;
     if (tid < 64) s_logtab[tid] = B.logtab[tid];
     if (tid < 128) reinterpret_cast<uint4*>(s_kth8)[tid] = reinterpret_cast<const uint4*>(g_kth8.w)[tid];
     if constexpr (!MOD)
