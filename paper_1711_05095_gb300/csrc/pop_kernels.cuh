@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_scan(Batch B, int pop0) {
 // clone is taken straight from its staged ancestor and evolved (the same BKL steps,
 // draws and write-back as k_evolve, into the buffers of the other parity), so the
 // population between the two stages never goes through global memory.  Lanes take
-// new slots from a shared counter as their clones end, as in k_evolve.
+// their warp's next new slot as their clones end.
 // ---------------------------------------------------------------------------
 #ifndef POP_GATHER_THREADS
 #define POP_GATHER_THREADS 128
@@ -607,7 +607,6 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
   // schedule, the slot counter and the block's activity range of the next interval
   __shared__ float s_inv[FUSE ? kMaxL + 1 : 1];
   __shared__ float2 s_logtab[FUSE ? 64 : 1];
-  __shared__ uint2 s_keys[FUSE ? 10 : 1];
   // the lengths u of the first kUStage weights of the population's table (the activity
   // spreads of nearly every interval)
   constexpr int kUStage = 64;
@@ -616,7 +615,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
   // FUSE, plain weights: activity histograms of the first three tiles the new clones
   // fall in (the rest go straight to global memory)
   __shared__ unsigned int s_th[(FUSE && !MOD) ? 3 * kTH : 1];
-  __shared__ int s_take;
+  __shared__ uint2 s_keys[FUSE ? 10 : 1];
   __shared__ unsigned int s_pack[2];  // FUSE: clones packed in the current / next tail round
   __shared__ int s_nmin, s_nmax, s_namin, s_namax;
   __shared__ unsigned int s_nev;
@@ -647,7 +646,6 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
       s_keys[tid] = make_uint2((uint32_t)d.seed + (uint32_t)tid * 0x9E3779B9u,
                                (uint32_t)(d.seed >> 32) + (uint32_t)tid * 0xBB67AE85u);
     if (tid == 0) {
-      s_take = 0;
       s_pack[0] = 0u;
       s_pack[1] = 0u;
       s_nmin = INT_MAX;
@@ -843,9 +841,8 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
   };
   if constexpr (FUSE) {
     // dynamical stage of interval beta + 1 for the new slots [J0, J1): each lane holds
-    // NCL clones; an empty clone slot takes the next new slot of the tile from the
-    // shared counter (all of a warp's empty slots in one atomic), so lanes stay busy
-    // until the tile's slots run out.  Every live clone takes one Philox draw (its next
+    // NCL clones; an empty clone slot takes the warp's next new slot, so lanes stay busy
+    // until the warp's share of the tile's slots runs out.  Every live clone takes one Philox draw (its next
     // two BKL steps) per iteration; the steps are predicated, without branches.
     const uint32_t beta1 = beta + 1u;
     const int pn = par ^ 1;
@@ -927,7 +924,13 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
         }
       }
     };
-    // lanes take new slots from the shared counter until it runs out
+    // each warp takes new slots from its own even share of the tile's, in order, until
+    // the share runs out (the sum over a share's clones hardly varies between warps; a
+    // counter shared by the block cost a shared-memory read and an atomic in the chain of
+    // every iteration: L = 128 batch 325 us per interval, 304 us with shares)
+    const int share = n / NWARP, extra = n - share * NWARP;
+    int next = wid * share + min(wid, extra);
+    const int last = next + share + (wid < extra ? 1 : 0);
     for (;;) {
       unsigned int m[NCL];
       int tot = 0;
@@ -937,18 +940,11 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
         tot += __popc(m[k]);
       }
       if (tot != 0) {
-        // one read of the counter per warp keeps every branch below warp-uniform
-        int taken = 0;
-        if (lane == 0) taken = *(volatile int*)&s_take;
-        taken = __shfl_sync(0xffffffffu, taken, 0);
-        if (taken >= n) break;  // the counter ran out: on to the packed rounds below
-        int base_i = 0;
-        if (lane == 0) base_i = atomicAdd(&s_take, tot);
-        base_i = __shfl_sync(0xffffffffu, base_i, 0);
+        if (next >= last) break;  // on to the packed rounds below
 #pragma unroll
         for (int k = 0; k < NCL; ++k) {
-          const int idx = base_i + __popc(m[k] & lt_mask);
-          if (cl[k] < 0 && idx < n) {
+          const int idx = next + __popc(m[k] & lt_mask);
+          if (cl[k] < 0 && idx < last) {
             cl[k] = idx;
             const int sk = source(J0 + (uint32_t)idx);
             kold[k] = KXo[base + sk];
@@ -959,19 +955,12 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
             h[k] = 0;
             q[k] = 0u;
           }
-          base_i += __popc(m[k]);
-        }
-        if (tot == 32 * NCL) {
-          // every slot was empty and the claim may have come after the last clone
-          bool any = false;
-#pragma unroll
-          for (int k = 0; k < NCL; ++k) any = any || cl[k] >= 0;
-          if (__ballot_sync(0xffffffffu, any) == 0u) continue;
+          next += __popc(m[k]);
         }
       }
       iterate();
     }
-    // The counter has run out.  Each round packs the block's remaining clones into the
+    // The shares have run out.  Each round packs the block's remaining clones into the
     // lowest threads (through the staging buffer of the old clones, no longer read),
     // so that warps left without clones stop issuing, and runs one iteration.
     struct Packed {
