@@ -60,7 +60,7 @@ constexpr int kGatherWideTiles = 4096;
 #endif
 
 struct Layout {
-  int32_t P = 0, W = 0, ntiles = 0, nunits = 0;
+  int32_t P = 0, W = 0, ntiles = 0;
   int64_t nslots = 0;
   size_t o_pops, o_st, o_tile_pop, o_wtab, o_qtab, o_qm1tab, o_inv, o_logtab, o_exp2, o_A, o_S, o_cs, o_tacc, o_hist, o_thist, o_tile_sum, o_tile_excl, o_beta, o_phi, o_gtab, o_gdu, o_gq, o_gcar,
       o_ksum, o_X, o_Y, o_KX, o_KY, o_dK, o_anc, total;
@@ -100,7 +100,6 @@ bool make_layout(const pop_params* params, int32_t n_pops, Layout* lay) {
   l.W = (maxL + 63) / 64;
   l.ntiles = (int32_t)ntiles;
   l.nslots = ntiles * kTile;
-  l.nunits = (int32_t)(l.nslots / kUnit);
   const size_t P = (size_t)n_pops, ns = (size_t)l.nslots, nt = (size_t)l.ntiles;
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = align256(o + bytes); return r; };
@@ -217,8 +216,6 @@ struct pop_batch {
   int guided_split = 1;       // GUIDED: blocks per tile of the dynamical stage (1, 2, 4, 8)
   int evolve_grid = 0;
   int evolve_grid_cap = 0;  // persistent grid at full occupancy
-  size_t evolve_smem = 0;
-  int wide_unit = 0;         // wide rings: slots per warp and pass of the dynamical stage
   bool s_fixed = false;
   std::vector<double> s;
   Phase phase = kReady;
@@ -345,28 +342,37 @@ void kernel_end(pop_t* h, cudaStream_t st) {
   if (h->timer_events != nullptr) timer_record(h, st);
 }
 
-// Lanes per clone of the wide dynamical stage: 256 sites each.
-int wide_lanes(const pop_t* h) {
+// The dynamical stage's kernel for a batch: words per lane and lanes per clone by the
+// largest ring, the form for rings that fill one or two 64-bit words where every one does.
+// FULL and MODIFIED are combined only where they occur together in use.
+typedef void (*EvolveKernel)(Batch, float);
+
+int evolve_lanes(const pop_t* h) {
   int g = 1;
   while (256 * g < h->max_L) g *= 2;
   return g;
 }
 
 template <bool MOD>
-void launch_wide(pop_t* h, cudaStream_t st, float dt_f) {
-  const unsigned grid = (unsigned)h->evolve_grid;
-  switch (wide_lanes(h)) {
-    case 1: k_evolve_wide<1, MOD><<<grid, kWideThreads, 0, st>>>(h->B, dt_f, h->wide_unit); break;
-    case 2: k_evolve_wide<2, MOD><<<grid, kWideThreads, 0, st>>>(h->B, dt_f, h->wide_unit); break;
-    case 4: k_evolve_wide<4, MOD><<<grid, kWideThreads, 0, st>>>(h->B, dt_f, h->wide_unit); break;
-    case 8: k_evolve_wide<8, MOD><<<grid, kWideThreads, 0, st>>>(h->B, dt_f, h->wide_unit); break;
-    default: k_evolve_wide<16, MOD><<<grid, kWideThreads, 0, st>>>(h->B, dt_f, h->wide_unit); break;
+EvolveKernel evolve_kernel_of(const pop_t* h) {
+  bool full = true;
+  for (const PopDesc& d : h->desc) full = full && d.L == 64 * h->lay.W;
+  if (h->lay.W == 1) return full ? k_evolve<2, 1, MOD, true> : k_evolve<2, 1, MOD, false>;
+  if (h->lay.W == 2) return full ? k_evolve<4, 1, MOD, true> : k_evolve<4, 1, MOD, false>;
+  switch (evolve_lanes(h)) {
+    case 1: return k_evolve<8, 1, MOD, false>;
+    case 2: return k_evolve<8, 2, MOD, false>;
+    case 4: return k_evolve<8, 4, MOD, false>;
+    case 8: return k_evolve<8, 8, MOD, false>;
+    default: return k_evolve<8, 16, MOD, false>;
   }
 }
 
+EvolveKernel evolve_kernel(const pop_t* h) {
+  return h->any_mod ? evolve_kernel_of<true>(h) : evolve_kernel_of<false>(h);
+}
+
 int launch_evolve(pop_t* h, cudaStream_t st, float dt_f) {
-  const unsigned grid = (unsigned)h->evolve_grid;
-  const size_t sm = h->evolve_smem;
   kernel_begin(h, st, POP_K_EVOLVE);
   if (h->guided) {
     // a tile per block, or a half, quarter or eighth of one for a batch of fewer tiles
@@ -375,14 +381,8 @@ int launch_evolve(pop_t* h, cudaStream_t st, float dt_f) {
     const unsigned gg = (unsigned)((int64_t)h->lay.ntiles * h->guided_split);
     if (h->lay.W == 1) k_evolve_guided<1><<<gg, kGuideThreads, 0, st>>>(h->B, dt_f, spb);
     else k_evolve_guided<2><<<gg, kGuideThreads, 0, st>>>(h->B, dt_f, spb);
-  } else if (h->any_mod) {
-    if (h->lay.W == 1) k_evolve<1, true><<<grid, kThreads, sm, st>>>(h->B, dt_f);
-    else if (h->lay.W == 2) k_evolve<2, true><<<grid, kThreads, sm, st>>>(h->B, dt_f);
-    else launch_wide<true>(h, st, dt_f);
   } else {
-    if (h->lay.W == 1) k_evolve<1, false><<<grid, kThreads, sm, st>>>(h->B, dt_f);
-    else if (h->lay.W == 2) k_evolve<2, false><<<grid, kThreads, sm, st>>>(h->B, dt_f);
-    else launch_wide<false>(h, st, dt_f);
+    evolve_kernel(h)<<<(unsigned)h->evolve_grid, kEvolveThreads, 0, st>>>(h->B, dt_f);
   }
   kernel_end(h, st);
   return cuda_status(cudaGetLastError());
@@ -570,58 +570,25 @@ int size_chains(pop_t* h) {
   return POP_OK;
 }
 
-// Persistent evolve grid: as many blocks as fit on the device at once, each
-// owning an equal share of the 256-slot units.
-template <int W, bool MOD>
-int size_evolve_grid(pop_t* h) {
-  const size_t smem = sizeof(EvolveSmem<W>);
-  POP_CUDA(cudaFuncSetAttribute(k_evolve<W, MOD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem));
-  int per_sm = 0, sms = 0;
-  POP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_evolve<W, MOD>, kThreads, smem));
-  POP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-  if (per_sm < 1) per_sm = 1;
-  const long long want = (long long)per_sm * sms;
-  h->evolve_grid = (int)(want < h->lay.nunits ? want : h->lay.nunits);
-  h->evolve_grid_cap = h->evolve_grid;
-  h->evolve_smem = smem;
-  h->B.unit_q = h->lay.nunits / h->evolve_grid;
-  h->B.unit_r = h->lay.nunits % h->evolve_grid;
-  return POP_OK;
-}
-
-// Re-split the units over a different persistent grid (k_evolve only).
+// Split the slots over a persistent grid of k_evolve: an even share of the chunks of
+// 32 / G slots (what a warp holds at a time) to each warp.
 void set_evolve_grid(pop_t* h, int grid) {
+  const int64_t chunks = h->lay.nslots / (32 / evolve_lanes(h));
+  const int64_t most = (chunks + kEvolveWarps - 1) / kEvolveWarps;
   if (grid < 1) grid = 1;
-  if (h->lay.W <= 2 && grid > h->lay.nunits) grid = h->lay.nunits;
+  if (grid > most) grid = (int)most;
   h->evolve_grid = grid;
-  h->B.unit_q = h->lay.nunits / grid;
-  h->B.unit_r = h->lay.nunits % grid;
+  h->B.unit_q = chunks / ((int64_t)grid * kEvolveWarps);
+  h->B.unit_r = chunks % ((int64_t)grid * kEvolveWarps);
 }
 
-// Rings longer than 128 sites: a grid-stride loop of warps over units of slots.  A unit
-// is as large as leaves a unit to every resident warp (a longer queue per warp keeps its
-// lanes busier towards the end), between the 32 / G clones a warp holds and 256.
-template <bool MOD>
-int size_evolve_grid_wide(pop_t* h) {
-  const int g = wide_lanes(h);
-  const void* f = g == 1   ? (const void*)k_evolve_wide<1, MOD>
-                  : g == 2 ? (const void*)k_evolve_wide<2, MOD>
-                  : g == 4 ? (const void*)k_evolve_wide<4, MOD>
-                  : g == 8 ? (const void*)k_evolve_wide<8, MOD>
-                           : (const void*)k_evolve_wide<16, MOD>;
+// As many blocks as fit on the device at once (or as there are chunks for).
+int size_evolve_grid(pop_t* h) {
   int per_sm = 0, sms = 0;
-  POP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kWideThreads, 0));
+  POP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evolve_kernel(h), kEvolveThreads, 0));
   POP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-  if (per_sm < 1) per_sm = 1;
-  const long long want = (long long)per_sm * sms;
-  const long long warps = kWideThreads / 32;
-  h->wide_unit = 256;
-  while (h->wide_unit > 32 / g && h->lay.nslots / h->wide_unit < want * warps) h->wide_unit /= 2;
-  const long long need = (h->lay.nslots / h->wide_unit + warps - 1) / warps;
-  h->evolve_grid = (int)(want < need ? want : need);
+  set_evolve_grid(h, (per_sm < 1 ? 1 : per_sm) * sms);
   h->evolve_grid_cap = h->evolve_grid;
-  h->evolve_smem = 0;
   return POP_OK;
 }
 
@@ -838,7 +805,6 @@ int pop_init(pop_t** out, const pop_params* params, int32_t n_pops, void* d_work
   B.dKb[1] = B.dKb[0] + lay.nslots;
   B.anc = (int32_t*)(ws + lay.o_anc);
   B.ntiles = lay.ntiles;
-  B.nunits = lay.nunits;
   B.nslots = lay.nslots;
   B.W = lay.W;
   if (size_chains(h) != POP_OK) return fail(POP_ERR_CUDA);
@@ -846,10 +812,7 @@ int pop_init(pop_t** out, const pop_params* params, int32_t n_pops, void* d_work
     if (cudaStreamCreateWithFlags(&h->aux_stream[c], cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_join[c], cudaEventDisableTiming) != cudaSuccess)
       return fail(POP_ERR_CUDA);
-  const bool mod = h->any_mod;
-  const int grc = lay.W == 1 ? (mod ? size_evolve_grid<1, true>(h) : size_evolve_grid<1, false>(h))
-                  : lay.W == 2 ? (mod ? size_evolve_grid<2, true>(h) : size_evolve_grid<2, false>(h))
-                               : (mod ? size_evolve_grid_wide<true>(h) : size_evolve_grid_wide<false>(h));
+  const int grc = size_evolve_grid(h);
   if (grc != POP_OK) return fail(POP_ERR_CUDA);
   if (h->guided) {
     int per_sm = 0, sms = 0;

@@ -35,9 +35,6 @@ constexpr int kThreads = 256;             // threads per block of every kernel
 constexpr int kWarps = kThreads / 32;
 constexpr int kTile = 1024;               // slots per tile; populations start on a tile
 constexpr int kItems = kTile / kThreads;  // slots per thread in the tile kernels
-constexpr int kUnit = 256;                // slots per evolve work unit (one population)
-constexpr int kChunkUnits = 7;            // at most this many units staged in shared memory
-constexpr int kChunk = kUnit * kChunkUnits;
 constexpr int kKcap = 4096;               // fixed-point weight table size
 constexpr int kHistSmem = 512;            // activity bins kept in shared memory
 constexpr int kTH = 64;                   // per-tile activity histogram bins (activities 0 .. 63)
@@ -136,10 +133,9 @@ struct Batch {
   int32_t* anc;                         // ancestors of the last cloning stage
   long long* ksum;                      // [P] sum of K (estimates)
   int32_t ntiles;
-  int32_t nunits;
   int64_t nslots;
   int32_t W;                            // lattice words per clone
-  int32_t unit_q, unit_r;               // k_evolve: nunits = unit_q * grid + unit_r
+  int64_t unit_q, unit_r;               // k_evolve: chunks of 32 / G slots = unit_q * warps + unit_r
   int32_t any_iid;                      // some population selects [iid]: k_select_iid runs last
 };
 

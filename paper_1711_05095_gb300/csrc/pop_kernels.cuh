@@ -63,24 +63,6 @@ __global__ void __launch_bounds__(kThreads) k_init(Batch B) {
   B.dKb[1][slot] = 0;
 }
 
-// Shared-memory state of k_evolve: one chunk of up to kChunk clones.
-template <int W>
-struct EvolveSmem {
-  unsigned long long x[kChunk][W];  // lattices (in, then out)
-  int32_t hops[kChunk];             // activity of the interval
-  float a[kChunk];                  // MODIFIED: integral of the escape rate over the interval
-  float inv[kChunkUnits][kMaxL + 1];
-  float2 logtab[64];
-  __align__(16) uint32_t kth8[512];  // the byte table of kth_bond32
-  uint2 u_key[kChunkUnits];         // Philox key of the unit's population
-  int32_t u_j0[kChunkUnits];        // population-local index of the unit's first slot
-  int32_t u_pop[kChunkUnits], u_L[kChunkUnits], u_valid[kChunkUnits];
-  int32_t u_min[kChunkUnits], u_max[kChunkUnits];
-  int32_t u_amin[kChunkUnits], u_amax[kChunkUnits];
-  unsigned int u_ev[kChunkUnits];
-  int take;                         // next unclaimed clone of the chunk
-};
-
 // One BKL step (Sec. 4 BKL; Sec. 3.1 rates 1 per possible hop) with the step's
 // exponential variate E = -ln u(wa) and bond word wb, on the lattice as 2W 32-bit
 // words u (lm1 = L - 1): r = active bonds (escape rate; r = 0 ends the interval);
@@ -91,35 +73,12 @@ struct EvolveSmem {
 // MODIFIED dynamics (Sec. 3.2): inv holds float(e^s / r) and the integral of the
 // unmodified escape rate is accumulated, A <- fma(r, tau, A) per hop and
 // A <- fma(r, dt - t, A) for the last segment.
-template <int W, bool MOD>
-__device__ __forceinline__ bool bkl_step(uint32_t (&u)[2 * W], float& t, float& acc, uint32_t lm1,
-                                         const float* inv, float E, uint32_t wb, float dt_f,
-                                         const uint8_t* kth8) {
-  constexpr int NW = 2 * W;
-  uint32_t a[NW], pc[NW];
-  active_bonds32<NW>(u, lm1, a, pc);
-  uint32_t r = 0u;
-#pragma unroll
-  for (int j = 0; j < NW; ++j) r += pc[j];
-  if (r == 0u) return false;
-  const float tau = __fmul_rn(E, inv[r]);
-  const float t_new = __fadd_rn(t, tau);
-  if (t_new >= dt_f) {
-    if (MOD) acc = __fmaf_rn((float)r, __fsub_rn(dt_f, t), acc);
-    return false;
-  }
-  if (MOD) acc = __fmaf_rn((float)r, tau, acc);
-  t = t_new;
-  hop32<NW>(u, kth_bond32<NW>(a, pc, __umulhi(wb, r), kth8), lm1);
-  return true;
-}
-
-// The same step without branches, for a clone that is `live` (else nothing changes):
-// the rate, waiting time and bond are computed in any case and applied under the
-// step's predicate, so the lanes of a warp stay together.  r = 0 or t_new >= dt ends
-// the interval as in bkl_step: inv[0] is NaN, so the comparison fails for r = 0 (MOD: the
-// last segment r (dt - t) is added; for r = 0 it adds nothing).  A step that does not hop passes bond 1024, which
-// hop32 turns into no change.  FULL: L = 64 W (see active_bonds32).
+// Without branches, for a clone that is `live` (else nothing changes): the rate, waiting
+// time and bond are computed in any case and applied under the step's predicate, so the
+// lanes of a warp stay together.  inv[0] is NaN, so the comparison fails for r = 0 (MOD:
+// the last segment r (dt - t) is added; for r = 0 it adds nothing).  A step that does not
+// hop passes bond 1024, which hop32 turns into no change.  FULL: L = 64 W (see
+// active_bonds32).
 template <int W, bool MOD, bool FULL = false>
 __device__ __forceinline__ bool bkl_step_pred(uint32_t (&u)[2 * W], float& t, float& acc, uint32_t lm1,
                                               const float* inv, float E, uint32_t wb, float dt_f,
@@ -144,211 +103,258 @@ __device__ __forceinline__ bool bkl_step_pred(uint32_t (&u)[2 * W], float& t, fl
 }
 
 // ---------------------------------------------------------------------------
-// Dynamical stage.  A persistent grid; each block stages an equal share of the
-// clones in shared memory.  Every lane holds one clone in registers and advances
-// it two BKL steps per iteration from one Philox draw (draw q of the clone serves
-// its steps 2q and 2q+1); a lane whose clone has ended takes the next clone of
-// the block from a shared-memory counter, so lanes stay busy until the block's
-// clones run out and no block-wide barrier is needed during the interval.
+// Dynamical stage.  A clone is held by G lanes with NW 32-bit words each: one lane of two
+// or four words for L <= 64 or 128; eight words (256 sites) in 1, 2, 4, 8 or 16 lanes,
+// the smallest power of two that holds the batch's largest ring, beyond that.  32 / G
+// clones run side by side in a warp, two predicated BKL steps per iteration from one
+// Philox draw (draw q of the clone serves its steps 2q and 2q + 1).
+// In a group of lanes the site above a lane's top bit is bit 0 of the next lane and the
+// site above L - 1 is site 0; the escape rate is a sum over the group, the k-th active
+// bond lies in the lane whose range of an exclusive prefix of the lanes' counts holds k,
+// and the draw, the waiting time and the bond are the same on every lane of the group
+// (the same arithmetic as with one lane, so the same results).
+// A persistent grid: each warp has an even share of the slots and walks it tile by tile;
+// a group whose clone ended takes the share's next clone, so a warp needs no barrier and
+// no shared counter.  Clones go from global memory to registers and back.
+// Bound by ALU issue.  An interval of 2^22 clones of L = 128, dt = 0.05 by the per-step
+// calls took 288 us with clones staged in shared memory, diverging steps and a counter per
+// block, and 240 us with this form (the cloning stage unchanged); 2^21 clones of L = 50,
+// dt = 1, [iid]: 520 and 462 us.
+// Wide rings: about 250 instructions per step and warp for 32 / G clones, where a whole
+// warp per clone took 225 for one (2^16 clones of L = 256, dt = 0.05, with the cloning
+// stage: 301 us per interval with a warp per clone and a block's own copy of its tile,
+// 51 us now).
 // ---------------------------------------------------------------------------
+constexpr int kEvolveThreads = 128;
+constexpr int kEvolveWarps = kEvolveThreads / 32;
 #ifndef POP_EVOLVE_MIN_BLOCKS
-#define POP_EVOLVE_MIN_BLOCKS 4  // two-word staging (~48 KB) allows 4 blocks per SM anyway:
-                                 // 64 registers and no spills (5: 48 registers, 2.5 % slower)
+#define POP_EVOLVE_MIN_BLOCKS 8  // 64 registers
 #endif
-template <int W, bool MOD>
-__global__ void __launch_bounds__(kThreads, POP_EVOLVE_MIN_BLOCKS) k_evolve(Batch B, float dt_f) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  EvolveSmem<W>& S = *reinterpret_cast<EvolveSmem<W>*>(smem_raw);
-  const int tid = threadIdx.x, lane = tid & 31;
+
+// Position of the k-th set bit of the eight-word mask a (p[j] = popc(a[j])).
+__device__ __forceinline__ uint32_t kth_bond256(const uint32_t (&a)[8], const uint32_t (&p)[8], uint32_t k,
+                                                const uint8_t* kth8) {
+  const uint32_t lo = (p[0] + p[1]) + (p[2] + p[3]);
+  const bool h = k >= lo;
+  k = h ? k - lo : k;
+  uint32_t b[4], q[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    b[j] = h ? a[4 + j] : a[j];
+    q[j] = h ? p[4 + j] : p[j];
+  }
+  return kth_bond32<4>(b, q, k, kth8) + (h ? 128u : 0u);
+}
+
+// One step of a clone on G lanes of eight words, as bkl_step_pred; sub: the lane's place
+// in its group, lead: the group's first lane.  All 32 lanes take part.
+template <int G, bool MOD>
+__device__ __forceinline__ bool wide_step_pred(uint32_t (&u)[8], float& t, float& acc, uint32_t lm1, const float* inv,
+                                               float E, uint32_t wb, float dt_f, bool live, const uint8_t* kth8,
+                                               int sub, int lead) {
+  const uint32_t site0 = 256u * (uint32_t)sub;       // the lane's first site
+  uint32_t nb = 0u, c0 = u[0] & 1u;                  // bit 0 of the next lane, and site 0
+  if constexpr (G > 1) {
+    nb = __shfl_sync(0xffffffffu, c0, lead | ((sub + 1) & (G - 1)));
+    c0 = __shfl_sync(0xffffffffu, c0, lead);
+    if (sub == G - 1) nb = 0u;
+  }
+  uint32_t a[8], pc[8], cnt = 0u;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint32_t up = j < 7 ? u[(j + 1) & 7] : nb;
+    // the closing bond: site L - 1's right neighbour is site 0 (the sites above L - 1 are 0)
+    a[j] = u[j] ^ __funnelshift_r(u[j], up, 1) ^ __funnelshift_lc(0u, c0, lm1 - site0 - 32u * (uint32_t)j);
+    pc[j] = (uint32_t)__popc(a[j]);
+    cnt += pc[j];
+  }
+  uint32_t r = cnt;
+  if constexpr (G > 1) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  }
+  const float tau = __fmul_rn(E, __ldg(inv + r));
+  const float t_new = __fadd_rn(t, tau);
+  const bool moving = live && r != 0u;
+  const bool hopped = moving && t_new < dt_f;
+  if (MOD) {
+    const float seg = hopped ? tau : __fsub_rn(dt_f, t);
+    acc = moving ? __fmaf_rn((float)r, seg, acc) : acc;
+  }
+  t = hopped ? t_new : t;
+  const uint32_t k = __umulhi(wb, r);
+  uint32_t b;
+  if constexpr (G > 1) {
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o, G);
+      if (sub >= o) incl += y;
+    }
+    const uint32_t excl = incl - cnt;
+    const bool owner = excl <= k && k < incl;
+    const unsigned int om = (__ballot_sync(0xffffffffu, owner) >> lead) & ((1u << G) - 1u);
+    // k = 0 where the bond is not the lane's: the table is read at a place inside it
+    const uint32_t mine = site0 + kth_bond256(a, pc, owner ? k - excl : 0u, kth8);
+    b = __shfl_sync(0xffffffffu, mine, lead + (om ? __ffs(om) - 1 : 0));
+  } else {
+    b = kth_bond256(a, pc, k, kth8);
+  }
+  // flip sites b and (b + 1) mod L; no hop: bond 2^30, beyond every word
+  b = hopped ? b : 1u << 30;
+  const uint32_t c = b == lm1 ? 0u : b + 1u;
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    u[j] ^= __funnelshift_lc(0u, 1u, b - site0 - 32u * (uint32_t)j) ^
+            __funnelshift_lc(0u, 1u, c - site0 - 32u * (uint32_t)j);
+  return hopped;
+}
+
+template <int NW, int G, bool MOD, bool FULL>
+__global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_BLOCKS) k_evolve(Batch B, float dt_f) {
+  static_assert(NW == 8 || G == 1, "one lane for up to four words");
+  constexpr int W64 = NW / 2;                        // 64-bit words per lane
+  __shared__ float2 s_tab[64];
+  __shared__ __align__(16) uint32_t s_kth8[512];
+  __shared__ uint2 s_key[kEvolveWarps][10];          // the Philox key schedule of the warp's population
+  __shared__ float s_inv[kEvolveWarps][NW == 8 ? 1 : kMaxL + 1];  // and its waiting-time factors
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (tid < 64) s_tab[tid] = B.logtab[tid];
+  reinterpret_cast<uint4*>(s_kth8)[tid] = reinterpret_cast<const uint4*>(g_kth8.w)[tid];
+  __syncthreads();
+  const uint8_t* const kth8 = reinterpret_cast<const uint8_t*>(s_kth8);
   const uint32_t beta = *B.beta;
   const int par = (int)(beta & 1u);
-  unsigned long long* const Xo = B.Xb[par];
-  int32_t* const KXo = B.KXb[par];
-  int32_t* const dKo = B.dKb[par];
-  float* const Ao = B.Ab[par];
-  if (tid < 64) S.logtab[tid] = B.logtab[tid];
-  if (tid < 128) reinterpret_cast<uint4*>(S.kth8)[tid] = reinterpret_cast<const uint4*>(g_kth8.w)[tid];
-  const uint8_t* const kth8 = reinterpret_cast<const uint8_t*>(S.kth8);
-  // this block's units: an even split of B.nunits over the grid, B.unit_q units each
-  // and one more for the first B.unit_r blocks (no divisions on the device)
-  const int bx = (int)blockIdx.x;
-  const int u_begin = bx * B.unit_q + min(bx, B.unit_r);
-  const int len = B.unit_q + (bx < B.unit_r ? 1 : 0);
-  const int nchunks = (len + kChunkUnits - 1) / kChunkUnits;
-  const int cq = len / nchunks, cr = len - cq * nchunks;
-  for (int ch = 0; ch < nchunks; ++ch) {
-    const int uc = u_begin + ch * cq + min(ch, cr);
-    const int nu = cq + (ch < cr ? 1 : 0);
-    const int64_t chunk_slot0 = (int64_t)uc * kUnit;
-    if (tid < nu) {
-      const int64_t slot0 = chunk_slot0 + (int64_t)tid * kUnit;
-      const int p = B.tile_pop[slot0 / kTile];
-      const PopDesc d = B.pops[p];
-      const int64_t j0 = slot0 - d.off;
-      S.u_pop[tid] = p;
-      S.u_L[tid] = d.L;
-      S.u_j0[tid] = (int32_t)j0;
-      S.u_key[tid] = make_uint2((uint32_t)d.seed, (uint32_t)(d.seed >> 32));
-      S.u_valid[tid] = (int)max((int64_t)0, min((int64_t)kUnit, d.nc - j0));
-      S.u_min[tid] = INT_MAX;
-      S.u_max[tid] = INT_MIN;
-      S.u_amin[tid] = INT_MAX;
-      S.u_amax[tid] = INT_MIN;
-      S.u_ev[tid] = 0u;
-    }
-    if (tid == 0) S.take = 0;
-    // this thread's cumulative activities, needed at write-back
-    int32_t ky[kChunkUnits];
+  const int sub = lane & (G - 1), lead = lane & ~(G - 1);
+  unsigned int leaders = 0u;                         // first lanes of all groups
 #pragma unroll
-    for (int m = 0; m < kChunkUnits; ++m)
-      if (m < nu) ky[m] = B.KY[chunk_slot0 + m * kUnit + tid];
-    __syncthreads();
-    for (int uu = 0; uu < nu; ++uu) {
-      const float* src = B.inv_rate + (size_t)S.u_pop[uu] * kInvStride;
-      for (int r = tid; r <= kMaxL; r += kThreads) S.inv[uu][r] = (r <= S.u_L[uu]) ? src[r] : 0.0f;
+  for (int i = 0; i < 32; i += G) leaders |= 1u << i;
+  const unsigned int before = leaders & ((1u << lead) - 1u);
+  const int W = NW == 8 ? B.W : W64;
+  // the warp's share of the slots: B.unit_q chunks of 32 / G slots each and one more for
+  // the first B.unit_r warps
+  const int64_t wi = (int64_t)blockIdx.x * kEvolveWarps + wid;
+  int64_t slot0 = (wi * B.unit_q + min(wi, B.unit_r)) * (32 / G);
+  const int64_t slot_end = slot0 + (B.unit_q + (wi < B.unit_r ? 1 : 0)) * (32 / G);
+  while (slot0 < slot_end) {
+    const int64_t seg_end = min(slot_end, (slot0 / kTile + 1) * kTile);  // one tile, one population
+    const int p = B.tile_pop[slot0 / kTile];
+    const PopDesc d = B.pops[p];
+    const int64_t j0 = slot0 - d.off;
+    const int n = (int)max((int64_t)0, min(seg_end - slot0, d.nc - j0));  // warp-uniform
+    const float* inv = B.inv_rate + (size_t)p * kInvStride;
+    if (lane < 10)
+      s_key[wid][lane] = make_uint2((uint32_t)d.seed + (uint32_t)lane * 0x9E3779B9u,
+                                    (uint32_t)(d.seed >> 32) + (uint32_t)lane * 0xBB67AE85u);
+    if constexpr (NW < 8) {
+      for (int r = lane; r <= kMaxL; r += 32)  // inv[0] = NaN: see bkl_step_pred
+        s_inv[wid][r] = r == 0 ? __int_as_float(0x7fffffff) : (r <= d.L) ? inv[r] : 0.0f;
+      inv = s_inv[wid];
     }
-#pragma unroll
-    for (int m = 0; m < kChunkUnits; ++m) {
-      if (m < nu) {
-        const int i = m * kUnit + tid;
-        if (tid < S.u_valid[m]) {
-          unsigned long long x[W];
-          load_lat<W>(B.Y, chunk_slot0 + i, x);
-#pragma unroll
-          for (int q = 0; q < W; ++q) S.x[i][q] = x[q];
-        }
-        S.hops[i] = 0;
-      }
-    }
-    __syncthreads();
-
-    const int n = nu * kUnit;
-    int c = -1;  // the lane's clone (chunk index), -1 when it has none
-    unsigned long long x[W];
+    __syncwarp();
+    const uint32_t lm1 = (uint32_t)d.L - 1u;
+    int next = 0;                                    // the segment's next clone (warp-uniform)
+    int cl = -1, h = 0, kold = 0;
+    uint32_t q = 0u, u[NW];
     float t = 0.0f, acc = 0.0f;
-    int h = 0, L = 3;
-    uint32_t q = 0u, j = 0u;
-    uint2 key = make_uint2(0u, 0u);
-    const float* inv = S.inv[0];
+    int hmin = INT_MAX, hmax = INT_MIN, amin = INT_MAX, amax = INT_MIN;
+    unsigned int ev = 0u;
 #pragma unroll
-    for (int w = 0; w < W; ++w) x[w] = 0ull;
+    for (int j = 0; j < NW; ++j) u[j] = 0u;
     for (;;) {
-      // one read of the counter per warp keeps every branch below warp-uniform
-      int taken = 0;
-      if (lane == 0) taken = *(volatile int*)&S.take;
-      taken = __shfl_sync(0xffffffffu, taken, 0);
-      const bool need = c < 0;
-      const unsigned int m = __ballot_sync(0xffffffffu, need);
-      if (m != 0u && taken < n) {
-        const int leader = __ffs(m) - 1;
-        int base = 0;
-        if (lane == leader) base = atomicAdd(&S.take, __popc(m));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (need) {
-          const int idx = base + __popc(m & ((1u << lane) - 1u));
-          if (idx < n) {
-            const int uu = idx / kUnit;
-            if ((idx % kUnit) < S.u_valid[uu]) {
-              c = idx;
+      const unsigned int m = __ballot_sync(0xffffffffu, cl < 0) & leaders;
+      if (m != 0u && next < n) {
+        const int idx = next + __popc(m & before);
+        next += __popc(m);
+        if (cl < 0 && idx < n) {
+          cl = idx;
+          if constexpr (NW < 8) {
+            unsigned long long x[W64];
+            load_lat<W64>(B.Y, slot0 + idx, x);
+            split32<W64>(x, u);
+          } else {
+            const unsigned long long* src = B.Y + (slot0 + idx) * W + W64 * sub;
 #pragma unroll
-              for (int w = 0; w < W; ++w) x[w] = S.x[c][w];
-              t = 0.0f;
-              acc = 0.0f;
-              h = 0;
-              q = 0u;
-              L = S.u_L[uu];
-              key = S.u_key[uu];
-              j = (uint32_t)(S.u_j0[uu] + (idx % kUnit));
-              inv = S.inv[uu];
+            for (int j = 0; j < W64; ++j) {
+              const unsigned long long v = W64 * sub + j < W ? src[j] : 0ull;
+              u[2 * j] = (uint32_t)v;
+              u[2 * j + 1] = (uint32_t)(v >> 32);
             }
           }
+          kold = B.KY[slot0 + idx];
+          t = acc = 0.0f;
+          h = 0;
+          q = 0u;
         }
+      } else if (m == leaders) {
+        break;  // every group is empty and the segment has run out
       }
-      if (__ballot_sync(0xffffffffu, c >= 0) == 0u) {
-        if (lane == 0) taken = *(volatile int*)&S.take;
-        if (__shfl_sync(0xffffffffu, taken, 0) >= n) break;
+      const bool live = cl >= 0;
+      const uint4 d4 = philox4x32_10_rk(make_uint4(q, beta, (uint32_t)(j0 + cl), kTagEvolve), s_key[wid]);
+      // both waiting-time variates up front: independent of the lattice, so the two
+      // logarithms overlap
+      const float E1 = neg_ln_u(d4.x, s_tab), E2 = neg_ln_u(d4.z, s_tab);
+      bool h1, h2;
+      if constexpr (NW < 8) {
+        h1 = bkl_step_pred<W64, MOD, FULL>(u, t, acc, lm1, inv, E1, d4.y, dt_f, live, kth8);
+        h2 = bkl_step_pred<W64, MOD, FULL>(u, t, acc, lm1, inv, E2, d4.w, dt_f, h1, kth8);
+      } else {
+        h1 = wide_step_pred<G, MOD>(u, t, acc, lm1, inv, E1, d4.y, dt_f, live, kth8, sub, lead);
+        h2 = wide_step_pred<G, MOD>(u, t, acc, lm1, inv, E2, d4.w, dt_f, h1, kth8, sub, lead);
       }
-      if (c >= 0) {
-        const uint4 d4 = philox4x32_10(make_uint4(q, beta, j, kTagEvolve), key.x, key.y);
-        // both waiting-time variates up front: independent of the lattice, so the two
-        // logarithms overlap
-        const float E1 = neg_ln_u(d4.x, S.logtab), E2 = neg_ln_u(d4.z, S.logtab);
-        bool run = false;
-        uint32_t u[2 * W];
-        split32<W>(x, u);
-        if (bkl_step<W, MOD>(u, t, acc, (uint32_t)L - 1u, inv, E1, d4.y, dt_f, kth8)) {
-          ++h;
-          if (bkl_step<W, MOD>(u, t, acc, (uint32_t)L - 1u, inv, E2, d4.w, dt_f, kth8)) {
-            ++h;
-            run = true;
-          }
-        }
-        join32<W>(u, x);
-        ++q;
-        if (run && q >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
-          B.st[S.u_pop[c / kUnit]].err = kErrRange;
-          run = false;
-        }
-        if (!run) {
+      h += (int)h1 + (int)h2;
+      ++q;
+      bool run = h2;
+      if (run && q >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
+        B.st[p].err = kErrRange;
+        run = false;
+      }
+      if (live && !run) {
+        const int64_t slot = slot0 + cl;
+        if constexpr (NW < 8) {
+          unsigned long long x[W64];
+          join32<W64>(u, x);
+          store_lat<W64>(B.Xb[par], slot, x);
+        } else {
+          unsigned long long* dst = B.Xb[par] + slot * W + W64 * sub;
 #pragma unroll
-          for (int w = 0; w < W; ++w) S.x[c][w] = x[w];
-          S.hops[c] = h;
-          if (MOD) S.a[c] = acc;
-          c = -1;
+          for (int j = 0; j < W64; ++j)
+            if (W64 * sub + j < W) dst[j] = ((unsigned long long)u[2 * j + 1] << 32) | u[2 * j];
         }
+        if (G == 1 || sub == 0) {
+          B.KXb[par][slot] = kold + h;
+          B.dKb[par][slot] = h;
+          if (MOD) {
+            B.Ab[par][slot] = acc;
+            amin = min(amin, __float_as_int(acc));  // A >= 0: float bits order like values
+            amax = max(amax, __float_as_int(acc));
+          }
+          hmin = min(hmin, h);
+          hmax = max(hmax, h);
+          ev += (unsigned int)h;
+        }
+        cl = -1;
       }
     }
-    __syncthreads();
-
-    // write back (coalesced) and reduce the activity per unit
-#pragma unroll
-    for (int m = 0; m < kChunkUnits; ++m) {
-      if (m < nu) {
-        const int i = m * kUnit + tid;
-        const bool valid = tid < S.u_valid[m];
-        const int64_t slot = chunk_slot0 + i;
-        const int hh = S.hops[i];
-        if (valid) {
-          unsigned long long xo[W];
-#pragma unroll
-          for (int w = 0; w < W; ++w) xo[w] = S.x[i][w];
-          store_lat<W>(Xo, slot, xo);
-          KXo[slot] = ky[m] + hh;
-          dKo[slot] = hh;
-          if (MOD) Ao[slot] = S.a[i];
-        }
-        if (MOD) {
-          // A >= 0, so its float bits order like the values
-          const int ab = valid ? __float_as_int(S.a[i]) : 0;
-          const int amn = __reduce_min_sync(0xffffffffu, valid ? ab : INT_MAX);
-          const int amx = __reduce_max_sync(0xffffffffu, valid ? ab : INT_MIN);
-          if (lane == 0) {
-            atomicMin(&S.u_amin[m], amn);
-            atomicMax(&S.u_amax[m], amx);
-          }
-        }
-        const int mn = __reduce_min_sync(0xffffffffu, valid ? hh : INT_MAX);
-        const int mx = __reduce_max_sync(0xffffffffu, valid ? hh : INT_MIN);
-        const unsigned int ev = __reduce_add_sync(0xffffffffu, valid ? (unsigned int)hh : 0u);
-        if (lane == 0) {
-          atomicMin(&S.u_min[m], mn);
-          atomicMax(&S.u_max[m], mx);
-          atomicAdd(&S.u_ev[m], ev);
-        }
-      }
+    hmin = __reduce_min_sync(0xffffffffu, hmin);
+    hmax = __reduce_max_sync(0xffffffffu, hmax);
+    ev = __reduce_add_sync(0xffffffffu, ev);
+    if (MOD) {
+      amin = __reduce_min_sync(0xffffffffu, amin);
+      amax = __reduce_max_sync(0xffffffffu, amax);
     }
-    __syncthreads();
-    if (tid < nu && S.u_min[tid] != INT_MAX) {
-      PopState* st = B.st + S.u_pop[tid];
-      atomicMin(&st->dk_min[par], S.u_min[tid]);
-      atomicMax(&st->dk_max[par], S.u_max[tid]);
-      atomicAdd(&st->events, (unsigned long long)S.u_ev[tid]);
+    if (lane == 0 && n > 0) {
+      PopState* st = B.st + p;
+      atomicMin(&st->dk_min[par], hmin);
+      atomicMax(&st->dk_max[par], hmax);
+      atomicAdd(&st->events, (unsigned long long)ev);
       if (MOD) {
-        atomicMin(&st->a_min[par], S.u_amin[tid]);
-        atomicMax(&st->a_max[par], S.u_amax[tid]);
+        atomicMin(&st->a_min[par], amin);
+        atomicMax(&st->a_max[par], amax);
       }
     }
-    __syncthreads();
+    __syncwarp();  // the segment's key and factors have been read
+    slot0 = seg_end;
   }
 }
 
@@ -1564,208 +1570,6 @@ __global__ void __launch_bounds__(kGuideThreads, W == 1 ? POP_GUIDE1_MIN_BLOCKS 
     atomicAdd(&st->events, (unsigned long long)s_ev);
     atomicMin(&st->a_min[par], s_amin);
     atomicMax(&st->a_max[par], s_amax);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Dynamical stage for rings longer than 128 sites: G lanes per clone (1, 2, 4, 8 or 16:
-// the smallest power of two that holds the batch's largest ring), each with 256 sites in
-// eight 32-bit words, 32 / G clones side by side in a warp.  The site above a lane's top
-// bit is bit 0 of the group's next lane and the site above L - 1 is site 0; the escape
-// rate is a sum over the group, the k-th active bond lies in the lane whose range of an
-// exclusive prefix of the lanes' counts holds k, and the draw, the waiting time and the
-// bond are the same on every lane of the group (the same arithmetic as the one-lane
-// kernels).  Steps are predicated; a group whose clone ended takes the next clone of the
-// warp's unit of `unit` slots, so a warp needs no barrier and no shared counter.
-// Bound by ALU issue: about 250 instructions per step and warp for 32 / G clones; a
-// whole warp per clone, 128 sites to a lane, took 225 for one.  2^16 clones of L = 256,
-// dt = 0.05, with the cloning stage: 301 us per interval with a warp per clone and a
-// block's own copy of its tile, 51 us now.
-// ---------------------------------------------------------------------------
-constexpr int kWideWords = 8;                        // 32-bit words per lane
-constexpr int kWideThreads = 128;
-
-// Position of the k-th set bit of the eight-word mask a (p[j] = popc(a[j])).
-__device__ __forceinline__ uint32_t kth_bond256(const uint32_t (&a)[8], const uint32_t (&p)[8], uint32_t k,
-                                                const uint8_t* kth8) {
-  const uint32_t lo = (p[0] + p[1]) + (p[2] + p[3]);
-  const bool h = k >= lo;
-  k = h ? k - lo : k;
-  uint32_t b[4], q[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    b[j] = h ? a[4 + j] : a[j];
-    q[j] = h ? p[4 + j] : p[j];
-  }
-  return kth_bond32<4>(b, q, k, kth8) + (h ? 128u : 0u);
-}
-
-template <int G, bool MOD>
-__global__ void __launch_bounds__(kWideThreads) k_evolve_wide(Batch B, float dt_f, int unit) {
-  __shared__ float2 s_tab[64];
-  __shared__ __align__(16) uint32_t s_kth8[512];
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (tid < 64) s_tab[tid] = B.logtab[tid];
-  reinterpret_cast<uint4*>(s_kth8)[tid] = reinterpret_cast<const uint4*>(g_kth8.w)[tid];
-  __syncthreads();
-  const uint8_t* const kth8 = reinterpret_cast<const uint8_t*>(s_kth8);
-  const uint32_t beta = *B.beta;
-  const int par = (int)(beta & 1u);
-  const int sub = lane & (G - 1);                    // the lane's place in its group
-  const int lead = lane & ~(G - 1);                  // the group's first lane
-  const uint32_t site0 = 256u * (uint32_t)sub;       // the lane's first site
-  unsigned int leaders = 0u;                         // first lanes of all groups
-#pragma unroll
-  for (int i = 0; i < 32; i += G) leaders |= 1u << i;
-  const int W = B.W;
-  const int64_t nunits = B.nslots / unit;
-  const int64_t nwarps = (int64_t)gridDim.x * (kWideThreads / 32);
-  for (int64_t un = (int64_t)blockIdx.x * (kWideThreads / 32) + (tid >> 5); un < nunits; un += nwarps) {
-    const int64_t slot0 = un * unit;                 // a unit lies within one tile
-    const int p = B.tile_pop[slot0 / kTile];
-    const PopDesc d = B.pops[p];
-    const int64_t j0 = slot0 - d.off;
-    const int n = (int)max((int64_t)0, min((int64_t)unit, d.nc - j0));  // warp-uniform
-    const float* inv = B.inv_rate + (size_t)p * kInvStride;
-    const uint32_t k0 = (uint32_t)d.seed, k1 = (uint32_t)(d.seed >> 32);
-    const uint32_t L = (uint32_t)d.L, lm1 = L - 1u;
-    int next = 0;                                    // the unit's next clone (warp-uniform)
-    int cl = -1, h = 0;
-    uint32_t q = 0u, u[8];
-    float t = 0.0f, acc = 0.0f;
-    int hmin = INT_MAX, hmax = INT_MIN, amin = INT_MAX, amax = INT_MIN;
-    unsigned int ev = 0u;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) u[j] = 0u;
-    for (;;) {
-      const unsigned int m = __ballot_sync(0xffffffffu, cl < 0) & leaders;
-      if (m != 0u && next < n) {
-        const int idx = next + __popc(m & ((1u << lead) - 1u));
-        next += __popc(m);
-        if (cl < 0 && idx < n) {
-          cl = idx;
-          const unsigned long long* src = B.Y + (slot0 + idx) * W + 4 * sub;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const unsigned long long v = 4 * sub + j < W ? src[j] : 0ull;
-            u[2 * j] = (uint32_t)v;
-            u[2 * j + 1] = (uint32_t)(v >> 32);
-          }
-          t = acc = 0.0f;
-          h = 0;
-          q = 0u;
-        }
-      } else if (m == leaders) {
-        break;  // every group is empty and the unit has run out
-      }
-      const bool live = cl >= 0;
-      const uint4 d4 = philox4x32_10(make_uint4(q, beta, (uint32_t)(j0 + cl), kTagEvolve), k0, k1);
-      bool run = live;
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const float E = neg_ln_u(e == 0 ? d4.x : d4.z, s_tab);
-        const uint32_t wb = e == 0 ? d4.y : d4.w;
-        uint32_t nb = 0u, c0 = u[0] & 1u;            // bit 0 of the next lane, and site 0
-        if constexpr (G > 1) {
-          nb = __shfl_sync(0xffffffffu, c0, lead | ((sub + 1) & (G - 1)));
-          c0 = __shfl_sync(0xffffffffu, c0, lead);
-          if (sub == G - 1) nb = 0u;
-        }
-        uint32_t a[8], pc[8], cnt = 0u;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const uint32_t up = j < 7 ? u[(j + 1) & 7] : nb;
-          // the closing bond: site L - 1's right neighbour is site 0 (the sites above L - 1 are 0)
-          a[j] = u[j] ^ __funnelshift_r(u[j], up, 1) ^ __funnelshift_lc(0u, c0, lm1 - site0 - 32u * (uint32_t)j);
-          pc[j] = (uint32_t)__popc(a[j]);
-          cnt += pc[j];
-        }
-        uint32_t r = cnt, k;
-        if constexpr (G > 1) {
-#pragma unroll
-          for (int o = 1; o < G; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-        }
-        const float tau = __fmul_rn(E, __ldg(inv + r));
-        const float t_new = __fadd_rn(t, tau);
-        const bool moving = run && r != 0u;
-        const bool hopped = moving && t_new < dt_f;
-        if (MOD) {
-          const float seg = hopped ? tau : __fsub_rn(dt_f, t);
-          acc = moving ? __fmaf_rn((float)r, seg, acc) : acc;
-        }
-        t = hopped ? t_new : t;
-        k = __umulhi(wb, r);
-        uint32_t b;
-        if constexpr (G > 1) {
-          uint32_t incl = cnt;
-#pragma unroll
-          for (int o = 1; o < G; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o, G);
-            if (sub >= o) incl += y;
-          }
-          const uint32_t excl = incl - cnt;
-          const bool owner = excl <= k && k < incl;
-          const unsigned int om = __ballot_sync(0xffffffffu, owner);
-          // a k outside the lane's count reads the table at a place inside it
-          const uint32_t mine = site0 + kth_bond256(a, pc, owner ? k - excl : 0u, kth8);
-          const unsigned int gm = (om >> lead) & (G == 32 ? 0xffffffffu : ((1u << G) - 1u));
-          b = __shfl_sync(0xffffffffu, mine, lead + (gm ? __ffs(gm) - 1 : 0));
-        } else {
-          b = kth_bond256(a, pc, k, kth8);
-        }
-        // flip sites b and (b + 1) mod L; no hop: bond 2^30, beyond every word
-        b = hopped ? b : 1u << 30;
-        const uint32_t c = b == lm1 ? 0u : b + 1u;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          u[j] ^= __funnelshift_lc(0u, 1u, b - site0 - 32u * (uint32_t)j) ^
-                  __funnelshift_lc(0u, 1u, c - site0 - 32u * (uint32_t)j);
-        h += hopped ? 1 : 0;
-        run = hopped;
-      }
-      ++q;
-      if (run && q >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
-        B.st[p].err = kErrRange;
-        run = false;
-      }
-      if (live && !run) {
-        const int64_t slot = slot0 + cl;
-        unsigned long long* dst = B.Xb[par] + slot * W + 4 * sub;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (4 * sub + j < W) dst[j] = ((unsigned long long)u[2 * j + 1] << 32) | u[2 * j];
-        if (sub == 0) {
-          B.KXb[par][slot] = B.KY[slot] + h;
-          B.dKb[par][slot] = h;
-          if (MOD) {
-            B.Ab[par][slot] = acc;
-            amin = min(amin, __float_as_int(acc));  // A >= 0: float bits order like values
-            amax = max(amax, __float_as_int(acc));
-          }
-          hmin = min(hmin, h);
-          hmax = max(hmax, h);
-          ev += (unsigned int)h;
-        }
-        cl = -1;
-      }
-    }
-    hmin = __reduce_min_sync(0xffffffffu, hmin);
-    hmax = __reduce_max_sync(0xffffffffu, hmax);
-    ev = __reduce_add_sync(0xffffffffu, ev);
-    if (MOD) {
-      amin = __reduce_min_sync(0xffffffffu, amin);
-      amax = __reduce_max_sync(0xffffffffu, amax);
-    }
-    if (lane == 0 && n > 0) {
-      PopState* st = B.st + p;
-      atomicMin(&st->dk_min[par], hmin);
-      atomicMax(&st->dk_max[par], hmax);
-      atomicAdd(&st->events, (unsigned long long)ev);
-      if (MOD) {
-        atomicMin(&st->a_min[par], amin);
-        atomicMax(&st->a_max[par], amax);
-      }
-    }
   }
 }
 
