@@ -216,6 +216,7 @@ struct pop_batch {
   int guided_split = 1;       // GUIDED: blocks per tile of the dynamical stage (1, 2, 4, 8)
   int evolve_grid = 0;
   int evolve_grid_cap = 0;  // persistent grid at full occupancy
+  int small_threads = 0;    // pop_run in one launch (k_run_small): threads per block, 0: not
   bool s_fixed = false;
   std::vector<double> s;
   Phase phase = kReady;
@@ -592,6 +593,63 @@ int size_evolve_grid(pop_t* h) {
   return POP_OK;
 }
 
+// Whether pop_run advances the batch by whole intervals in one launch (k_run_small):
+// every population fits one tile, and there are at most three times as many as blocks of
+// its size are resident at once.  A wave of blocks takes its intervals before the next
+// wave starts, while the fused kernel's launches share the SMs between all populations:
+// populations of 1000 clones (L = 50, dt = 0.1) took 8, 8, 16, 32, 64 us per interval here
+// for 1, 152, 304, 608, 1216 of them (152 resident), and 26, 29, 31, 35, 46 us by the
+// launch sequence; at dt = 1, 27, 27, 53, 106, 212 and 94, 99, 108, 130, 194 us.
+constexpr int kSmallWaves = 3;
+bool run_small(const pop_t* h) { return h->small_threads > 0; }
+
+template <int W, bool MOD>
+int size_small_form(pop_t* h) {
+  h->small_threads = 0;
+  int64_t most = 0;
+  for (const PopDesc& d : h->desc) most = std::max(most, d.nc);
+  const int threads = (int)((most + 31) / 32 * 32);
+  const int smem = (int)sizeof(SmallSmem<W>);
+  int per_sm = 0, sms = 0;
+  POP_CUDA(cudaFuncSetAttribute(k_run_small<W, MOD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  POP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_run_small<W, MOD>, threads, smem));
+  POP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+  if (h->lay.P <= (int64_t)kSmallWaves * per_sm * sms) h->small_threads = threads;
+  return POP_OK;
+}
+
+int size_small(pop_t* h) {
+  if (!fusable(h) || h->lay.ntiles != h->lay.P) return POP_OK;
+  if (h->lay.W == 1) return h->any_mod ? size_small_form<1, true>(h) : size_small_form<1, false>(h);
+  return h->any_mod ? size_small_form<2, true>(h) : size_small_form<2, false>(h);
+}
+
+template <int W, bool MOD>
+int launch_small_form(pop_t* h, cudaStream_t st, float dt_f, uint32_t beta0, int n) {
+  kernel_begin(h, st, POP_K_GATHER_EVOLVE);
+  k_run_small<W, MOD><<<(unsigned)h->lay.P, (unsigned)h->small_threads, sizeof(SmallSmem<W>), st>>>(h->B, dt_f, beta0, n);
+  kernel_end(h, st);
+  return cuda_status(cudaGetLastError());
+}
+
+// n intervals of a batch of one-tile populations, the first of them interval beta0;
+// kSmallIntervals to a launch.
+constexpr int kSmallIntervals = 1024;
+int launch_small(pop_t* h, cudaStream_t st, float dt_f, uint32_t beta0, int64_t n) {
+  int lr = POP_OK;
+  for (int64_t at = 0; at < n && lr == POP_OK; at += kSmallIntervals) {
+    const int k = (int)std::min<int64_t>(n - at, kSmallIntervals);
+    const uint32_t b = beta0 + (uint32_t)at;
+    if (h->lay.W == 1)
+      lr = h->any_mod ? launch_small_form<1, true>(h, st, dt_f, b, k)
+                      : launch_small_form<1, false>(h, st, dt_f, b, k);
+    else
+      lr = h->any_mod ? launch_small_form<2, true>(h, st, dt_f, b, k)
+                      : launch_small_form<2, false>(h, st, dt_f, b, k);
+  }
+  return lr;
+}
+
 // n fused intervals over the chains: chain 0 on st, the others on the auxiliary
 // streams forked from st and joined back into it, each chain with its own interval
 // counter (copy_chain_counters brings them in line with the batch's counter before and
@@ -812,8 +870,7 @@ int pop_init(pop_t** out, const pop_params* params, int32_t n_pops, void* d_work
     if (cudaStreamCreateWithFlags(&h->aux_stream[c], cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_join[c], cudaEventDisableTiming) != cudaSuccess)
       return fail(POP_ERR_CUDA);
-  const int grc = size_evolve_grid(h);
-  if (grc != POP_OK) return fail(POP_ERR_CUDA);
+  if (size_evolve_grid(h) != POP_OK || size_small(h) != POP_OK) return fail(POP_ERR_CUDA);
   if (h->guided) {
     int per_sm = 0, sms = 0;
     const void* f = lay.W == 1 ? (const void*)k_evolve_guided<1> : (const void*)k_evolve_guided<2>;
@@ -897,6 +954,13 @@ int pop_run(pop_t* h, double dt, const double* s, int64_t n_intervals) {
   if (rc != POP_OK) return rc;
   if (n_intervals == 0) return POP_OK;
   const float dt_f = (float)dt;
+  if (run_small(h)) {
+    rc = launch_small(h, h->stream, dt_f, (uint32_t)(h->intervals + 1), n_intervals);
+    if (rc != POP_OK) return rc;
+    h->intervals += n_intervals;
+    h->t_obs += (double)n_intervals * dt;
+    return POP_OK;
+  }
   // fused: evolve, then (n - 1) x [weights, gather + next evolve] over the chains, then
   // weights, gather; otherwise n x [evolve, weights, gather].  The graph holds
   // kGraphIntervals of the repeated part.  The first fused interval follows the
@@ -996,11 +1060,15 @@ int pop_kernel_times(pop_t* h, double dt, const double* s, int64_t n_intervals, 
   h->timer_intervals = &ivs;
   h->timer_interval = 0;
   const float dt_f = (float)dt;
-  const bool fuse = per_step == 0 && fusable(h);
+  const bool small = per_step == 0 && run_small(h);
+  const bool fuse = per_step == 0 && !small && fusable(h);
   set_hist(h, dt_f);
   // the same launches, in the same order and on the same streams, as pop_run (or the
   // per-step calls), each interval's launches tagged with its index
-  if (fuse) {
+  if (small) {
+    rc = launch_small(h, h->stream, dt_f, (uint32_t)(h->intervals + 1), n_intervals);
+    hops1 = hops0;
+  } else if (fuse) {
     rc = launch_evolve(h, h->stream, dt_f);
     if (rc == POP_OK) rc = total_hops(&hops1);
     if (rc == POP_OK) rc = copy_chain_counters(h, true) == cudaSuccess ? POP_OK : POP_ERR_CUDA;
@@ -1086,7 +1154,7 @@ int pop_kernel_times(pop_t* h, double dt, const double* s, int64_t n_intervals, 
     if (h_hops) h_hops[k] = 0;
   }
   if (h_hops) {
-    if (fuse) {
+    if (fuse || small) {
       h_hops[POP_K_EVOLVE] = hops1 - hops0;
       h_hops[POP_K_GATHER_EVOLVE] = hops2 - hops1;
     } else {
@@ -1280,7 +1348,7 @@ int pop_autotune(pop_t* h, double dt, const double* s, int32_t trials, int32_t* 
   // the chains of pop_run and, where activities of 64 or more are very unlikely
   // (dt * (largest L) <= 16, no MODIFIED weights), whether the fused stage counts them
   // per tile, by the time per interval of `trials` fused intervals
-  if (rc == POP_OK && fusable(h)) {
+  if (rc == POP_OK && fusable(h) && !run_small(h)) {
     const int forms[3][2] = {{128, 1}, {128, 2}, {256, 1}};
     const int wants[4] = {1, 2, 4, 8};
     const int def_threads = h->fuse_threads, def_clones = h->fuse_clones, def_nch = h->nch;
@@ -1388,6 +1456,19 @@ int pop_autotune(pop_t* h, double dt, const double* s, int32_t trials, int32_t* 
     POP_CUDA(cudaMemcpyAsync(h->B.KY, h->B.KXb[0], ks, cudaMemcpyDeviceToDevice, h->stream));
     h->tuned_default_us = 1e3f * def_ms;
     h->tuned_us = 1e3f * bms;
+  }
+  // (4) batches that pop_run advances in one launch have nothing to choose there: its time
+  // (the population is kept as in (3))
+  if (rc == POP_OK && run_small(h)) {
+    const size_t lat = (size_t)h->lay.nslots * h->lay.W * sizeof(unsigned long long);
+    const size_t ks = (size_t)h->lay.nslots * sizeof(int32_t);
+    POP_CUDA(cudaMemcpyAsync(h->B.Xb[0], h->B.Y, lat, cudaMemcpyDeviceToDevice, h->stream));
+    POP_CUDA(cudaMemcpyAsync(h->B.KXb[0], h->B.KY, ks, cudaMemcpyDeviceToDevice, h->stream));
+    float ms = 0.0f;
+    rc = timed([&](bool) { return launch_small(h, h->stream, dt_f, 1u, trials); }, 3, &ms);
+    POP_CUDA(cudaMemcpyAsync(h->B.Y, h->B.Xb[0], lat, cudaMemcpyDeviceToDevice, h->stream));
+    POP_CUDA(cudaMemcpyAsync(h->B.KY, h->B.KXb[0], ks, cudaMemcpyDeviceToDevice, h->stream));
+    h->tuned_default_us = h->tuned_us = 1e3f * ms / (float)trials;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

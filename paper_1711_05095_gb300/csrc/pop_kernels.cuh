@@ -1140,6 +1140,251 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
 }
 
 // ---------------------------------------------------------------------------
+// Whole intervals of populations of at most one tile, one block per population and one
+// clone per thread: n_int intervals, beta0 the first, in one launch.  Lattices and
+// cumulative activities stay in shared memory (two buffers; a new clone starts from its
+// ancestor's in the other one, so the gather is part of taking the clone); three barriers
+// per interval.  The arithmetic is that of the separate stages, with the exact j_lo.
+// Bound by one SM's issue rate (32 warps, about 280 instructions per two steps) and the
+// latency of the barriers: 1000 clones of L = 20, dt = 0.1 take 6.5 us per interval, where
+// the launch sequence (weights, then one 128-thread block per population) took 21.8; of
+// L = 128, dt = 0.1, 13.7 and 40.3.
+// The psi terms need FP64 logarithms, slow on one thread: warp 0 keeps what they are
+// formed from and takes 32 of them at once, one per lane, then adds them in order.
+// ---------------------------------------------------------------------------
+constexpr int kSmallThreads = kTile;
+template <int W>
+struct SmallSmem {
+  unsigned long long x[2][kTile][W];
+  int32_t K[2][kTile];
+  uint16_t src[kTile];                // ancestor of each new clone
+  unsigned long long wt[64];          // the first fixed-point weights
+  unsigned long long wsum[32];
+  double pend[32][2];                 // what the psi terms of up to 32 intervals are formed from
+  float pend_a[32];
+  int32_t pend_k[32];
+  float2 logtab[64];
+  __align__(16) uint32_t kth8[512];
+  uint2 keys[10];
+  float inv[kMaxL + 1];
+  unsigned int hist[kHistSmem];
+  int32_t mn[32], mx[32], amn[32], amx[32];
+  uint32_t U[32];                     // [eq] offset words of 32 intervals
+};
+
+template <int W, bool MOD>
+__global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float dt_f, uint32_t beta0, int n_int) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SmallSmem<W>& S = *reinterpret_cast<SmallSmem<W>*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarps = (int)blockDim.x >> 5;
+  const int p = blockIdx.x;
+  const PopDesc d = B.pops[p];
+  PopState* const st = B.st + p;
+  const int n = (int)d.nc;
+  const uint32_t nc = (uint32_t)n;
+  const bool valid = tid < n;
+  const unsigned long long* const wt = B.wtab + (size_t)p * kKcap;
+  for (int r = tid; r <= kMaxL; r += (int)blockDim.x)  // inv[0] = NaN: see bkl_step_pred
+    S.inv[r] = r == 0 ? __int_as_float(0x7fffffff) : (r <= d.L) ? B.inv_rate[(size_t)p * kInvStride + r] : 0.0f;
+  for (int e = tid; e < 512; e += (int)blockDim.x) S.kth8[e] = g_kth8.w[e];
+  for (int e = tid; e < kHistSmem; e += (int)blockDim.x) S.hist[e] = 0u;
+  for (int e = tid; e < 64; e += (int)blockDim.x) {
+    S.logtab[e] = B.logtab[e];
+    S.wt[e] = wt[e];
+  }
+  if (tid < 10)
+    S.keys[tid] = make_uint2((uint32_t)d.seed + (uint32_t)tid * 0x9E3779B9u,
+                             (uint32_t)(d.seed >> 32) + (uint32_t)tid * 0xBB67AE85u);
+  if (valid) {
+    unsigned long long x[W];
+    load_lat<W>(B.Y, d.off + tid, x);
+#pragma unroll
+    for (int w = 0; w < W; ++w) S.x[0][tid][w] = x[w];
+    S.K[0][tid] = B.KY[d.off + tid];
+  }
+  S.src[tid] = (uint16_t)tid;
+  double psi = 0.0;  // thread 0: the population's accumulator
+  if (tid == 0) psi = st->psi_acc;
+  __syncthreads();
+  const uint8_t* const kth8 = reinterpret_cast<const uint8_t*>(S.kth8);
+  const uint32_t lm1 = (uint32_t)d.L - 1u;
+  unsigned long long ev = 0ull;
+  int cur = 0, h = 0;
+  for (int it = 0; it < n_int; ++it) {
+    const uint32_t beta = beta0 + (uint32_t)it;
+    if (wid == 0 && (it & 31) == 0)  // read after the first barrier below
+      S.U[lane] = philox4x32_10_rk(make_uint4(0u, beta + (uint32_t)lane, 0u, kTagResample), S.keys).x;
+    // dynamical stage: the thread's clone, from its ancestor's state
+    const int a = S.src[tid];
+    unsigned long long x[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) x[w] = S.x[cur][a][w];
+    uint32_t u[2 * W];
+    split32<W>(x, u);
+    float t = 0.0f, acc = 0.0f;
+    h = 0;
+    bool run = valid;
+    for (uint32_t q = 0u; __ballot_sync(0xffffffffu, run) != 0u; ++q) {
+      const uint4 d4 = philox4x32_10_rk(make_uint4(q, beta, (uint32_t)tid, kTagEvolve), S.keys);
+      const float E1 = neg_ln_u(d4.x, S.logtab), E2 = neg_ln_u(d4.z, S.logtab);
+      const bool h1 = bkl_step_pred<W, MOD>(u, t, acc, lm1, S.inv, E1, d4.y, dt_f, run, kth8);
+      run = bkl_step_pred<W, MOD>(u, t, acc, lm1, S.inv, E2, d4.w, dt_f, h1, kth8);
+      h += (int)h1 + (int)run;
+      if (q + 1u >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
+        if (run) st->err = kErrRange;
+        run = false;
+      }
+    }
+    join32<W>(u, x);
+    if (valid) {
+#pragma unroll
+      for (int w = 0; w < W; ++w) S.x[cur ^ 1][tid][w] = x[w];
+      S.K[cur ^ 1][tid] = S.K[cur][a] + h;
+      ev += (unsigned long long)h;
+    }
+    // the population's activity range (MOD: and that of the rate integral)
+    int mn = __reduce_min_sync(0xffffffffu, valid ? h : INT_MAX);
+    int mx = __reduce_max_sync(0xffffffffu, valid ? h : INT_MIN);
+    int amn = INT_MAX, amx = INT_MIN;
+    if (MOD) {
+      amn = __reduce_min_sync(0xffffffffu, valid ? __float_as_int(acc) : INT_MAX);  // A >= 0
+      amx = __reduce_max_sync(0xffffffffu, valid ? __float_as_int(acc) : INT_MIN);
+    }
+    if (lane == 0) {
+      S.mn[wid] = mn;
+      S.mx[wid] = mx;
+      if (MOD) {
+        S.amn[wid] = amn;
+        S.amx[wid] = amx;
+      }
+    }
+    __syncthreads();
+    mn = __reduce_min_sync(0xffffffffu, lane < nwarps ? S.mn[lane] : INT_MAX);
+    mx = __reduce_max_sync(0xffffffffu, lane < nwarps ? S.mx[lane] : INT_MIN);
+    if (MOD) {
+      amn = __reduce_min_sync(0xffffffffu, lane < nwarps ? S.amn[lane] : INT_MAX);
+      amx = __reduce_max_sync(0xffffffffu, lane < nwarps ? S.amx[lane] : INT_MIN);
+    }
+    const int kref = d.s_neg ? mx : mn;
+    const float a_ref = __int_as_float(d.s_neg ? amx : amn);
+    // weights, their sum and the activity histogram
+    unsigned long long w = 0ull;
+    if (valid) {
+      unsigned int k = 0u;
+      if (MOD && d.modified) {
+        clone_weight(d, h, kref, acc, a_ref, wt, B.exp2tab, w, k);
+      } else {
+        k = abs_diff(h, kref);
+        if (k < 64u) {
+          w = S.wt[k];
+        } else if (k < (unsigned int)kKcap) {
+          w = wt[k];
+        } else {
+          st->err = kErrRange;
+        }
+        if (k < (unsigned int)kHistSmem) atomicAdd(&S.hist[k], 1u);
+        else if (k < (unsigned int)kKcap) atomicAdd(&B.hist[(size_t)p * kKcap + k], 1u);
+      }
+    }
+    unsigned long long xs = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, xs, o);
+      if (lane >= o) xs += y;
+    }
+    if (lane == 31) S.wsum[wid] = xs;
+    __syncthreads();
+    // the warps' sums: total and what lies before this warp
+    unsigned long long ws = lane < nwarps ? S.wsum[lane] : 0ull;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, ws, o);
+      if (lane >= o) ws += y;
+    }
+    const unsigned long long T = __shfl_sync(0xffffffffu, ws, 31);
+    const unsigned long long before = wid == 0 ? 0ull : __shfl_sync(0xffffffffu, ws, wid - 1);
+    const unsigned long long c = 2ull * (unsigned long long)S.U[it & 31] + 1ull;
+    const int sh = max(0, 64 - __clzll((long long)T) - 24);
+    const float ratio = __fdiv_rn((float)nc, __uint2float_rn((uint32_t)(T >> sh)));
+    const unsigned long long w1[1] = {w};
+    uint32_t jl[2];
+    j_lo_run<1>(before + xs - w, w1, T, c, nc, sh, ratio, jl);
+    if (valid)
+      for (uint32_t jj = jl[0]; jj < jl[1]; ++jj) S.src[jj] = (uint16_t)tid;
+    if (wid == 0) {
+      // psi term of eq. (psihat), as in the separate cloning stage
+      const int slot = it & 31;
+      if (d.modified) {
+        if (lane == 0) {
+          S.pend[slot][0] = (double)((long long)T - (long long)((unsigned long long)d.nc << d.F));
+          S.pend_a[slot] = a_ref;
+        }
+      } else {
+        const int R = hist_bins(mn, mx, kKcap);
+        unsigned int* const hg = B.hist + (size_t)p * kKcap;
+        const double* qt = B.qtab + (size_t)p * kKcap;
+        const double* qm = B.qm1tab + (size_t)p * kKcap;
+        double sa = 0.0, sq = 0.0;
+        for (int b = lane; b < R; b += 32) {
+          // the global bins were added to by other threads of this block: past L1
+          const unsigned int cnt = b < kHistSmem ? S.hist[b] : __ldcg(hg + b);
+          if (cnt) {
+            sa = fma((double)cnt, qm[b], sa);
+            sq = fma((double)cnt, qt[b], sq);
+            if (b < kHistSmem) S.hist[b] = 0u;
+            else hg[b] = 0u;
+          }
+        }
+        sa = warp_sum_f64(sa);
+        sq = warp_sum_f64(sq);
+        if (lane == 0) {
+          S.pend[slot][0] = sa;
+          S.pend[slot][1] = sq;
+          S.pend_k[slot] = kref;
+        }
+      }
+      if (slot == 31 || it == n_int - 1) {
+        __syncwarp();
+        double term = 0.0;
+        if (lane <= slot) {
+          if (d.modified) {
+            const double base_w = ldexp((double)d.nc, d.F);
+            const double ref = -(double)d.c_f * (double)S.pend_a[lane];
+            term = ref + log1p(S.pend[lane][0] / base_w);
+          } else {
+            const double ncd = (double)d.nc;
+            const double mean_q = S.pend[lane][1] / ncd;
+            const double ln_mean = (mean_q > 0.5) ? log1p(S.pend[lane][0] / ncd) : log(mean_q);
+            term = -d.s * (double)S.pend_k[lane] + ln_mean;
+          }
+        }
+        for (int e = 0; e <= slot; ++e) psi += __shfl_sync(0xffffffffu, term, e);
+      }
+    }
+    __syncthreads();
+    cur ^= 1;
+  }
+  // the population after the last cloning stage, its ancestors and activities
+  if (valid) {
+    const int a = S.src[tid];
+    unsigned long long x[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) x[w] = S.x[cur][a][w];
+    const int64_t slot = d.off + tid;
+    store_lat<W>(B.Y, slot, x);
+    B.KY[slot] = S.K[cur][a];
+    B.anc[slot] = a;
+    B.dKb[(beta0 + (uint32_t)n_int - 1u) & 1u][slot] = h;
+  }
+  ev = warp_sum_u64(ev);
+  if (lane == 0) atomicAdd(&st->events, ev);
+  if (tid == 0) {
+    st->psi_acc = psi;
+    if (p == 0) *B.beta = beta0 + (uint32_t)n_int;  // beta0 came with the launch: no block reads the counter
+  }
+}
+
+// ---------------------------------------------------------------------------
 // [iid] selection (Sec. 4.1): new clone j of the population pulls old clone k with
 // S_k <= alpha_j < S_{k+1}, alpha_j = floor(U64_j T / 2^64), U64_j from draw
 // (j, beta, 0, 4).  The search runs in two levels over the same non-decreasing prefix

@@ -672,3 +672,67 @@ def test_parity_at_the_edges_of_the_lanes_of_a_wide_ring(pg, L, nc, mode, sel):
     pops = [dict(L=L, N=L // 3, n_clones=nc, seed=300 + L, weight_mode=mode, selection=sel),
             dict(L=11, N=5, n_clones=nc + 3, seed=301 + L, selection=sel)]
     run_parity(pg, pops, [10.0 / L ** 2, -0.1], 8.0 / L, 3)
+
+
+@pytest.mark.parametrize("pops,s,dt,splits", [
+    ([dict(L=20, N=10, n_clones=1, seed=1)], [0.3], 0.1, [2, 1]),
+    ([dict(L=20, N=10, n_clones=31, seed=2), dict(L=50, N=25, n_clones=33, seed=3)], [0.3, -0.1], 0.1, [31, 1, 33]),
+    ([dict(L=64, N=32, n_clones=1024, seed=4), dict(L=3, N=1, n_clones=32, seed=5, weight_mode=MOD)],
+     [0.02, 0.4], 0.2, [34]),                    # every thread a clone; MODIFIED beside plain
+    ([dict(L=65, N=30, n_clones=1023, seed=6, weight_mode=MOD), dict(L=12, N=0, n_clones=40, seed=7, weight_mode=MOD)],
+     [-0.05, 0.3], 0.3, [40]),                   # two words; an empty ring
+    ([dict(L=128, N=64, n_clones=700, seed=8), dict(L=40, N=20, n_clones=900, seed=9)], [0.5, 2.5], 0.2, [33]),
+    ([dict(L=128, N=1, n_clones=1000, seed=10)], [1e-4], 3000.0, [2]),  # activities over more bins than shared memory counts
+    ([dict(L=16, N=8, n_clones=40, seed=11)], [0.1], 0.1, [1030]),      # more intervals than one launch takes
+])
+def test_one_tile_populations_run_equals_steps(pg, pops, s, dt, splits):
+    a = pg.PopulationBatch(pops)
+    b = pg.PopulationBatch(pops)
+    for n in splits:
+        a.run(dt, s, n)
+    assert a.launch_count()["gather_evolve"] == sum((n + 1023) // 1024 for n in splits)
+    for _ in range(sum(splits)):
+        b.evolve(dt, s)
+        b.resample()
+    for p in range(len(pops)):
+        ga, gb = a.copy_state(p), b.copy_state(p)
+        for key in ("lattice", "K", "anc", "dK"):
+            assert np.array_equal(ga[key], gb[key]), (p, key)
+    pa, ka, ta = a.estimate_psi()
+    pb, kb, tb = b.estimate_psi()
+    np.testing.assert_allclose(pa * ta, pb * tb, rtol=1e-15)
+    np.testing.assert_allclose(ka * ta, kb * tb, rtol=1e-14)
+    np.testing.assert_array_equal(a.events(), b.events())
+    a.evolve(dt, s)                             # and the per-step calls go on from there
+    b.run(dt, s, 1)
+    a.resample()
+    assert np.array_equal(a.copy_state(0)["lattice"], b.copy_state(0)["lattice"])
+
+
+def test_one_tile_populations_tune_and_time_without_changing_results(pg):
+    pops = [dict(L=50, N=25, n_clones=500 + 100 * i, seed=80 + i) for i in range(4)]
+    s = [0.01, 0.02, -0.01, 0.0]
+    a, b, c = (pg.PopulationBatch(pops) for _ in range(3))
+    assert a.autotune(0.1, s)["tuned_us_per_interval"] > 0.0
+    for x in (a, b):
+        x.run(0.1, s, 36)
+    kt = c.kernel_times(0.1, s, 36)
+    assert kt["gather_evolve"][1] == 1 and kt["gather_evolve"][2] == int(c.events().sum())
+    for p in range(4):
+        ga, gb, gc = (x.copy_state(p) for x in (a, b, c))
+        for key in ("lattice", "K", "anc", "dK"):
+            assert np.array_equal(ga[key], gb[key]) and np.array_equal(gc[key], gb[key]), (p, key)
+
+
+def test_many_one_tile_populations_keep_the_launch_sequence(pg):
+    # four times as many populations as blocks of 1024 threads the device holds
+    import torch
+    P = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    pops = [dict(L=20, N=10, n_clones=1000 + i % 3, seed=i) for i in range(P)]
+    a = pg.PopulationBatch(pops)
+    a.run(0.1, [0.05] * P, 3)
+    assert a.launch_count()["evolve"] == 1
+    b = pg.PopulationBatch(pops[:5])
+    b.run(0.1, [0.05] * 5, 3)
+    for p in range(5):
+        assert np.array_equal(a.copy_state(p)["lattice"], b.copy_state(p)["lattice"])
