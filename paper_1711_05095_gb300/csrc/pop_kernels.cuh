@@ -765,7 +765,8 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     }
     if (tid == NT - 1) s_J1 = jl[NI];
   };
-  if (!d.iid) {
+  const bool iid = !FUSE && d.iid;  // batches with [iid] populations do not fuse
+  if (!iid) {
     unsigned long long u[NI], sum = 0ull;
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
@@ -792,7 +793,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     fill_map();
     near = __syncthreads_or(near) != 0;
   }
-  if (d.iid || near) {
+  if (iid || near) {
     // a position too close to a slot, or [iid]: the exact prefix sums
     const unsigned long long T = s_T;
     unsigned long long w[NI], sum = 0ull;
@@ -807,13 +808,23 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     } else {
       for (int i = 0; i < lt; ++i) run += B.tile_sum[d.first_tile + i];
     }
-    if (d.iid) {
-      // publish this tile's prefix sums; k_select_iid draws the points
+    if (iid) {
+      // publish this tile's prefix sums; k_select_iid draws the points.  jl: the guide
+      // table's slots, the multiples of 2^f at or (by the rounding of a position) a little
+      // beyond the position of each prefix sum, so a guide entry is never too late; a
+      // function of the prefix sum alone, so the tiles' ranges meet
 #pragma unroll
-      for (int i = 0; i < NI; ++i) {
-        B.S[base + (int64_t)tid * NI + i] = run;
-        run += w[i];
+      for (int i = 0; i <= NI; ++i) {
+        if (i < NI) B.S[base + (int64_t)tid * NI + i] = run;
+        const unsigned long long e = pos_of(run, s_ps) + ((1ull << (d.F + 1)) - 1ull) + kPosMargin;
+        jl[i] = run == 0ull ? 0u : min((uint32_t)(e >> (d.F + 1)), nc);
+        if (i < NI) run += w[i];
       }
+      if (tid == 0) s_J0 = jl[0];
+      __syncthreads();
+      J0 = s_J0;
+      fill_map();
+      __syncthreads();
       if (lt == 0 && tid == 0) st->T = T;
     } else {
       const int sh = max(0, 64 - __clzll((long long)T) - 24);
@@ -826,7 +837,6 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
       __syncthreads();
     }
   }
-  if (!d.iid) {
   J1 = s_J1;
   const bool mapped = (J1 - J0) <= (uint32_t)kMap;
   if (!mapped) {
@@ -1066,6 +1076,9 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
       }
       if (ovf) st->hovf = 1;
     }
+  } else if (iid) {
+    int32_t* const guide = B.dKb[par ^ 1];  // the last interval's activities are no longer needed
+    for (uint32_t jj = J0 + (uint32_t)tid; jj < J1; jj += NT) guide[d.off + (int64_t)jj] = lt * kTile + source(jj);
   } else if constexpr (W > 0) {
     for (uint32_t jj = J0 + (uint32_t)tid; jj < J1; jj += NT) {
       const int k = source(jj);
@@ -1086,7 +1099,6 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
       B.anc[dst] = lt * kTile + k;
     }
   }
-  }  // [eq]
 
   // psi term of eq. (psihat) for this interval, once per population.
   // MODIFIED (reading of eq. def-ups-ssep): -c A_ref + log1p((T - N_c 2^F) / (N_c 2^F))
@@ -1387,59 +1399,80 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
 // ---------------------------------------------------------------------------
 // [iid] selection (Sec. 4.1): new clone j of the population pulls old clone k with
 // S_k <= alpha_j < S_{k+1}, alpha_j = floor(U64_j T / 2^64), U64_j from draw
-// (j, beta, 0, 4).  The search runs in two levels over the same non-decreasing prefix
-// sums: the last tile whose first prefix (k_tile_scan's tile_excl) is <= alpha_j,
-// from a shared-memory copy of the population's tile prefixes, then the last k of
-// that tile with S_k <= alpha_j.  One block per tile of new slots; populations with
-// [eq] selection are skipped.  The last block advances the interval counter.
+// (j, beta, 0, 4).  The search starts from the guide table of the cloning stage: entry m
+// is a clone with S_k <= m T / N_c, as close to it as the clones allow, and alpha_j lies
+// at or beyond m T / N_c for m = floor(U64_j N_c / 2^64), so the answer is one or two
+// clones further on: three or four loads, where a bisection of the tile's 1024 prefix sums
+// was ten in a row behind one another (an interval of 2^21 clones of L = 50, dt = 1:
+// 462 us with that, 395 us so).  A run of tiny weights is bisected.  One block per tile of new slots; populations with [eq] selection are
+// skipped.  The last block advances the interval counter.
 // ---------------------------------------------------------------------------
-constexpr int kIidSmemTiles = 2048;  // tile prefixes kept in shared memory (16 KB)
 template <int W>
 __global__ void __launch_bounds__(kThreads) k_select_iid(Batch B) {
-  __shared__ unsigned long long s_te[kIidSmemTiles];
   const int tid = threadIdx.x;
   const int tile = blockIdx.x;
   const int p = B.tile_pop[tile];
   const PopDesc d = B.pops[p];
   if (d.iid) {
-    const unsigned long long* te = B.tile_excl + d.first_tile;
-    const bool staged = d.ntiles <= kIidSmemTiles;
-    if (staged)
-      for (int i = tid; i < d.ntiles; i += kThreads) s_te[i] = te[i];
-    __syncthreads();
     const PopState* st = B.st + p;
     const unsigned long long T = st->T;
     const uint32_t beta = st->beta;
     const int par = (int)(beta & 1u);
     const unsigned long long* const Xo = B.Xb[par];
     const int32_t* const KXo = B.KXb[par];
+    const int32_t* const guide = B.dKb[par ^ 1] + d.off;
     const int lt = tile - d.first_tile;
     const unsigned long long* S = B.S + d.off;
     const uint32_t k0 = (uint32_t)d.seed, k1 = (uint32_t)(d.seed >> 32);
-    for (int i = tid; i < kTile; i += kThreads) {
-      const int64_t j = (int64_t)lt * kTile + i;
-      if (j >= d.nc) break;
-      const uint4 r = philox4x32_10(make_uint4((uint32_t)j, beta, 0u, kTagIid), k0, k1);
-      const unsigned long long alpha = __umul64hi(((unsigned long long)r.y << 32) | r.x, T);
-      int tlo = 0, thi = d.ntiles - 1;  // the last tile whose first prefix is <= alpha
-      while (tlo < thi) {
-        const int mid = (tlo + thi + 1) >> 1;
-        if ((staged ? s_te[mid] : te[mid]) <= alpha) tlo = mid; else thi = mid - 1;
+    const int nc = (int)d.nc;
+    // the thread's clones side by side, so their loads overlap
+    unsigned long long alpha[kItems];
+    int k[kItems];
+    bool on[kItems];  // the answer may lie further on
+#pragma unroll
+    for (int i = 0; i < kItems; ++i) {
+      const uint32_t j = (uint32_t)(lt * kTile + i * kThreads + tid);
+      const uint4 r = philox4x32_10(make_uint4(j, beta, 0u, kTagIid), k0, k1);
+      const unsigned long long u64 = ((unsigned long long)r.y << 32) | r.x;
+      alpha[i] = __umul64hi(u64, T);
+      k[i] = guide[(int)__umul64hi(u64, (unsigned long long)nc)];
+    }
+#pragma unroll
+    for (int i = 0; i < kItems; ++i) {
+      // two at a time: the prefix sums of neighbours come together
+      const unsigned long long s1 = S[min(k[i] + 1, nc - 1)], s2 = S[min(k[i] + 2, nc - 1)];
+      const bool f1 = k[i] + 1 < nc && s1 <= alpha[i];
+      on[i] = k[i] + 2 < nc && s2 <= alpha[i];
+      k[i] += on[i] ? 2 : (f1 ? 1 : 0);
+    }
+#pragma unroll
+    for (int i = 0; i < kItems; ++i) {
+      for (int e = 0; e < 6 && on[i]; ++e) {
+        on[i] = k[i] + 1 < nc && S[k[i] + 1] <= alpha[i];
+        if (on[i]) ++k[i];
       }
-      long long lo = (long long)tlo * kTile;  // the last k of the tile with S_k <= alpha
-      long long hi = min((long long)d.nc, lo + kTile) - 1;
-      while (lo < hi) {
-        const long long mid = lo + (hi - lo + 1) / 2;
-        if (S[mid] <= alpha) lo = mid; else hi = mid - 1;
+      if (on[i]) {
+        int lo = k[i], hi = nc - 1;  // the last k with S_k <= alpha
+        while (lo < hi) {
+          const int mid = lo + (hi - lo + 1) / 2;
+          if (S[mid] <= alpha[i]) lo = mid; else hi = mid - 1;
+        }
+        k[i] = lo;
       }
-      const int64_t src = d.off + lo, dst = d.off + j;
-      if constexpr (W > 0) {  // wide lattices: k_copy_wide copies the words
-        unsigned long long x[W];
-        load_lat<W>(Xo, src, x);
-        store_lat<W>(B.Y, dst, x);
+    }
+#pragma unroll
+    for (int i = 0; i < kItems; ++i) {
+      const int64_t j = (int64_t)lt * kTile + i * kThreads + tid;
+      if (j < d.nc) {
+        const int64_t src = d.off + k[i], dst = d.off + j;
+        if constexpr (W > 0) {  // wide lattices: k_copy_wide copies the words
+          unsigned long long x[W];
+          load_lat<W>(Xo, src, x);
+          store_lat<W>(B.Y, dst, x);
+        }
+        B.KY[dst] = KXo[src];
+        B.anc[dst] = k[i];
       }
-      B.KY[dst] = KXo[src];
-      B.anc[dst] = (int32_t)lo;
     }
   }
   if (blockIdx.x == gridDim.x - 1 && tid == 0) *B.beta += 1u;

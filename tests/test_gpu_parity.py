@@ -736,3 +736,13 @@ def test_many_one_tile_populations_keep_the_launch_sequence(pg):
     b.run(0.1, [0.05] * 5, 3)
     for p in range(5):
         assert np.array_equal(a.copy_state(p)["lattice"], b.copy_state(p)["lattice"])
+
+
+@pytest.mark.parametrize("mode,sel", [(0, IID), (MOD, IID), (0, 0)])
+@pytest.mark.parametrize("L,nc,s,dt", [
+    (40, 5000, 2.5, 0.3),    # long runs of tiny weights
+    (10, 9000, 6.0, 2.0),    # a few clones own nearly every new slot, more than a tile's map holds
+    (20, 2049, -1.5, 0.3),   # the largest activity is the reference; a tile of one clone
+])
+def test_parity_under_strong_bias(pg, L, nc, s, dt, mode, sel):
+    run_parity(pg, [dict(L=L, N=L // 2, n_clones=nc, seed=600 + L, weight_mode=mode, selection=sel)], [s], dt, 3)
