@@ -213,7 +213,6 @@ struct pop_batch {
   bool any_mod = false;
   bool guided = false;       // every population GUIDED
   bool guided_q_stale = true; // GUIDED: the rate tables need (re)building once s is fixed
-  int guided_split = 1;       // GUIDED: blocks per tile of the dynamical stage (1, 2, 4, 8)
   int evolve_grid = 0;
   int evolve_grid_cap = 0;  // persistent grid at full occupancy
   int small_threads = 0;    // pop_run in one launch (k_run_small): threads per block, 0: not
@@ -345,7 +344,6 @@ void kernel_end(pop_t* h, cudaStream_t st) {
 
 // The dynamical stage's kernel for a batch: words per lane and lanes per clone by the
 // largest ring, the form for rings that fill one or two 64-bit words where every one does.
-// FULL and MODIFIED are combined only where they occur together in use.
 typedef void (*EvolveKernel)(Batch, float);
 
 int evolve_lanes(const pop_t* h) {
@@ -370,21 +368,13 @@ EvolveKernel evolve_kernel_of(const pop_t* h) {
 }
 
 EvolveKernel evolve_kernel(const pop_t* h) {
+  if (h->guided) return h->lay.W == 1 ? k_evolve_guided<1> : k_evolve_guided<2>;
   return h->any_mod ? evolve_kernel_of<true>(h) : evolve_kernel_of<false>(h);
 }
 
 int launch_evolve(pop_t* h, cudaStream_t st, float dt_f) {
   kernel_begin(h, st, POP_K_EVOLVE);
-  if (h->guided) {
-    // a tile per block, or a half, quarter or eighth of one for a batch of fewer tiles
-    // than two waves of blocks
-    const int spb = kTile / h->guided_split;
-    const unsigned gg = (unsigned)((int64_t)h->lay.ntiles * h->guided_split);
-    if (h->lay.W == 1) k_evolve_guided<1><<<gg, kGuideThreads, 0, st>>>(h->B, dt_f, spb);
-    else k_evolve_guided<2><<<gg, kGuideThreads, 0, st>>>(h->B, dt_f, spb);
-  } else {
-    evolve_kernel(h)<<<(unsigned)h->evolve_grid, kEvolveThreads, 0, st>>>(h->B, dt_f);
-  }
+  evolve_kernel(h)<<<(unsigned)h->evolve_grid, kEvolveThreads, 0, st>>>(h->B, dt_f);
   kernel_end(h, st);
   return cuda_status(cudaGetLastError());
 }
@@ -871,15 +861,6 @@ int pop_init(pop_t** out, const pop_params* params, int32_t n_pops, void* d_work
         cudaEventCreateWithFlags(&h->ev_join[c], cudaEventDisableTiming) != cudaSuccess)
       return fail(POP_ERR_CUDA);
   if (size_evolve_grid(h) != POP_OK || size_small(h) != POP_OK) return fail(POP_ERR_CUDA);
-  if (h->guided) {
-    int per_sm = 0, sms = 0;
-    const void* f = lay.W == 1 ? (const void*)k_evolve_guided<1> : (const void*)k_evolve_guided<2>;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kGuideThreads, 0) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
-      return fail(POP_ERR_CUDA);
-    const long long want = 2ll * (per_sm < 1 ? 1 : per_sm) * sms;
-    while (h->guided_split < 8 && (long long)lay.ntiles * h->guided_split < want) h->guided_split *= 2;
-  }
 
   const unsigned grid = (unsigned)(lay.nslots / kThreads);
   h->launches[POP_K_OTHER] += 1;

@@ -1497,15 +1497,17 @@ __global__ void __launch_bounds__(kThreads) k_select_iid(Batch B) {
 // this is the weight of the rates simulated, so the estimate is unbiased for any
 // potential.  Requires 18 <= L <= 128.
 // ---------------------------------------------------------------------------
-constexpr int kGuideThreads = 128;
+constexpr int kGuideThreads = kEvolveThreads;
 constexpr int kGuideGroup = 8;              // bonds per rate-sum group
 constexpr int kGuideSegBits = 17;
 constexpr int kGuideSeg = 1 << kGuideSegBits;
 
-// The table index of an active bond's segment: its bits 0..8 (sites b-8..b) and
-// 10..17 (sites b+2..b+9); bit 9 (site b+1) is the complement of bit 8.
-__device__ __forceinline__ uint32_t guided_index(uint32_t seg) {
-  return (seg & 0x1FFu) | ((seg >> 10) << 9);
+// The table index of an active bond's segment (sites b-8 .. b+9): sites b-8 .. b-1 are
+// its bits 0..7 and sites b+1 .. b+9 its bits 8..16; site b is the complement of b+1.  For
+// the bond whose segment starts at bit o of a window v: v's bits o..o+7, and from bit o+1
+// on the bits 8..16, so neighbouring bonds share a shift.
+__device__ __forceinline__ uint32_t guided_index(uint32_t v, int o) {
+  return ((v >> o) & 0xFFu) | ((v >> (o + 1)) & 0x1FF00u);
 }
 
 // Q(k) = floor(TA[a] TB[c] / 2^44).
@@ -1519,8 +1521,8 @@ __device__ __forceinline__ unsigned long long guided_q(int k, const unsigned lon
 __global__ void __launch_bounds__(kThreads) k_guided_table(Batch B, int p) {
   const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
   if (i >= (uint32_t)kGuideSeg) return;
-  const uint32_t b8 = (i >> 8) & 1u;
-  const uint32_t seg = (i & 0x1FFu) | ((b8 ^ 1u) << 9) | ((i >> 9) << 10);
+  const uint32_t next = (i >> 8) & 1u;  // site b+1
+  const uint32_t seg = (i & 0xFFu) | ((next ^ 1u) << 8) | ((i >> 8) << 9);
   const uint32_t seg2 = seg ^ (3u << 8);
   const int32_t* phi = B.phi + (size_t)p * 512;
   int dU = 0;
@@ -1537,43 +1539,6 @@ __global__ void __launch_bounds__(kThreads) k_guided_qtab(Batch B) {
   const size_t at = (size_t)p * kGuideSeg + i;
   const int k = min(max(B.gdu[at] - s_q, -kGuideKmax), kGuideKmax);
   B.gq[at] = guided_q(k, B.gtab);
-}
-
-// Sites start, start+1, ..., start+63 (mod L) of a configuration as the bits of one
-// word (bit k = site (start + k) mod L), 18 <= L, 0 <= start < L; bits of x at or
-// above L are zero.
-template <int W>
-__device__ __forceinline__ unsigned long long ring_window(const unsigned long long (&x)[W], int L,
-                                                         int start) {
-  if (W == 1 || L <= 64) {
-    const unsigned long long x0 = x[0];
-    unsigned long long y = (start == 0) ? x0 : ((x0 >> start) | (x0 << (L - start)));
-    if (L < 64) {
-      y &= (1ull << L) - 1ull;
-      y |= y << L;                       // 2L >= 36 sites
-      if (2 * L < 64) y |= y << (2 * L);  // 4L >= 72 sites
-    }
-    return y;
-  } else {
-    const unsigned long long x0 = x[0], x1 = x[W - 1];
-    unsigned long long y = (start == 0) ? x0 : (start < 64 ? ((x0 >> start) | (x1 << (64 - start)))
-                                                           : (x1 >> (start - 64)));
-    const int valid = L - start;  // sites before the wrap to site 0
-    if (valid < 64) y |= x0 << valid;
-    return y;
-  }
-}
-
-// Rate of the bond whose 18-site segment starts at bit o of window v (its sites at bits
-// o + 8 and o + 9): Q from the table if they differ, else 0 (the table is read only for
-// an active bond).
-__device__ __forceinline__ unsigned long long guided_q_at(unsigned long long v, int o,
-                                                          const unsigned long long* qtab) {
-  const uint32_t seg = (uint32_t)(v >> o) & 0x3FFFFu;
-  const bool act = ((seg >> 8) ^ (seg >> 9)) & 1u;
-  unsigned long long q = 0ull;
-  if (act) q = __ldg(qtab + guided_index(seg));
-  return q;
 }
 
 // float(v) rounded to nearest (ties to even) for a 64-bit unsigned v, in 32-bit integer
@@ -1605,249 +1570,274 @@ __device__ __forceinline__ float i64_to_float_rn(long long v) {
   return v < 0 ? -f : f;
 }
 
-// One lane per clone; a lane whose clone has ended takes the next clone of the block's
-// share of a tile (spb slots: a whole tile, or a half, quarter or eighth of one for a
-// batch of few tiles, so that it still fills the GPU).  The rate sums of a clone's
-// groups of eight bonds live in shared memory
-// (group-major: the lanes of a warp never share a bank); a newly taken clone's sums
-// are formed by the whole warp (each lane four or two bonds), so refills stay uniform.
+// One lane per clone.  A persistent grid as k_evolve's: each warp has an even share of the
+// slots and walks it tile by tile, a lane whose clone ended takes the share's next one.
+// Per lane in shared memory: the rate sums of the clone's groups of eight bonds and its
+// sites as a bit string that starts eight sites before site 0 and goes on past the closing
+// bond, so the sites that rate group g are the 25 bits from bit 8 g on, one unaligned word.
+// A hop across bond b changes the rates of the bonds b-9 .. b+9, whose segments see site b
+// or b+1; the three or four groups that hold them are summed anew (about half of their
+// bonds are active, and only those read the table).
+// Bound by issue and by the latency of the table loads.  32 populations of 2^14 clones,
+// L = 128, dt = 0.05: 405 us per interval with a block's share of at most a tile (one
+// clone per lane and no refill for this batch: 13.4 of 32 lanes), windows cut from the
+// lattice words and each of the 19 bonds re-rated before and after the hop; 230 us now.
 #ifndef POP_GUIDE_MIN_BLOCKS
-#define POP_GUIDE_MIN_BLOCKS 8   // 64 registers, 32 warps per SM (5 blocks at 96 registers: 5 % slower)
-#endif
-#ifndef POP_GUIDE1_MIN_BLOCKS
-#define POP_GUIDE1_MIN_BLOCKS 8  // one-word lattices too (1 block at 140 registers and
-                                 // unpredicated table loads: 1.3x slower)
+#define POP_GUIDE_MIN_BLOCKS 8   // 64 registers, 32 warps per SM
 #endif
 
-template <int W>
-__global__ void __launch_bounds__(kGuideThreads, W == 1 ? POP_GUIDE1_MIN_BLOCKS : POP_GUIDE_MIN_BLOCKS)
-    k_evolve_guided(Batch B, float dt_f, int spb) {
-  constexpr int nb = 64 * W, ng = nb / kGuideGroup;
-  constexpr int BPL = nb / 32;  // bonds per lane in the cooperative sums
-  __shared__ unsigned long long s_g[ng][kGuideThreads];
-  __shared__ float2 s_log[64];
-  __shared__ int s_take;
-  __shared__ int s_min, s_max, s_amin, s_amax;
-  __shared__ unsigned int s_ev;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int64_t base = (int64_t)blockIdx.x * spb;  // the block's first slot
-  const int p = B.tile_pop[base / kTile];
-  const PopDesc d = B.pops[p];
-  if (tid < 64) s_log[tid] = B.logtab[tid];
-  if (tid == 0) {
-    s_take = 0;
-    s_min = INT_MAX;
-    s_max = INT_MIN;
-    s_amin = INT_MAX;
-    s_amax = INT_MIN;
-    s_ev = 0u;
+// Rate sum of the bonds of one group: v its window, am its active bonds.
+__device__ __forceinline__ unsigned long long guided_group(uint32_t v, uint32_t am, const unsigned long long* qtab) {
+  unsigned long long q[kGuideGroup];
+#pragma unroll
+  for (int i = 0; i < kGuideGroup; ++i) {
+    q[i] = 0ull;
+    if ((am >> i) & 1u) q[i] = __ldg(qtab + guided_index(v, i));
   }
+  return ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
+}
+
+template <int W>
+__global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_guided(Batch B, float dt_f) {
+  constexpr int nb = 64 * W, ng = nb / kGuideGroup, NW = 2 * W, NE = NW + 1;
+  constexpr int kWarpsG = kGuideThreads / 32;
+  __shared__ unsigned long long s_g[ng][kGuideThreads];
+  __shared__ uint32_t s_e[NE][kGuideThreads];        // bit t: site (t - 8) mod L, t < L + 17
+  __shared__ float2 s_log[64];
+  __shared__ uint2 s_key[kWarpsG][10];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (tid < 64) s_log[tid] = B.logtab[tid];
   __syncthreads();
   const uint32_t beta = *B.beta;
   const int par = (int)(beta & 1u);
-  const int n = (int)max((int64_t)0, min((int64_t)spb, d.nc - (base - d.off)));  // clones of the block
-  const int L = d.L;
-  const unsigned long long* const qtab = B.gq + (size_t)p * kGuideSeg;
-  const int32_t* const dtab = B.gdu + (size_t)p * kGuideSeg;
-  const uint32_t k0 = (uint32_t)d.seed, k1 = (uint32_t)(d.seed >> 32);
   const unsigned int lt_mask = (1u << lane) - 1u;
-  // the rate sums of the clones' final configurations of the last interval, if carried:
-  // a new clone starts from its ancestor's
-  const bool carry = B.st[p].gcarry != 0;
   const unsigned long long* const gin = B.gcar[par ^ 1];
   unsigned long long* const gout = B.gcar[par];
-  int cl = -1;  // the lane's clone (offset in the tile), -1 when it has none
-  unsigned long long x[W], a[W];
-  unsigned long long R = 0ull;
-  int r = 0, h = 0;
-  uint32_t e = 0u;
-  float t = 0.0f, a_r = 0.0f, a_h = 0.0f;
-  int hmin = INT_MAX, hmax = INT_MIN, xmin = INT_MAX, xmax = INT_MIN;
-  unsigned int ev = 0u;
+  const int64_t wi = (int64_t)blockIdx.x * kWarpsG + wid;
+  int64_t slot0 = (wi * B.unit_q + min(wi, B.unit_r)) * 32;
+  const int64_t slot_end = slot0 + (B.unit_q + (wi < B.unit_r ? 1 : 0)) * 32;
+  while (slot0 < slot_end) {
+    const int64_t seg_end = min(slot_end, (slot0 / kTile + 1) * kTile);  // one tile, one population
+    const int p = B.tile_pop[slot0 / kTile];
+    const PopDesc d = B.pops[p];
+    const int64_t j0 = slot0 - d.off;
+    const int n = (int)max((int64_t)0, min(seg_end - slot0, d.nc - j0));  // warp-uniform
+    const int L = d.L;
+    const uint32_t lm1 = (uint32_t)L - 1u;
+    const unsigned long long* const qtab = B.gq + (size_t)p * kGuideSeg;
+    const int32_t* const dtab = B.gdu + (size_t)p * kGuideSeg;
+    if (lane < 10)
+      s_key[wid][lane] = make_uint2((uint32_t)d.seed + (uint32_t)lane * 0x9E3779B9u,
+                                    (uint32_t)(d.seed >> 32) + (uint32_t)lane * 0xBB67AE85u);
+    __syncwarp();
+    // the rate sums of the clones' final configurations of the last interval, if carried:
+    // a new clone starts from its ancestor's
+    const bool carry = B.st[p].gcarry != 0;
+    // the lane's bit string from its lattice words
+    const int hw = (L - 8) >> 5, hs = (L - 8) & 31;    // sites L-8 .. L-1 go in front
+    const int tw = (L + 8) >> 5, ts = (L + 8) & 31;    // sites 0 .. 8 again behind
+    auto put_string = [&](const uint32_t (&u)[NW]) {
+      uint32_t lo = u[0], up = NW > 1 ? u[1] : 0u;
 #pragma unroll
-  for (int w = 0; w < W; ++w) x[w] = a[w] = 0ull;
-  for (;;) {
-    const unsigned int m = __ballot_sync(0xffffffffu, cl < 0);
-    int taken = 0;
-    if (lane == 0) taken = *(volatile int*)&s_take;
-    taken = __shfl_sync(0xffffffffu, taken, 0);
-    if (m != 0u && taken < n) {
-      int base_i = 0;
-      if (lane == 0) base_i = atomicAdd(&s_take, __popc(m));
-      base_i = __shfl_sync(0xffffffffu, base_i, 0);
-      const int idx = base_i + __popc(m & lt_mask);
-      const bool got = cl < 0 && idx < n;
-      if (got) {
-        cl = idx;
-        load_lat<W>(B.Y, base + idx, x);
-        active_bonds<W>(x, L, a);
-        r = popc_lat<W>(a);
-        h = 0;
-        e = 0u;
-        t = a_r = a_h = 0.0f;
-        if (carry) {
-          const unsigned long long* src = gin + (d.off + (int64_t)B.anc[base + idx]) * ng;
-          R = 0ull;
-#pragma unroll
-          for (int g = 0; g < ng; ++g) {
-            const unsigned long long v = src[g];
-            s_g[g][tid] = v;
-            R += v;
-          }
+      for (int j = 1; j < NW; ++j)
+        if (hw == j) {
+          lo = u[j];
+          up = j + 1 < NW ? u[(j + 1) % NW] : 0u;
         }
+      const uint32_t head = __funnelshift_r(lo, up, hs) & 0xFFu, tail = u[0] & 0x1FFu;
+      const uint32_t t0 = tail << ts, t1 = (tail >> 1) >> (31 - ts);
+#pragma unroll
+      for (int j = 0; j < NE; ++j) {
+        uint32_t e = j == 0 ? (u[0] << 8) | head : (j < NW ? __funnelshift_l(u[j - 1], u[j % NW], 8) : u[NW - 1] >> 24);
+        if (j == tw) e |= t0;
+        if (j == tw + 1) e |= t1;
+        s_e[j][tid] = e;
       }
-      // the rate sums of every new clone without carried ones, one clone at a time by
-      // the whole warp
-      unsigned int todo = __ballot_sync(0xffffffffu, got && !carry);
-      while (todo != 0u) {
-        const int o = __ffs(todo) - 1;
-        todo &= todo - 1u;
-        unsigned long long xo[W];
+    };
+    // window of group g of the clone whose string lies in column col, and its active bonds
+    auto window = [&](int g, int col) {
+      return __funnelshift_r(s_e[g >> 2][col], s_e[(g >> 2) + 1][col], 8 * (g & 3));
+    };
+    auto active = [&](uint32_t v, int g) {
+      const int m = L - kGuideGroup * g;               // bonds of the group
+      return ((v ^ (v >> 1)) >> 8) & (m >= kGuideGroup ? 0xFFu : m > 0 ? (1u << m) - 1u : 0u);
+    };
+    int next = 0;                                      // the segment's next clone (warp-uniform)
+    int cl = -1, r = 0, h = 0;
+    uint32_t u[NW], e = 0u;
+    unsigned long long R = 0ull;
+    float t = 0.0f, a_r = 0.0f, a_h = 0.0f;
+    int hmin = INT_MAX, hmax = INT_MIN, xmin = INT_MAX, xmax = INT_MIN;
+    unsigned int ev = 0u;
 #pragma unroll
-        for (int w = 0; w < W; ++w) xo[w] = __shfl_sync(0xffffffffu, x[w], o);
-        // the lane's bonds b0 .. b0 + BPL - 1 (those below L): segments from one window
-        const int b0 = lane * BPL;
-        unsigned long long v = 0ull;
-        if (b0 < L) {
-          const int st0 = b0 >= 8 ? b0 - 8 : b0 - 8 + L;
-          const unsigned long long win = ring_window<W>(xo, L, st0);
+    for (int j = 0; j < NW; ++j) u[j] = 0u;
+    for (;;) {
+      const unsigned int m = __ballot_sync(0xffffffffu, cl < 0);
+      if (m != 0u && next < n) {
+        const int idx = next + __popc(m & lt_mask);
+        next += __popc(m);
+        const bool got = cl < 0 && idx < n;
+        if (got) {
+          cl = idx;
+          unsigned long long x[W];
+          load_lat<W>(B.Y, slot0 + idx, x);
+          split32<W>(x, u);
+          put_string(u);
+          uint32_t a[NW], pc[NW];
+          active_bonds32<NW>(u, lm1, a, pc);
+          r = 0;
 #pragma unroll
-          for (int i = 0; i < BPL; ++i)
-            if (b0 + i < L) v += guided_q_at(win, i, qtab);
-        }
-        // a group of eight bonds spans 8 / BPL lanes
+          for (int j = 0; j < NW; ++j) r += (int)pc[j];
+          h = 0;
+          e = 0u;
+          t = a_r = a_h = 0.0f;
+          if (carry) {
+            const ulonglong2* src = reinterpret_cast<const ulonglong2*>(gin + (d.off + (int64_t)B.anc[slot0 + idx]) * ng);
+            R = 0ull;
 #pragma unroll
-        for (int off = 1; off < kGuideGroup / BPL; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane % (kGuideGroup / BPL) == 0) s_g[lane / (kGuideGroup / BPL)][(tid & ~31) + o] = v;
-#pragma unroll
-        for (int off = kGuideGroup / BPL; off < 32; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == o) R = v;
-      }
-      __syncwarp();
-    }
-    if (__ballot_sync(0xffffffffu, cl >= 0) == 0u) {
-      if (lane == 0) taken = *(volatile int*)&s_take;
-      if (__shfl_sync(0xffffffffu, taken, 0) >= n) break;
-      continue;
-    }
-    if (cl >= 0) {
-      const uint32_t j = (uint32_t)(base - d.off + cl);
-      const float Rf = u64_to_float_rn(R);
-      const float rp = __fmul_rn(Rf, 0x1p-40f);
-      const long long D = (long long)(float_to_u64_exact(Rf) - R);
-      const float eta = __fdiv_rn(i64_to_float_rn(D), Rf);
-      const float dr = __fsub_rn(__int2float_rn(r), rp);
-      const uint4 w = philox4x32_10(make_uint4(e, beta, j, kTagGuided), k0, k1);
-      const float E = neg_ln_u(w.x, s_log);
-      const float tau = __fdiv_rn(E, rp);
-      const float t_new = __fadd_rn(t, tau);
-      bool run = r != 0;
-      if (run && e >= kStepLimit) {  // guard: an interval must end; report, never spin
-        B.st[p].err = kErrRange;
-        run = false;
-      }
-      if (run && t_new >= dt_f) {
-        a_r = __fmaf_rn(dr, __fsub_rn(dt_f, t), a_r);
-        run = false;
-      }
-      if (run) {
-        a_r = __fmaf_rn(dr, tau, a_r);
-        t = t_new;
-        const unsigned long long kk = __umul64hi(((unsigned long long)w.z << 32) | w.y, R);
-        // the first bond whose inclusive cumulative rate exceeds kk < R: the group from the
-        // group sums, then the bond inside it (the last group if the sums run out first)
-        unsigned long long cum = 0ull;
-        int g = ng - 1;
-        bool found = false;
-#pragma unroll
-        for (int gg = 0; gg < ng - 1; ++gg) {
-          const unsigned long long v = s_g[gg][tid];
-          if (!found) {
-            if (cum + v <= kk) cum += v;
-            else { found = true; g = gg; }
-          }
-        }
-        const int gb = g * kGuideGroup;  // < L: the group holds the bond kk falls on
-        const unsigned long long gwin = ring_window<W>(x, L, gb >= 8 ? gb - 8 : gb - 8 + L);
-        int b = gb + kGuideGroup - 1;
-        uint32_t bseg = 0u;
-        found = false;
-#pragma unroll
-        for (int i = 0; i < kGuideGroup; ++i) {
-          const unsigned long long q = gb + i < L ? guided_q_at(gwin, i, qtab) : 0ull;
-          if (!found) {
-            cum += q;
-            if (cum > kk) {
-              found = true;
-              b = gb + i;
-              bseg = (uint32_t)(gwin >> i) & 0x3FFFFu;
+            for (int g = 0; g < ng / 2; ++g) {
+              const ulonglong2 v = src[g];
+              s_g[2 * g][tid] = v.x;
+              s_g[2 * g + 1][tid] = v.y;
+              R += v.x + v.y;
             }
           }
         }
-        const int kb = min(max(__ldg(dtab + guided_index(bseg)) - d.s_q, -kGuideKmax), kGuideKmax);
-        a_h = __fadd_rn(a_h, __fsub_rn(__fsub_rn(d.c_s, __fmul_rn(__int2float_rn(kb + d.s_q), 0x1p-17f)), eta));
-        // the bonds b-9 .. b+9, whose windows contain site b or b+1, change rate: their
-        // segments (sites b-17 .. b+18) from one window before and one after the hop
-        const int ws = b >= 17 ? b - 17 : b - 17 + L;
-        const unsigned long long wo = ring_window<W>(x, L, ws);
-        hop<W>(x, b, L);
-        ++h;
-        active_bonds<W>(x, L, a);
-        r = popc_lat<W>(a);
-        const unsigned long long wn = ring_window<W>(x, L, ws);
+        // the rate sums of every new clone without carried ones, one clone at a time by
+        // the whole warp, a group per lane
+        unsigned int todo = __ballot_sync(0xffffffffu, got && !carry);
+        __syncwarp();  // the strings are read by other lanes
+        while (todo != 0u) {
+          const int o = __ffs(todo) - 1;
+          todo &= todo - 1u;
+          unsigned long long v = 0ull;
+          if (lane < ng) {
+            const uint32_t win = window(lane, (tid & ~31) + o);
+            v = guided_group(win, active(win, lane), qtab);
+            s_g[lane][(tid & ~31) + o] = v;
+          }
+          v = warp_sum_u64(v);
+          if (lane == o) R = v;
+        }
+        __syncwarp();
+      } else if (m == 0xffffffffu) {
+        break;  // every lane is empty and the segment has run out
+      }
+      if (cl >= 0) {
+        const uint32_t j = (uint32_t)(j0 + cl);
+        const float Rf = u64_to_float_rn(R);
+        const float rp = __fmul_rn(Rf, 0x1p-40f);
+        const long long D = (long long)(float_to_u64_exact(Rf) - R);
+        const float eta = __fdiv_rn(i64_to_float_rn(D), Rf);
+        const float dr = __fsub_rn(__int2float_rn(r), rp);
+        const uint4 w = philox4x32_10_rk(make_uint4(e, beta, j, kTagGuided), s_key[wid]);
+        const float E = neg_ln_u(w.x, s_log);
+        const float tau = __fdiv_rn(E, rp);
+        const float t_new = __fadd_rn(t, tau);
+        bool run = r != 0;
+        if (run && e >= kStepLimit) {  // guard: an interval must end; report, never spin
+          B.st[p].err = kErrRange;
+          run = false;
+        }
+        if (run && t_new >= dt_f) {
+          a_r = __fmaf_rn(dr, __fsub_rn(dt_f, t), a_r);
+          run = false;
+        }
+        if (run) {
+          a_r = __fmaf_rn(dr, tau, a_r);
+          t = t_new;
+          const unsigned long long kk = __umul64hi(((unsigned long long)w.z << 32) | w.y, R);
+          // the first bond whose inclusive cumulative rate exceeds kk < R: the group from the
+          // group sums, then the bond inside it (the last group if the sums run out first)
+          unsigned long long cum = 0ull;
+          int g = 0;
+          bool on = true;
 #pragma unroll
-        for (int db = -9; db <= 9; ++db) {
-          if (db == 9 && L <= 18) continue;  // on 18 sites bond b+9 is bond b-9
-          int c = b + db;
-          if (c < 0) c += L;
-          if (c >= L) c -= L;
-          const unsigned long long qo = guided_q_at(wo, db + 9, qtab);
-          const unsigned long long qn = guided_q_at(wn, db + 9, qtab);
-          if (qn != qo) {
-            s_g[c / kGuideGroup][tid] += qn - qo;
-            R += qn - qo;
+          for (int gg = 0; gg < ng - 1; ++gg) {
+            const unsigned long long c = cum + s_g[gg][tid];
+            on = on && c <= kk;
+            cum = on ? c : cum;
+            g += on ? 1 : 0;
+          }
+          const uint32_t gw = window(g, tid);
+          const uint32_t am = active(gw, g);
+          unsigned long long q[kGuideGroup];
+#pragma unroll
+          for (int i = 0; i < kGuideGroup; ++i) {
+            q[i] = 0ull;
+            if ((am >> i) & 1u) q[i] = __ldg(qtab + guided_index(gw, i));
+          }
+          int i_b = 0;
+          on = true;
+#pragma unroll
+          for (int i = 0; i < kGuideGroup - 1; ++i) {
+            cum += q[i];
+            on = on && cum <= kk;
+            i_b += on ? 1 : 0;
+          }
+          const int b = kGuideGroup * g + i_b;
+          const int kb = min(max(__ldg(dtab + guided_index(gw, i_b)) - d.s_q, -kGuideKmax), kGuideKmax);
+          a_h = __fadd_rn(a_h, __fsub_rn(__fsub_rn(d.c_s, __fmul_rn(__int2float_rn(kb + d.s_q), 0x1p-17f)), eta));
+          hop32<NW>(u, (uint32_t)b, lm1);
+          ++h;
+          put_string(u);
+          uint32_t a[NW], pc[NW];
+          active_bonds32<NW>(u, lm1, a, pc);
+          r = 0;
+#pragma unroll
+          for (int j2 = 0; j2 < NW; ++j2) r += (int)pc[j2];
+          // the groups of the bonds b-9 .. b+9 round the ring, summed anew (a group met
+          // twice on a short ring adds nothing the second time)
+          int c = b >= 9 ? b - 9 : b - 9 + L;
+          for (int left = 19; left > 0;) {
+            const int gg = c >> 3;
+            const uint32_t win = window(gg, tid);
+            const unsigned long long v = guided_group(win, active(win, gg), qtab);
+            R += v - s_g[gg][tid];
+            s_g[gg][tid] = v;
+            const int end = min(kGuideGroup * (gg + 1), L);
+            left -= end - c;
+            c = end == L ? 0 : end;
           }
         }
-      }
-      ++e;
-      if (!run) {
-        const float X = __fsub_rn(a_h, a_r);
-        const int64_t slot = base + cl;
+        ++e;
+        if (!run) {
+          const float X = __fsub_rn(a_h, a_r);
+          const int64_t slot = slot0 + cl;
+          ulonglong2* dst = reinterpret_cast<ulonglong2*>(gout + slot * ng);
 #pragma unroll
-        for (int g = 0; g < ng; ++g) gout[slot * ng + g] = s_g[g][tid];
-        store_lat<W>(B.Xb[par], slot, x);
-        B.KXb[par][slot] = B.KY[slot] + h;
-        B.dKb[par][slot] = h;
-        B.Ab[par][slot] = X;
-        hmin = min(hmin, h);
-        hmax = max(hmax, h);
-        ev += (unsigned int)h;
-        xmin = min(xmin, float_order(X));
-        xmax = max(xmax, float_order(X));
-        cl = -1;
+          for (int g = 0; g < ng / 2; ++g) dst[g] = make_ulonglong2(s_g[2 * g][tid], s_g[2 * g + 1][tid]);
+          unsigned long long x[W];
+          join32<W>(u, x);
+          store_lat<W>(B.Xb[par], slot, x);
+          B.KXb[par][slot] = B.KY[slot] + h;
+          B.dKb[par][slot] = h;
+          B.Ab[par][slot] = X;
+          hmin = min(hmin, h);
+          hmax = max(hmax, h);
+          ev += (unsigned int)h;
+          xmin = min(xmin, float_order(X));
+          xmax = max(xmax, float_order(X));
+          cl = -1;
+        }
       }
+      __syncwarp();
     }
-  }
-  hmin = __reduce_min_sync(0xffffffffu, hmin);
-  hmax = __reduce_max_sync(0xffffffffu, hmax);
-  ev = __reduce_add_sync(0xffffffffu, ev);
-  xmin = __reduce_min_sync(0xffffffffu, xmin);
-  xmax = __reduce_max_sync(0xffffffffu, xmax);
-  if (lane == 0 && hmin != INT_MAX) {
-    atomicMin(&s_min, hmin);
-    atomicMax(&s_max, hmax);
-    atomicAdd(&s_ev, ev);
-    atomicMin(&s_amin, xmin);
-    atomicMax(&s_amax, xmax);
-  }
-  __syncthreads();
-  if (tid == 0 && s_min != INT_MAX) {
-    PopState* st = B.st + p;
-    atomicMin(&st->dk_min[par], s_min);
-    atomicMax(&st->dk_max[par], s_max);
-    atomicAdd(&st->events, (unsigned long long)s_ev);
-    atomicMin(&st->a_min[par], s_amin);
-    atomicMax(&st->a_max[par], s_amax);
+    hmin = __reduce_min_sync(0xffffffffu, hmin);
+    hmax = __reduce_max_sync(0xffffffffu, hmax);
+    ev = __reduce_add_sync(0xffffffffu, ev);
+    xmin = __reduce_min_sync(0xffffffffu, xmin);
+    xmax = __reduce_max_sync(0xffffffffu, xmax);
+    if (lane == 0 && n > 0) {
+      PopState* st = B.st + p;
+      atomicMin(&st->dk_min[par], hmin);
+      atomicMax(&st->dk_max[par], hmax);
+      atomicAdd(&st->events, (unsigned long long)ev);
+      atomicMin(&st->a_min[par], xmin);
+      atomicMax(&st->a_max[par], xmax);
+    }
+    __syncwarp();
+    slot0 = seg_end;
   }
 }
 
