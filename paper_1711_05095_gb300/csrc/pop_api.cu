@@ -343,7 +343,7 @@ void kernel_end(pop_t* h, cudaStream_t st) {
 }
 
 // The dynamical stage's kernel for a batch: words per lane and lanes per clone by the
-// largest ring, the form for rings that fill one or two 64-bit words where every one does.
+// largest ring.
 typedef void (*EvolveKernel)(Batch, float);
 
 int evolve_lanes(const pop_t* h) {
@@ -352,10 +352,16 @@ int evolve_lanes(const pop_t* h) {
   return g;
 }
 
+// Whether every ring of the populations [pop0, pop1) fills the batch's lattice words.
+bool full_rings(const pop_t* h, int pop0, int pop1) {
+  bool full = true;
+  for (int p = pop0; p < pop1; ++p) full = full && h->desc[p].L == 64 * h->lay.W;
+  return full;
+}
+
 template <bool MOD>
 EvolveKernel evolve_kernel_of(const pop_t* h) {
-  bool full = true;
-  for (const PopDesc& d : h->desc) full = full && d.L == 64 * h->lay.W;
+  const bool full = full_rings(h, 0, h->lay.P);
   if (h->lay.W == 1) return full ? k_evolve<2, 1, MOD, true> : k_evolve<2, 1, MOD, false>;
   if (h->lay.W == 2) return full ? k_evolve<4, 1, MOD, true> : k_evolve<4, 1, MOD, false>;
   switch (evolve_lanes(h)) {
@@ -450,7 +456,6 @@ void launch_fused_form(pop_t* h, unsigned grid, cudaStream_t st, const Batch& Bx
     k_gather<W, 128, true, MOD, SCAN, 1, FULL><<<grid, 128, 0, st>>>(Bx, dt_f, tile0);
 }
 
-// full: every population of the launch has L = 64 W (the ring fills the lattice words)
 template <int W, bool MOD, bool SCAN>
 void launch_fused(pop_t* h, unsigned grid, cudaStream_t st, const Batch& Bx, float dt_f, int tile0, bool full) {
   if (full) launch_fused_form<W, MOD, SCAN, true>(h, grid, st, Bx, dt_f, tile0);
@@ -481,8 +486,7 @@ int launch_resample_evolve_range(pop_t* h, cudaStream_t st, float dt_f, const Ba
     for (int p = pop0; p < pop1; ++p) scan = scan && h->desc[p].ntiles > kScanTiles;
     if (scan) launch_tile_scan(h, st, Bx, pop0, pop1);
   }
-  bool full = true;
-  for (int p = pop0; p < pop1; ++p) full = full && h->desc[p].L == 64 * h->lay.W;
+  const bool full = full_rings(h, pop0, pop1);
   kernel_begin(h, st, POP_K_GATHER_EVOLVE);
   if (h->lay.W == 1) {
     if (h->any_mod) {

@@ -311,23 +311,40 @@ __device__ __forceinline__ void join32(const uint32_t (&u)[2 * W], unsigned long
   for (int w = 0; w < W; ++w) x[w] = ((unsigned long long)u[2 * w + 1] << 32) | u[2 * w];
 }
 
-// a = x XOR rot(x) on 2W words; lm1 = L - 1 (site L-1's right neighbour is site 0).
-// p[j] = popc(a[j]).  FULL: L = 32 NW, the ring fills the words, and rot is a
-// rotation of the words' concatenation by one bit.
-template <int NW, bool FULL = false>
-__device__ __forceinline__ void active_bonds32(const uint32_t (&u)[NW], uint32_t lm1, uint32_t (&a)[NW],
-                                               uint32_t (&p)[NW]) {
-  const uint32_t c0 = u[0] & 1u;
+// Padding.  A ring shorter than its words keeps a copy of site 0 in every bit at or above
+// L while it is in registers: then a = x XOR rot(x) is a plain rotation of the words'
+// concatenation by one bit for every L (bit L - 1 meets site 0 in bit L, the padding and
+// the wrap-around bit cancel), with no closing bond to place.  In memory the padding is 0.
+template <int NW>
+struct __align__(8 * (NW / 2)) LatWords {
+  uint32_t w[NW];
+};
+
+template <int NW>
+__device__ __forceinline__ LatWords<NW> pad_mask(uint32_t L) {
+  LatWords<NW> m;
+#pragma unroll
+  for (int j = 0; j < NW; ++j) m.w[j] = L >= 32u * (j + 1) ? 0u : (L <= 32u * j ? 0xffffffffu : 0xffffffffu << (L & 31u));
+  return m;
+}
+template <int NW>
+__device__ __forceinline__ void pad_fill(uint32_t (&u)[NW], const LatWords<NW>& pad) {
+  const uint32_t s0 = 0u - (u[0] & 1u);
+#pragma unroll
+  for (int j = 0; j < NW; ++j) u[j] |= s0 & pad.w[j];
+}
+template <int NW>
+__device__ __forceinline__ void pad_clear(uint32_t (&u)[NW], const LatWords<NW>& pad) {
+#pragma unroll
+  for (int j = 0; j < NW; ++j) u[j] &= ~pad.w[j];
+}
+
+// Active bonds of a padded lattice; p[j] = popc(a[j]).
+template <int NW>
+__device__ __forceinline__ void active_bonds32(const uint32_t (&u)[NW], uint32_t (&a)[NW], uint32_t (&p)[NW]) {
 #pragma unroll
   for (int j = 0; j < NW; ++j) {
-    uint32_t rot;
-    if constexpr (FULL) {
-      rot = __funnelshift_r(u[j], u[(j + 1) % NW], 1);
-    } else {
-      const uint32_t nxt = (j + 1 < NW) ? u[j + 1] : 0u;
-      rot = __funnelshift_r(u[j], nxt, 1) | __funnelshift_lc(0u, c0, lm1 - 32u * (uint32_t)j);
-    }
-    a[j] = u[j] ^ rot;
+    a[j] = u[j] ^ __funnelshift_r(u[j], u[(j + 1) % NW], 1);
     p[j] = (uint32_t)__popc(a[j]);
   }
 }
@@ -363,14 +380,58 @@ __device__ __forceinline__ uint32_t kth_bond32(const uint32_t (&a)[NW], const ui
   return pos + kth8[((w & 0xffu) << 3) | (k & 7u)];
 }
 
-// A hop across bond b flips sites b and c = (b + 1) mod L (lm1 = L - 1); b >= 32 NW
-// (with b != lm1) flips nothing, which is the predicated step's "no hop".
+// Escape rate (active bonds) of a lattice whose padding is 0.
+template <int NW>
+__device__ __forceinline__ int escape_rate(const uint32_t (&u)[NW], const LatWords<NW>& pad) {
+  uint32_t v[NW], a[NW], p[NW], r = 0u;
+#pragma unroll
+  for (int j = 0; j < NW; ++j) v[j] = u[j];
+  pad_fill<NW>(v, pad);
+  active_bonds32<NW>(v, a, p);
+#pragma unroll
+  for (int j = 0; j < NW; ++j) r += p[j];
+  return (int)r;
+}
+
+// A hop across bond b < L flips sites b and c = (b + 1) mod L (lm1 = L - 1; the padding,
+// if any, stays as it is): one-hot masks by clamped shifts.
 template <int NW>
 __device__ __forceinline__ void hop32(uint32_t (&u)[NW], uint32_t b, uint32_t lm1) {
   const uint32_t c = (b == lm1) ? 0u : b + 1u;
 #pragma unroll
   for (int j = 0; j < NW; ++j)
     u[j] ^= __funnelshift_lc(0u, 1u, b - 32u * (uint32_t)j) ^ __funnelshift_lc(0u, 1u, c - 32u * (uint32_t)j);
+}
+
+// A hop across bond b flips sites b and (b + 1) mod L, and the padding when one of them is
+// site 0: entry b < L of a table in shared memory; entry kNoHop flips nothing.  One load
+// and NW exclusive ors, where two one-hot masks made by shifts were 20 instructions on two
+// words (four 32-bit ones), all on the ALU pipe, the one that bounds the dynamical stage
+// (60 % busy, with the shared-memory pipe at 29 %).
+constexpr uint32_t kNoHop = kMaxL;
+constexpr int kPadEntry = kMaxL + 1, kHopEntries = kMaxL + 2;  // the last one: the padding mask
+template <int NW>
+__device__ __forceinline__ void build_hop_table(LatWords<NW>* tab, uint32_t L, int first, int stride) {
+  const LatWords<NW> pad = pad_mask<NW>(L);
+  if (first == 0) tab[kPadEntry] = pad;
+  for (int b = first; b <= kMaxL; b += stride) {
+    const uint32_t b0 = (uint32_t)b, b1 = b0 + 1u == L ? 0u : b0 + 1u;
+    LatWords<NW> e;
+#pragma unroll
+    for (int j = 0; j < NW; ++j) {
+      // (shifts by 32 or more, "negative" ones too, give 0)
+      const uint32_t m = __funnelshift_lc(0u, 1u, b0 - 32u * (uint32_t)j) ^ __funnelshift_lc(0u, 1u, b1 - 32u * (uint32_t)j) ^
+                         (b0 == 0u || b1 == 0u ? pad.w[j] : 0u);
+      e.w[j] = b0 < L && b < kMaxL ? m : 0u;
+    }
+    tab[b] = e;
+  }
+}
+template <int NW>
+__device__ __forceinline__ void hop_by_table(uint32_t (&u)[NW], uint32_t b, const LatWords<NW>* tab) {
+  const LatWords<NW> e = tab[b];
+#pragma unroll
+  for (int j = 0; j < NW; ++j) u[j] ^= e.w[j];
 }
 
 // kth8 as 512 words (4 table bytes per word, little-endian), built at compile time.

@@ -64,8 +64,8 @@ __global__ void __launch_bounds__(kThreads) k_init(Batch B) {
 }
 
 // One BKL step (Sec. 4 BKL; Sec. 3.1 rates 1 per possible hop) with the step's
-// exponential variate E = -ln u(wa) and bond word wb, on the lattice as 2W 32-bit
-// words u (lm1 = L - 1): r = active bonds (escape rate; r = 0 ends the interval);
+// exponential variate E = -ln u(wa) and bond word wb, on the padded lattice as 2W
+// 32-bit words u: r = active bonds (escape rate; r = 0 ends the interval);
 // tau = E * float(1/r); t_new = t + tau; t_new >= dt ends the interval (the residual
 // waiting time is dropped, as the exponential law's memorylessness allows);
 // otherwise hop across the floor(wb r / 2^32)-th active bond (kth8: the byte table of
@@ -77,15 +77,15 @@ __global__ void __launch_bounds__(kThreads) k_init(Batch B) {
 // time and bond are computed in any case and applied under the step's predicate, so the
 // lanes of a warp stay together.  inv[0] is NaN, so the comparison fails for r = 0 (MOD:
 // the last segment r (dt - t) is added; for r = 0 it adds nothing).  A step that does not
-// hop passes bond 1024, which hop32 turns into no change.  FULL: L = 64 W (see
-// active_bonds32).
-template <int W, bool MOD, bool FULL = false>
-__device__ __forceinline__ bool bkl_step_pred(uint32_t (&u)[2 * W], float& t, float& acc, uint32_t lm1,
-                                              const float* inv, float E, uint32_t wb, float dt_f,
-                                              bool live, const uint8_t* kth8) {
+// hop passes kNoHop, which changes nothing.
+// t is advanced in any case: after a step that did not hop it is not used again.
+template <int W, bool MOD>
+__device__ __forceinline__ bool bkl_step_pred(uint32_t (&u)[2 * W], float& t, float& acc, const float* inv, float E,
+                                              uint32_t wb, float dt_f, bool live, const uint8_t* kth8,
+                                              const LatWords<2 * W>* hops) {
   constexpr int NW = 2 * W;
   uint32_t a[NW], pc[NW];
-  active_bonds32<NW, FULL>(u, lm1, a, pc);
+  active_bonds32<NW>(u, a, pc);
   uint32_t r = 0u;
 #pragma unroll
   for (int j = 0; j < NW; ++j) r += pc[j];
@@ -96,9 +96,9 @@ __device__ __forceinline__ bool bkl_step_pred(uint32_t (&u)[2 * W], float& t, fl
     const float seg = hopped ? tau : __fsub_rn(dt_f, t);
     acc = live ? __fmaf_rn((float)r, seg, acc) : acc;
   }
-  t = hopped ? t_new : t;
+  t = t_new;
   const uint32_t b = kth_bond32<NW>(a, pc, __umulhi(wb, r), kth8);
-  hop32<NW>(u, hopped ? b : 1024u, lm1);
+  hop_by_table<NW>(u, hopped ? b : kNoHop, hops);
   return hopped;
 }
 
@@ -210,6 +210,7 @@ __device__ __forceinline__ bool wide_step_pred(uint32_t (&u)[8], float& t, float
   return hopped;
 }
 
+// FULL: every ring fills the words (L = 32 NW), so there is no padding to keep.
 template <int NW, int G, bool MOD, bool FULL>
 __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_BLOCKS) k_evolve(Batch B, float dt_f) {
   static_assert(NW == 8 || G == 1, "one lane for up to four words");
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
   __shared__ __align__(16) uint32_t s_kth8[512];
   __shared__ uint2 s_key[kEvolveWarps][10];          // the Philox key schedule of the warp's population
   __shared__ float s_inv[kEvolveWarps][NW == 8 ? 1 : kMaxL + 1];  // and its waiting-time factors
+  __shared__ LatWords<NW == 8 ? 2 : NW> s_hop[kEvolveWarps][NW == 8 ? 1 : kHopEntries];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (tid < 64) s_tab[tid] = B.logtab[tid];
   reinterpret_cast<uint4*>(s_kth8)[tid] = reinterpret_cast<const uint4*>(g_kth8.w)[tid];
@@ -250,6 +252,7 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
       for (int r = lane; r <= kMaxL; r += 32)  // inv[0] = NaN: see bkl_step_pred
         s_inv[wid][r] = r == 0 ? __int_as_float(0x7fffffff) : (r <= d.L) ? inv[r] : 0.0f;
       inv = s_inv[wid];
+      build_hop_table<NW>(s_hop[wid], (uint32_t)d.L, lane, 32);
     }
     __syncwarp();
     const uint32_t lm1 = (uint32_t)d.L - 1u;
@@ -272,6 +275,7 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
             unsigned long long x[W64];
             load_lat<W64>(B.Y, slot0 + idx, x);
             split32<W64>(x, u);
+            if (!FULL) pad_fill<NW>(u, s_hop[wid][kPadEntry]);
           } else {
             const unsigned long long* src = B.Y + (slot0 + idx) * W + W64 * sub;
 #pragma unroll
@@ -296,8 +300,8 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
       const float E1 = neg_ln_u(d4.x, s_tab), E2 = neg_ln_u(d4.z, s_tab);
       bool h1, h2;
       if constexpr (NW < 8) {
-        h1 = bkl_step_pred<W64, MOD, FULL>(u, t, acc, lm1, inv, E1, d4.y, dt_f, live, kth8);
-        h2 = bkl_step_pred<W64, MOD, FULL>(u, t, acc, lm1, inv, E2, d4.w, dt_f, h1, kth8);
+        h1 = bkl_step_pred<W64, MOD>(u, t, acc, inv, E1, d4.y, dt_f, live, kth8, s_hop[wid]);
+        h2 = bkl_step_pred<W64, MOD>(u, t, acc, inv, E2, d4.w, dt_f, h1, kth8, s_hop[wid]);
       } else {
         h1 = wide_step_pred<G, MOD>(u, t, acc, lm1, inv, E1, d4.y, dt_f, live, kth8, sub, lead);
         h2 = wide_step_pred<G, MOD>(u, t, acc, lm1, inv, E2, d4.w, dt_f, h1, kth8, sub, lead);
@@ -313,6 +317,7 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
         const int64_t slot = slot0 + cl;
         if constexpr (NW < 8) {
           unsigned long long x[W64];
+          if (!FULL) pad_clear<NW>(u, s_hop[wid][kPadEntry]);
           join32<W64>(u, x);
           store_lat<W64>(B.Xb[par], slot, x);
         } else {
@@ -582,8 +587,8 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_scan(Batch B, int pop0) {
 // the extra path costs registers and scheduling when compiled into the same kernel).
 // NCL (FUSE only): clones each lane advances together in the dynamical stage, 1 or 2
 // (two independent Philox and bit-select chains in flight per lane).
-// FULL (FUSE only): every population of the launch has L = 64 W, so the ring fills
-// the lattice words (active_bonds32<.., true>).
+// FULL (FUSE only): every ring of the launch fills the words (L = 64 W), so there is no
+// padding to keep (L = 128 batch: 297 us per interval, 307 us with it kept).
 template <int W, int NT, bool FUSE = false, bool MOD = false, bool SCAN = true, int NCL = 1, bool FULL = false>
 __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 128 / NT : POP_FUSE2_MIN_BLOCKS)
                                            : (NT == 128 ? 11 : (NT == 256 ? 6 : 3)))
@@ -618,6 +623,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
   constexpr int kUStage = 64;
   __shared__ unsigned long long s_u[kUStage];
   __shared__ __align__(16) uint32_t s_kth8[FUSE ? 512 : 1];
+  __shared__ LatWords<2 * WS> s_hop[FUSE ? kHopEntries : 1];
   // FUSE, plain weights: activity histograms of the first three tiles the new clones
   // fall in (the rest go straight to global memory)
   __shared__ unsigned int s_th[(FUSE && !MOD) ? 3 * kTH : 1];
@@ -646,6 +652,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
       s_inv[r] = r == 0 ? __int_as_float(0x7fffffff) : (r <= d.L) ? src[r] : 0.0f;
     if (tid < 64) s_logtab[tid] = B.logtab[tid];
     if (tid < 128) reinterpret_cast<uint4*>(s_kth8)[tid] = reinterpret_cast<const uint4*>(g_kth8.w)[tid];
+    build_hop_table<2 * WS>(s_hop, (uint32_t)d.L, tid, NT);
     if constexpr (!MOD)
       for (int e = tid; e < 3 * kTH; e += NT) s_th[e] = 0u;
     if (tid < 10)
@@ -867,14 +874,16 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     int32_t* const dKn = B.dKb[pn];
     float* const An = B.Ab[pn];
     const int n = (int)(J1 - J0);
-    const int L = d.L;
+    // the padding mask: in registers for one word, from shared memory for two (registers
+    // are short there: 2 % of the L = 128 batch's time)
+    const LatWords<2 * W> pad1 = pad_mask<2 * W>((uint32_t)d.L);
     // the tile of the new slot J0 (tiles of the next interval: 1024 slots, populations
     // tile-aligned), and whether an activity fell outside the histograms
     const int t0 = (int)((d.off + (int64_t)J0) >> 10);
     const bool hist_on = !MOD && B.hist_on != 0;
     bool ovf = false;
     const unsigned int lt_mask = (1u << lane) - 1u;
-    int cl[NCL], h[NCL];              // the slot's new clone (offset from J0, -1: empty)
+    int cl[NCL];                      // the slot's new clone (offset from J0, -1: empty)
     int kold[NCL];                    // its ancestor's cumulative activity
     uint32_t q[NCL];
     float t[NCL], acc[NCL];
@@ -885,7 +894,6 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     for (int k = 0; k < NCL; ++k) {
       cl[k] = -1;
       kold[k] = 0;
-      h[k] = 0;
       q[k] = 0u;
       t[k] = 0.0f;
       acc[k] = 0.0f;
@@ -894,7 +902,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     }
     // one iteration of the lane's clones: a Philox draw each, two predicated BKL steps,
     // and the write-back of a clone whose interval ended
-    auto iterate = [&]() {
+    auto iterate = [&](bool check) {
       uint4 d4[NCL];
       float E1[NCL], E2[NCL];
 #pragma unroll
@@ -911,31 +919,33 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
         uint32_t u[2 * W];
         split32<W>(x[k], u);
         const uint8_t* kth8 = reinterpret_cast<const uint8_t*>(s_kth8);
-        const bool h1 = bkl_step_pred<W, MOD, FULL>(u, t[k], acc[k], (uint32_t)L - 1u, s_inv, E1[k], d4[k].y,
-                                                    dt_f, live, kth8);
-        const bool h2 = bkl_step_pred<W, MOD, FULL>(u, t[k], acc[k], (uint32_t)L - 1u, s_inv, E2[k], d4[k].w,
-                                                    dt_f, h1, kth8);
+        const bool h1 = bkl_step_pred<W, MOD>(u, t[k], acc[k], s_inv, E1[k], d4[k].y, dt_f, live, kth8, s_hop);
+        const bool h2 = bkl_step_pred<W, MOD>(u, t[k], acc[k], s_inv, E2[k], d4[k].w, dt_f, h1, kth8, s_hop);
         join32<W>(u, x[k]);
-        h[k] += (int)h1 + (int)h2;
         ++q[k];
         bool run = h2;
-        if (run && q[k] >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
+        if (check && run && q[k] >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
           st->err = kErrRange;
           run = false;
         }
         if (live && !run) {
           const int64_t dst = d.off + (int64_t)J0 + cl[k];
-          store_lat<W>(Xn, dst, x[k]);
-          KXn[dst] = kold[k] + h[k];
-          dKn[dst] = h[k];
+          // every earlier draw of the clone made two hops
+          const int hops = 2 * (int)q[k] - 2 + (int)h1 + (int)h2;
+          if (!FULL) pad_clear<2 * W>(u, W == 1 ? pad1 : s_hop[kPadEntry]);
+          unsigned long long xo[W];
+          join32<W>(u, xo);
+          store_lat<W>(Xn, dst, xo);
+          KXn[dst] = kold[k] + hops;
+          dKn[dst] = hops;
           if (MOD) {
             An[dst] = acc[k];
             amin = min(amin, __float_as_int(acc[k]));  // A >= 0: float bits order like values
             amax = max(amax, __float_as_int(acc[k]));
           }
-          hmin = min(hmin, h[k]);
-          hmax = max(hmax, h[k]);
-          ev += (unsigned int)h[k];
+          hmin = min(hmin, hops);
+          hmax = max(hmax, hops);
+          ev += (unsigned int)hops;
           cl[k] = -1;
         }
       }
@@ -947,6 +957,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     const int share = n / NWARP, extra = n - share * NWARP;
     int next = wid * share + min(wid, extra);
     const int last = next + share + (wid < extra ? 1 : 0);
+    uint32_t iters = 0u;
     for (;;) {
       unsigned int m[NCL];
       int tot = 0;
@@ -966,15 +977,20 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
             kold[k] = KXo[base + sk];
 #pragma unroll
             for (int w = 0; w < W; ++w) x[k][w] = s_x[sk][w];
+            if constexpr (!FULL) {
+              uint32_t u[2 * W];
+              split32<W>(x[k], u);
+              pad_fill<2 * W>(u, W == 1 ? pad1 : s_hop[kPadEntry]);
+              join32<W>(u, x[k]);
+            }
             t[k] = 0.0f;
             acc[k] = 0.0f;
-            h[k] = 0;
             q[k] = 0u;
           }
           next += __popc(m[k]);
         }
       }
-      iterate();
+      iterate(++iters >= kStepLimit / 2u);  // no clone of the warp has made more draws
     }
     // The shares have run out.  Each round packs the block's remaining clones into the
     // lowest threads (through the staging buffer of the old clones, no longer read),
@@ -982,7 +998,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     struct Packed {
       unsigned long long x[W];
       float t, acc;
-      int cl, h, kold;
+      int cl, kold;
       uint32_t q;
     };
     static_assert(sizeof(Packed) * NT * NCL <= sizeof(s_x), "the packed clones fit the staging buffer");
@@ -999,7 +1015,6 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
           e.t = t[k];
           e.acc = acc[k];
           e.cl = cl[k];
-          e.h = h[k];
           e.kold = kold[k];
           e.q = q[k];
         }
@@ -1020,13 +1035,12 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
           t[k] = e.t;
           acc[k] = e.acc;
           cl[k] = e.cl;
-          h[k] = e.h;
           kold[k] = e.kold;
           q[k] = e.q;
           any = true;
         }
       }
-      if (__ballot_sync(0xffffffffu, any) != 0u) iterate();
+      if (__ballot_sync(0xffffffffu, any) != 0u) iterate(true);
     }
     hmin = __reduce_min_sync(0xffffffffu, hmin);
     hmax = __reduce_max_sync(0xffffffffu, hmax);
@@ -1177,6 +1191,7 @@ struct SmallSmem {
   int32_t pend_k[32];
   float2 logtab[64];
   __align__(16) uint32_t kth8[512];
+  LatWords<2 * W> hop[kHopEntries];
   uint2 keys[10];
   float inv[kMaxL + 1];
   unsigned int hist[kHistSmem];
@@ -1198,6 +1213,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
   const unsigned long long* const wt = B.wtab + (size_t)p * kKcap;
   for (int r = tid; r <= kMaxL; r += (int)blockDim.x)  // inv[0] = NaN: see bkl_step_pred
     S.inv[r] = r == 0 ? __int_as_float(0x7fffffff) : (r <= d.L) ? B.inv_rate[(size_t)p * kInvStride + r] : 0.0f;
+  build_hop_table<2 * W>(S.hop, (uint32_t)d.L, tid, (int)blockDim.x);
   for (int e = tid; e < 512; e += (int)blockDim.x) S.kth8[e] = g_kth8.w[e];
   for (int e = tid; e < kHistSmem; e += (int)blockDim.x) S.hist[e] = 0u;
   for (int e = tid; e < 64; e += (int)blockDim.x) {
@@ -1219,7 +1235,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
   if (tid == 0) psi = st->psi_acc;
   __syncthreads();
   const uint8_t* const kth8 = reinterpret_cast<const uint8_t*>(S.kth8);
-  const uint32_t lm1 = (uint32_t)d.L - 1u;
   unsigned long long ev = 0ull;
   int cur = 0, h = 0;
   for (int it = 0; it < n_int; ++it) {
@@ -1233,20 +1248,22 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
     for (int w = 0; w < W; ++w) x[w] = S.x[cur][a][w];
     uint32_t u[2 * W];
     split32<W>(x, u);
+    pad_fill<2 * W>(u, S.hop[kPadEntry]);
     float t = 0.0f, acc = 0.0f;
     h = 0;
     bool run = valid;
     for (uint32_t q = 0u; __ballot_sync(0xffffffffu, run) != 0u; ++q) {
       const uint4 d4 = philox4x32_10_rk(make_uint4(q, beta, (uint32_t)tid, kTagEvolve), S.keys);
       const float E1 = neg_ln_u(d4.x, S.logtab), E2 = neg_ln_u(d4.z, S.logtab);
-      const bool h1 = bkl_step_pred<W, MOD>(u, t, acc, lm1, S.inv, E1, d4.y, dt_f, run, kth8);
-      run = bkl_step_pred<W, MOD>(u, t, acc, lm1, S.inv, E2, d4.w, dt_f, h1, kth8);
+      const bool h1 = bkl_step_pred<W, MOD>(u, t, acc, S.inv, E1, d4.y, dt_f, run, kth8, S.hop);
+      run = bkl_step_pred<W, MOD>(u, t, acc, S.inv, E2, d4.w, dt_f, h1, kth8, S.hop);
       h += (int)h1 + (int)run;
       if (q + 1u >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
         if (run) st->err = kErrRange;
         run = false;
       }
     }
+    pad_clear<2 * W>(u, S.hop[kPadEntry]);
     join32<W>(u, x);
     if (valid) {
 #pragma unroll
@@ -1624,6 +1641,7 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
     const int n = (int)max((int64_t)0, min(seg_end - slot0, d.nc - j0));  // warp-uniform
     const int L = d.L;
     const uint32_t lm1 = (uint32_t)L - 1u;
+    const LatWords<NW> pad = pad_mask<NW>((uint32_t)L);
     const unsigned long long* const qtab = B.gq + (size_t)p * kGuideSeg;
     const int32_t* const dtab = B.gdu + (size_t)p * kGuideSeg;
     if (lane < 10)
@@ -1683,11 +1701,7 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
           load_lat<W>(B.Y, slot0 + idx, x);
           split32<W>(x, u);
           put_string(u);
-          uint32_t a[NW], pc[NW];
-          active_bonds32<NW>(u, lm1, a, pc);
-          r = 0;
-#pragma unroll
-          for (int j = 0; j < NW; ++j) r += (int)pc[j];
+          r = escape_rate<NW>(u, pad);
           h = 0;
           e = 0u;
           t = a_r = a_h = 0.0f;
@@ -1781,11 +1795,7 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
           hop32<NW>(u, (uint32_t)b, lm1);
           ++h;
           put_string(u);
-          uint32_t a[NW], pc[NW];
-          active_bonds32<NW>(u, lm1, a, pc);
-          r = 0;
-#pragma unroll
-          for (int j2 = 0; j2 < NW; ++j2) r += (int)pc[j2];
+          r = escape_rate<NW>(u, pad);
           // the groups of the bonds b-9 .. b+9 round the ring, summed anew (a group met
           // twice on a short ring adds nothing the second time)
           int c = b >= 9 ? b - 9 : b - 9 + L;
