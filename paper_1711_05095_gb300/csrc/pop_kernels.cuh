@@ -888,6 +888,10 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     uint32_t q[NCL];
     float t[NCL], acc[NCL];
     unsigned long long x[NCL][W];
+    // the pending draw of clone slot k: its next two steps' waiting-time variates and
+    // bond words
+    float E1[NCL], E2[NCL];
+    uint32_t wb1[NCL], wb2[NCL];
     int hmin = INT_MAX, hmax = INT_MIN, amin = INT_MAX, amax = INT_MIN;
     unsigned int ev = 0u;
 #pragma unroll
@@ -900,54 +904,51 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
 #pragma unroll
       for (int w = 0; w < W; ++w) x[k][w] = 0ull;
     }
-    // one iteration of the lane's clones: a Philox draw each, two predicated BKL steps,
-    // and the write-back of a clone whose interval ended
-    auto iterate = [&](bool check) {
-      uint4 d4[NCL];
-      float E1[NCL], E2[NCL];
-#pragma unroll
-      for (int k = 0; k < NCL; ++k)
-        d4[k] = philox4x32_10_rk(make_uint4(q[k], beta1, J0 + (uint32_t)cl[k], kTagEvolve), s_keys);
-#pragma unroll
-      for (int k = 0; k < NCL; ++k) {
-        E1[k] = neg_ln_u(d4[k].x, s_logtab);
-        E2[k] = neg_ln_u(d4[k].z, s_logtab);
+    auto draw = [&](int k) {
+      const uint4 d4 = philox4x32_10_rk(make_uint4(q[k], beta1, J0 + (uint32_t)cl[k], kTagEvolve), s_keys);
+      E1[k] = neg_ln_u(d4.x, s_logtab);
+      E2[k] = neg_ln_u(d4.z, s_logtab);
+      wb1[k] = d4.y;
+      wb2[k] = d4.w;
+    };
+    // its two predicated BKL steps, and the write-back of a clone whose interval ended
+    const uint8_t* const kth8 = reinterpret_cast<const uint8_t*>(s_kth8);
+    bool hp1[NCL], hp2[NCL];
+    auto steps = [&](int k) {
+      uint32_t u[2 * W];
+      split32<W>(x[k], u);
+      hp1[k] = bkl_step_pred<W, MOD>(u, t[k], acc[k], s_inv, E1[k], wb1[k], dt_f, cl[k] >= 0, kth8, s_hop);
+      hp2[k] = bkl_step_pred<W, MOD>(u, t[k], acc[k], s_inv, E2[k], wb2[k], dt_f, hp1[k], kth8, s_hop);
+      join32<W>(u, x[k]);
+      ++q[k];
+    };
+    auto finish = [&](int k, bool check) {
+      bool run = hp2[k];
+      if (check && run && q[k] >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
+        st->err = kErrRange;
+        run = false;
       }
-#pragma unroll
-      for (int k = 0; k < NCL; ++k) {
-        const bool live = cl[k] >= 0;
+      if (cl[k] >= 0 && !run) {
+        const int64_t dst = d.off + (int64_t)J0 + cl[k];
+        // every earlier draw of the clone made two hops
+        const int hops = 2 * (int)q[k] - 2 + (int)hp1[k] + (int)hp2[k];
         uint32_t u[2 * W];
         split32<W>(x[k], u);
-        const uint8_t* kth8 = reinterpret_cast<const uint8_t*>(s_kth8);
-        const bool h1 = bkl_step_pred<W, MOD>(u, t[k], acc[k], s_inv, E1[k], d4[k].y, dt_f, live, kth8, s_hop);
-        const bool h2 = bkl_step_pred<W, MOD>(u, t[k], acc[k], s_inv, E2[k], d4[k].w, dt_f, h1, kth8, s_hop);
-        join32<W>(u, x[k]);
-        ++q[k];
-        bool run = h2;
-        if (check && run && q[k] >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
-          st->err = kErrRange;
-          run = false;
+        if (!FULL) pad_clear<2 * W>(u, W == 1 ? pad1 : s_hop[kPadEntry]);
+        unsigned long long xo[W];
+        join32<W>(u, xo);
+        store_lat<W>(Xn, dst, xo);
+        KXn[dst] = kold[k] + hops;
+        dKn[dst] = hops;
+        if (MOD) {
+          An[dst] = acc[k];
+          amin = min(amin, __float_as_int(acc[k]));  // A >= 0: float bits order like values
+          amax = max(amax, __float_as_int(acc[k]));
         }
-        if (live && !run) {
-          const int64_t dst = d.off + (int64_t)J0 + cl[k];
-          // every earlier draw of the clone made two hops
-          const int hops = 2 * (int)q[k] - 2 + (int)h1 + (int)h2;
-          if (!FULL) pad_clear<2 * W>(u, W == 1 ? pad1 : s_hop[kPadEntry]);
-          unsigned long long xo[W];
-          join32<W>(u, xo);
-          store_lat<W>(Xn, dst, xo);
-          KXn[dst] = kold[k] + hops;
-          dKn[dst] = hops;
-          if (MOD) {
-            An[dst] = acc[k];
-            amin = min(amin, __float_as_int(acc[k]));  // A >= 0: float bits order like values
-            amax = max(amax, __float_as_int(acc[k]));
-          }
-          hmin = min(hmin, hops);
-          hmax = max(hmax, hops);
-          ev += (unsigned int)hops;
-          cl[k] = -1;
-        }
+        hmin = min(hmin, hops);
+        hmax = max(hmax, hops);
+        ev += (unsigned int)hops;
+        cl[k] = -1;
       }
     };
     // each warp takes new slots from its own even share of the tile's, in order, until
@@ -957,40 +958,48 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     const int share = n / NWARP, extra = n - share * NWARP;
     int next = wid * share + min(wid, extra);
     const int last = next + share + (wid < extra ? 1 : 0);
+    auto take = [&](int k, unsigned int m) {
+      const int idx = next + __popc(m & lt_mask);
+      next += __popc(m);
+      if (cl[k] < 0 && idx < last) {
+        cl[k] = idx;
+        const int sk = source(J0 + (uint32_t)idx);
+        kold[k] = KXo[base + sk];
+#pragma unroll
+        for (int w = 0; w < W; ++w) x[k][w] = s_x[sk][w];
+        if constexpr (!FULL) {
+          uint32_t u[2 * W];
+          split32<W>(x[k], u);
+          pad_fill<2 * W>(u, W == 1 ? pad1 : s_hop[kPadEntry]);
+          join32<W>(u, x[k]);
+        }
+        t[k] = 0.0f;
+        acc[k] = 0.0f;
+        q[k] = 0u;
+      }
+    };
     uint32_t iters = 0u;
     for (;;) {
-      unsigned int m[NCL];
-      int tot = 0;
+      // no clone of the warp has made more draws than iters
+      const bool check = ++iters >= kStepLimit / 2u;
+      unsigned int m[NCL], any = 0u;
 #pragma unroll
       for (int k = 0; k < NCL; ++k) {
         m[k] = __ballot_sync(0xffffffffu, cl[k] < 0);
-        tot += __popc(m[k]);
+        any |= m[k];
       }
-      if (tot != 0) {
+      if (any != 0u) {
         if (next >= last) break;  // on to the packed rounds below
 #pragma unroll
-        for (int k = 0; k < NCL; ++k) {
-          const int idx = next + __popc(m[k] & lt_mask);
-          if (cl[k] < 0 && idx < last) {
-            cl[k] = idx;
-            const int sk = source(J0 + (uint32_t)idx);
-            kold[k] = KXo[base + sk];
-#pragma unroll
-            for (int w = 0; w < W; ++w) x[k][w] = s_x[sk][w];
-            if constexpr (!FULL) {
-              uint32_t u[2 * W];
-              split32<W>(x[k], u);
-              pad_fill<2 * W>(u, W == 1 ? pad1 : s_hop[kPadEntry]);
-              join32<W>(u, x[k]);
-            }
-            t[k] = 0.0f;
-            acc[k] = 0.0f;
-            q[k] = 0u;
-          }
-          next += __popc(m[k]);
-        }
+        for (int k = 0; k < NCL; ++k) take(k, m[k]);
       }
-      iterate(++iters >= kStepLimit / 2u);  // no clone of the warp has made more draws
+#pragma unroll
+      for (int k = 0; k < NCL; ++k) draw(k);
+#pragma unroll
+      for (int k = 0; k < NCL; ++k) {
+        steps(k);
+        finish(k, check);
+      }
     }
     // The shares have run out.  Each round packs the block's remaining clones into the
     // lowest threads (through the staging buffer of the old clones, no longer read),
@@ -1040,7 +1049,14 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
           any = true;
         }
       }
-      if (__ballot_sync(0xffffffffu, any) != 0u) iterate(true);
+      if (__ballot_sync(0xffffffffu, any) != 0u) {
+#pragma unroll
+        for (int k = 0; k < NCL; ++k) {
+          draw(k);
+          steps(k);
+          finish(k, true);
+        }
+      }
     }
     hmin = __reduce_min_sync(0xffffffffu, hmin);
     hmax = __reduce_max_sync(0xffffffffu, hmax);
