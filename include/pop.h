@@ -157,7 +157,8 @@ int pop_run(pop_t* pop, double dt, const double* s, int64_t n_intervals);
  * NULL and K > 0, writes K + 1 entries: chain c runs the 1024-slot tiles
  * [h_first_tiles[c], h_first_tiles[c + 1]), whole populations, the last entry the
  * batch's tile count.  K is the largest number up to 8 (for a batch that fits in two
- * waves of the fused kernel on this device; up to 2 for a larger one) for which the
+ * waves of the fused kernel on this device or has at least 8 populations; up to 2 for a
+ * larger one of fewer) for which the
  * population starts nearest k/K of the tiles (k = 1 .. K-1) leave every chain at least
  * half of its equal share.
  */

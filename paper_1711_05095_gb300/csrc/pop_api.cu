@@ -31,8 +31,9 @@
 
 using namespace popgpu;
 
-// pop_run's chains (see pop_batch::nch): at most POP_RUN_CHAINS for a batch that fits
-// in two waves of the fused kernel, at most POP_RUN_CHAINS_LARGE for a larger one
+// pop_run's chains (see pop_batch::nch): at most POP_RUN_CHAINS for a batch that fits in
+// two waves of the fused kernel or has as many populations, at most POP_RUN_CHAINS_LARGE
+// for a larger one of few
 #ifndef POP_RUN_CHAINS
 #define POP_RUN_CHAINS 8
 #endif
@@ -545,8 +546,10 @@ void set_hist(pop_t* h, float dt_f) {
 
 // The rule pop_init starts from: in a batch of at most two waves of the fused kernel
 // the drain at the end of each launch and the k_weights between launches are a large
-// part of an interval, and more chains fill them; in a larger batch more chains only
-// compete.
+// part of an interval, and more chains fill them.  In a larger batch they still fill the
+// last wave of each launch, where there are populations enough to share out (8 of 2^20
+// clones, L = 128: 273 us per interval with 2 chains, 261 with 8; 256 uneven ones: 460 and
+// 458); of a few populations a chain is most of the batch and they only compete.
 int size_chains(pop_t* h) {
   int want = 1;
   if (fusable(h)) {
@@ -559,7 +562,7 @@ int size_chains(pop_t* h) {
     POP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 128, 0));
     POP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     const long long wave = (long long)(per_sm < 1 ? 1 : per_sm) * sms;
-    want = h->lay.ntiles <= 2 * wave ? POP_RUN_CHAINS : POP_RUN_CHAINS_LARGE;
+    want = h->lay.ntiles <= 2 * wave || h->lay.P >= kMaxChains ? POP_RUN_CHAINS : POP_RUN_CHAINS_LARGE;
   }
   set_chains(h, want);
   return POP_OK;
