@@ -1245,7 +1245,7 @@ int pop_lineage(pop_t* h, const int32_t* d_in, int32_t* d_out) {
   if (h == nullptr || d_in == nullptr || d_out == nullptr || d_in == d_out) return POP_ERR_ARG;
   if (h->intervals == 0 || h->phase != kReady) return POP_ERR_STATE;
   h->launches[POP_K_OTHER] += 1;
-  k_lineage<<<(unsigned)(h->lay.nslots / kThreads), kThreads, 0, h->stream>>>(h->B, d_in, d_out);
+  k_lineage<<<(unsigned)h->lay.ntiles, kThreads, 0, h->stream>>>(h->B, d_in, d_out);
   return cuda_status(cudaGetLastError());
 }
 

@@ -1911,9 +1911,15 @@ __global__ void __launch_bounds__(kThreads) k_copy_wide(Batch B) {
 // occupied sites in increasing order of float(cos), float(sin) of 2 pi n x / L
 // (cs[x], from the host); |delta rho_n|^2 = (C^2 + S^2) / L in FP32; per tile the
 // FP64 sum over its clones.
+// Every site in turn, with the additions under the site's bit and its pair of values read
+// from shared memory by all lanes at once: about five instructions a site without
+// divergence, where a loop over each clone's set bits with a table load for each took some
+// 28 per particle (2^21 clones of L = 128: 154 us).
 template <int W>
 __global__ void __launch_bounds__(kThreads) k_density(Batch B, const float2* cs, double* tile_acc) {
   __shared__ double s_part[kWarps];
+  __shared__ float4 s_cs[32 * (W > 0 ? W : 8)];  // pairs of sites; wide lattices 8 words at a time
+  constexpr int WB = W > 0 ? W : 8;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int tile = blockIdx.x;
   const int p = B.tile_pop[tile];
@@ -1921,22 +1927,52 @@ __global__ void __launch_bounds__(kThreads) k_density(Batch B, const float2* cs,
   const float2* tab = cs + (size_t)p * kInvStride;
   const int64_t base = (int64_t)tile * kTile;
   const int nw = W > 0 ? W : B.W;
-  double acc = 0.0;
-  for (int i = tid; i < kTile; i += kThreads) {
-    if (base - d.off + i >= d.nc) continue;
-    float c = 0.0f, sn = 0.0f;
-    for (int q = 0; q < nw; ++q) {
-      unsigned long long bits = B.Y[(base + i) * nw + q];
-      while (bits) {
-        const int b = __ffsll((long long)bits) - 1;
-        const float2 v = tab[64 * q + b];
-        c = __fadd_rn(c, v.x);
-        sn = __fadd_rn(sn, v.y);
-        bits &= bits - 1ull;
-      }
+  float c[kItems], sn[kItems];
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) c[i] = sn[i] = 0.0f;
+  for (int w0 = 0; w0 < nw; w0 += WB) {
+    __syncthreads();
+    for (int e = tid; e < 32 * WB; e += kThreads) {
+      const int x = 64 * w0 + 2 * e;
+      const float2 a = x < d.L ? tab[x] : make_float2(0.0f, 0.0f);
+      const float2 b = x + 1 < d.L ? tab[x + 1] : make_float2(0.0f, 0.0f);
+      s_cs[e] = make_float4(a.x, a.y, b.x, b.y);
     }
-    acc += (double)__fdiv_rn(__fadd_rn(__fmul_rn(c, c), __fmul_rn(sn, sn)), (float)d.L);
+    __syncthreads();
+    for (int w = 0; w < WB && w0 + w < nw; ++w) {
+      uint32_t v[kItems][2];
+#pragma unroll
+      for (int i = 0; i < kItems; ++i) {
+        const int64_t slot = base + i * kThreads + tid;
+        const unsigned long long x = slot - d.off < d.nc ? B.Y[slot * nw + w0 + w] : 0ull;
+        v[i][0] = (uint32_t)x;
+        v[i][1] = (uint32_t)(x >> 32);
+      }
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf)
+#pragma unroll 4
+        for (int e = 0; e < 16; ++e) {
+          const float4 q = s_cs[32 * w + 16 * hf + e];
+#pragma unroll
+          for (int i = 0; i < kItems; ++i) {
+            if (v[i][hf] & 1u) {
+              c[i] = __fadd_rn(c[i], q.x);
+              sn[i] = __fadd_rn(sn[i], q.y);
+            }
+            if (v[i][hf] & 2u) {
+              c[i] = __fadd_rn(c[i], q.z);
+              sn[i] = __fadd_rn(sn[i], q.w);
+            }
+            v[i][hf] >>= 2;
+          }
+        }
+    }
   }
+  double acc = 0.0;
+#pragma unroll
+  for (int i = 0; i < kItems; ++i)
+    if (base - d.off + i * kThreads + tid < d.nc)
+      acc += (double)__fdiv_rn(__fadd_rn(__fmul_rn(c[i], c[i]), __fmul_rn(sn[i], sn[i])), (float)d.L);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) s_part[wid] = acc;
@@ -1948,14 +1984,26 @@ __global__ void __launch_bounds__(kThreads) k_density(Batch B, const float2* cs,
   }
 }
 
-// Sum of the carried activities of each population (for k_hat, eq. khat).
-// Ancestry across the last cloning stage: out[off + j] = in[off + anc_j].
+// Ancestry across the last cloning stage: out[off + j] = in[off + anc_j].  One block per
+// tile, four slots per thread side by side (a slot per thread, with the population's
+// descriptor read for each, took 24 us for 2^22 clones); in and out are the caller's and
+// need no more than their own alignment.
 __global__ void __launch_bounds__(kThreads) k_lineage(Batch B, const int32_t* in, int32_t* out) {
-  const int64_t slot = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  const PopDesc d = B.pops[B.tile_pop[slot / kTile]];
-  if (slot - d.off < d.nc) out[slot] = in[d.off + B.anc[slot]];
+  const int tile = blockIdx.x, p = B.tile_pop[tile];
+  const int64_t off = B.pops[p].off, nc = B.pops[p].nc;
+  const int64_t base = (int64_t)tile * kTile;
+  const int32_t* const from = in + off;
+  int32_t a[kItems];
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) a[i] = B.anc[base + i * kThreads + threadIdx.x];
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    const int64_t slot = base + i * kThreads + threadIdx.x;
+    if (slot - off < nc) out[slot] = from[a[i]];
+  }
 }
 
+// Sum of the carried activities of each population (for k_hat, eq. khat).
 __global__ void __launch_bounds__(kThreads) k_ksum(Batch B) {
   __shared__ long long s_part[kWarps];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
