@@ -113,7 +113,8 @@ __device__ __forceinline__ bool bkl_step_pred(uint32_t (&u)[2 * W], float& t, fl
 // bond lies in the lane whose range of an exclusive prefix of the lanes' counts holds k,
 // and the draw, the waiting time and the bond are the same on every lane of the group
 // (the same arithmetic as with one lane, so the same results).
-// A persistent grid: each warp has an even share of the slots and walks it tile by tile;
+// A persistent grid: each warp has an even share of the slots and walks it population by
+// population (it drains at the end of each: by tiles, 395 us per interval of the [iid] study);
 // a group whose clone ended takes the share's next clone, so a warp needs no barrier and
 // no shared counter.  Clones go from global memory to registers and back.
 // Bound by ALU issue.  An interval of 2^22 clones of L = 128, dt = 0.05 by the per-step
@@ -239,9 +240,9 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
   int64_t slot0 = (wi * B.unit_q + min(wi, B.unit_r)) * (32 / G);
   const int64_t slot_end = slot0 + (B.unit_q + (wi < B.unit_r ? 1 : 0)) * (32 / G);
   while (slot0 < slot_end) {
-    const int64_t seg_end = min(slot_end, (slot0 / kTile + 1) * kTile);  // one tile, one population
     const int p = B.tile_pop[slot0 / kTile];
     const PopDesc d = B.pops[p];
+    const int64_t seg_end = min(slot_end, d.off + (int64_t)d.ntiles * kTile);  // within one population
     const int64_t j0 = slot0 - d.off;
     const int n = (int)max((int64_t)0, min(seg_end - slot0, d.nc - j0));  // warp-uniform
     const float* inv = B.inv_rate + (size_t)p * kInvStride;
@@ -1622,7 +1623,8 @@ __device__ __forceinline__ float i64_to_float_rn(long long v) {
 }
 
 // One lane per clone.  A persistent grid as k_evolve's: each warp has an even share of the
-// slots and walks it tile by tile, a lane whose clone ended takes the share's next one.
+// slots and walks it population by population, a lane whose clone ended takes the share's
+// next one.
 // Per lane in shared memory: the rate sums of the clone's groups of eight bonds and its
 // sites as a bit string that starts eight sites before site 0 and goes on past the closing
 // bond, so the sites that rate group g are the 25 bits from bit 8 g on, one unaligned word.
@@ -1668,9 +1670,9 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
   int64_t slot0 = (wi * B.unit_q + min(wi, B.unit_r)) * 32;
   const int64_t slot_end = slot0 + (B.unit_q + (wi < B.unit_r ? 1 : 0)) * 32;
   while (slot0 < slot_end) {
-    const int64_t seg_end = min(slot_end, (slot0 / kTile + 1) * kTile);  // one tile, one population
     const int p = B.tile_pop[slot0 / kTile];
     const PopDesc d = B.pops[p];
+    const int64_t seg_end = min(slot_end, d.off + (int64_t)d.ntiles * kTile);  // within one population
     const int64_t j0 = slot0 - d.off;
     const int n = (int)max((int64_t)0, min(seg_end - slot0, d.nc - j0));  // warp-uniform
     const int L = d.L;
