@@ -388,23 +388,27 @@ int launch_evolve(pop_t* h, cudaStream_t st, float dt_f) {
 
 // The tile prefixes and totals of the populations [pop0, pop1); hist: the tile sums and
 // activity histograms too, from the tile histograms of the fused stage.
-void launch_tile_scan(pop_t* h, cudaStream_t st, const Batch& Bx, int pop0, int pop1, bool hist = false) {
+void launch_tile_scan(pop_t* h, cudaStream_t st, const Batch& Bx, int pop0, int pop1, bool hist = false,
+                      bool early = false) {
   kernel_begin(h, st, hist ? POP_K_WEIGHTS : POP_K_OTHER);
-  if (hist) k_tile_scan<true><<<(unsigned)(pop1 - pop0), kScanThreads, 0, st>>>(Bx, pop0);
-  else k_tile_scan<false><<<(unsigned)(pop1 - pop0), kScanThreads, 0, st>>>(Bx, pop0);
+  const unsigned grid = (unsigned)(pop1 - pop0);
+  if (early) launch_early(hist ? k_tile_scan<true> : k_tile_scan<false>, grid, kScanThreads, 0, st, Bx, pop0);
+  else if (hist) k_tile_scan<true><<<grid, kScanThreads, 0, st>>>(Bx, pop0);
+  else k_tile_scan<false><<<grid, kScanThreads, 0, st>>>(Bx, pop0);
   kernel_end(h, st);
 }
 
 // k_weights over the tiles [tile0, tile0 + ntiles), one block per tile
-void launch_weights_range(pop_t* h, cudaStream_t st, const Batch& Bx, int tile0, int ntiles) {
+void launch_weights_range(pop_t* h, cudaStream_t st, const Batch& Bx, int tile0, int ntiles, bool early = false) {
   kernel_begin(h, st, POP_K_WEIGHTS);
-  k_weights<<<(unsigned)ntiles, kThreads, 0, st>>>(Bx, tile0);
+  if (early) launch_early(k_weights, (unsigned)ntiles, kThreads, 0, st, Bx, tile0);
+  else k_weights<<<(unsigned)ntiles, kThreads, 0, st>>>(Bx, tile0);
   kernel_end(h, st);
 }
 
 void launch_weights(pop_t* h, cudaStream_t st) {
-  launch_weights_range(h, st, h->B, 0, h->lay.ntiles);
-  launch_tile_scan(h, st, h->B, 0, h->lay.P);
+  launch_weights_range(h, st, h->B, 0, h->lay.ntiles, true);
+  launch_tile_scan(h, st, h->B, 0, h->lay.P, false, true);
 }
 
 int launch_resample(pop_t* h, cudaStream_t st) {
@@ -419,15 +423,15 @@ int launch_resample(pop_t* h, cudaStream_t st) {
     // many waves of tiles: 256-thread blocks keep more bytes in flight (measured
     // 4567 against 4379 GB/s on 2^25 two-word clones)
     constexpr int GW = POP_GATHER_WIDE_THREADS;
-    if (h->lay.W == 1) k_gather<1, GW><<<grid, GW, 0, st>>>(h->B, 0.0f, 0);
-    else if (h->lay.W == 2) k_gather<2, GW><<<grid, GW, 0, st>>>(h->B, 0.0f, 0);
-    else k_gather<0, GW><<<grid, GW, 0, st>>>(h->B, 0.0f, 0);
+    if (h->lay.W == 1) launch_early(k_gather<1, GW>, grid, GW, 0, st, h->B, 0.0f, 0);
+    else if (h->lay.W == 2) launch_early(k_gather<2, GW>, grid, GW, 0, st, h->B, 0.0f, 0);
+    else launch_early(k_gather<0, GW>, grid, GW, 0, st, h->B, 0.0f, 0);
   } else if (h->lay.W == 1) {
-    k_gather<1, GT><<<grid, GT, 0, st>>>(h->B, 0.0f, 0);
+    launch_early(k_gather<1, GT>, grid, GT, 0, st, h->B, 0.0f, 0);
   } else if (h->lay.W == 2) {
-    k_gather<2, GT><<<grid, GT, 0, st>>>(h->B, 0.0f, 0);
+    launch_early(k_gather<2, GT>, grid, GT, 0, st, h->B, 0.0f, 0);
   } else {
-    k_gather<0, GT><<<grid, GT, 0, st>>>(h->B, 0.0f, 0);
+    launch_early(k_gather<0, GT>, grid, GT, 0, st, h->B, 0.0f, 0);
   }
   kernel_end(h, st);
   if (h->B.any_iid) {
@@ -439,7 +443,7 @@ int launch_resample(pop_t* h, cudaStream_t st) {
   }
   if (h->lay.W > 2) {
     kernel_begin(h, st, POP_K_GATHER);
-    k_copy_wide<<<dim3(grid, (unsigned)h->lay.W), kThreads, 0, st>>>(h->B);
+    launch_early(k_copy_wide, dim3(grid, (unsigned)h->lay.W), kThreads, 0, st, h->B);
     kernel_end(h, st);
   }
   return cuda_status(cudaGetLastError());
@@ -1245,7 +1249,7 @@ int pop_lineage(pop_t* h, const int32_t* d_in, int32_t* d_out) {
   if (h == nullptr || d_in == nullptr || d_out == nullptr || d_in == d_out) return POP_ERR_ARG;
   if (h->intervals == 0 || h->phase != kReady) return POP_ERR_STATE;
   h->launches[POP_K_OTHER] += 1;
-  k_lineage<<<(unsigned)h->lay.ntiles, kThreads, 0, h->stream>>>(h->B, d_in, d_out);
+  launch_early(k_lineage, (unsigned)h->lay.ntiles, kThreads, 0, h->stream, h->B, d_in, d_out);
   return cuda_status(cudaGetLastError());
 }
 

@@ -226,6 +226,7 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
   reinterpret_cast<uint4*>(s_kth8)[tid] = reinterpret_cast<const uint4*>(g_kth8.w)[tid];
   __syncthreads();
   const uint8_t* const kth8 = reinterpret_cast<const uint8_t*>(s_kth8);
+  grid_release();
   const uint32_t beta = *B.beta;
   const int par = (int)(beta & 1u);
   const int sub = lane & (G - 1), lead = lane & ~(G - 1);
@@ -380,6 +381,9 @@ __global__ void __launch_bounds__(kThreads) k_weights(Batch B, int tile0) {
   PopState* st = B.st + p;
   const int64_t base = (int64_t)tile * kTile;
   const int64_t j0 = base - d.off + (int64_t)tid * kItems;
+  for (int i = tid; i < kHistSmem; i += kThreads) s_hist[i] = 0u;
+  grid_wait();
+  grid_release();
   const uint32_t beta = *B.beta;  // the interval being resampled (no kernel advances it meanwhile)
   const int par = (int)(beta & 1u);
   const int4 dk4 = reinterpret_cast<const int4*>(B.dKb[par] + base)[tid];
@@ -388,7 +392,6 @@ __global__ void __launch_bounds__(kThreads) k_weights(Batch B, int tile0) {
     const float4 a4 = reinterpret_cast<const float4*>(B.Ab[par] + base)[tid];
     av[0] = a4.x; av[1] = a4.y; av[2] = a4.z; av[3] = a4.w;
   }
-  for (int i = tid; i < kHistSmem; i += kThreads) s_hist[i] = 0u;
   const int dk_min = st->dk_min[par], dk_max = st->dk_max[par];
   const int kref = d.s_neg ? dk_max : dk_min;
   // MODIFIED reference: the smallest (s >= 0) or largest (s < 0) rate integral;
@@ -464,6 +467,8 @@ __global__ void __launch_bounds__(kScanThreads, 3) k_tile_scan(Batch B, int pop0
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int p = pop0 + (int)blockIdx.x;
   const PopDesc d = B.pops[p];
+  grid_wait();
+  grid_release();
   if constexpr (HIST) {
     PopState* st = B.st + p;
     const uint32_t beta = *B.beta;  // the interval being resampled
@@ -659,12 +664,6 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
   const uint32_t nc = (uint32_t)d.nc;
   const int64_t base = (int64_t)tile * kTile;
   const int64_t j0 = base - d.off + (int64_t)tid * NI;
-  // the interval being resampled, as recorded by k_weights: the device counter is
-  // advanced by this kernel's last block and may not be read here
-  const uint32_t beta = st->beta;
-  const int par = (int)(beta & 1u);
-  const unsigned long long* const Xo = B.Xb[par];
-  const int32_t* const KXo = B.KXb[par];
   if constexpr (FUSE) {
     const float* src = B.inv_rate + (size_t)p * kInvStride;
     for (int r = tid; r <= kMaxL; r += NT)  // inv[0] = NaN: see bkl_step_pred
@@ -688,6 +687,16 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     }
   }
 
+  if constexpr (!FUSE) {
+    grid_wait();
+    grid_release();
+  }
+  // the interval being resampled, as recorded by k_weights: the device counter is
+  // advanced by this kernel's last block and may not be read here
+  const uint32_t beta = st->beta;
+  const int par = (int)(beta & 1u);
+  const unsigned long long* const Xo = B.Xb[par];
+  const int32_t* const KXo = B.KXb[par];
   const unsigned long long* wt = B.wtab + (size_t)p * kKcap;
   // independent loads first: activities and the old clones of this tile
   int dkv[NI];
@@ -1461,6 +1470,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
 // ---------------------------------------------------------------------------
 template <int W>
 __global__ void __launch_bounds__(kThreads) k_select_iid(Batch B) {
+  grid_release();
   const int tid = threadIdx.x;
   const int tile = blockIdx.x;
   const int p = B.tile_pop[tile];
@@ -1661,6 +1671,7 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (tid < 64) s_log[tid] = B.logtab[tid];
   __syncthreads();
+  grid_release();
   const uint32_t beta = *B.beta;
   const int par = (int)(beta & 1u);
   const unsigned int lt_mask = (1u << lane) - 1u;
@@ -1893,6 +1904,8 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
 // clone, one after the other) it was 64 blocks of dependent loads for 2^16 clones of
 // four words: 176 us.
 __global__ void __launch_bounds__(kThreads) k_copy_wide(Batch B) {
+  grid_wait();
+  grid_release();
   const int tile = blockIdx.x;
   const int p = B.tile_pop[tile];
   const PopDesc d = B.pops[p];
@@ -1991,6 +2004,8 @@ __global__ void __launch_bounds__(kThreads) k_density(Batch B, const float2* cs,
 // descriptor read for each, took 24 us for 2^22 clones); in and out are the caller's and
 // need no more than their own alignment.
 __global__ void __launch_bounds__(kThreads) k_lineage(Batch B, const int32_t* in, int32_t* out) {
+  grid_wait();
+  grid_release();
   const int tile = blockIdx.x, p = B.tile_pop[tile];
   const int64_t off = B.pops[p].off, nc = B.pops[p].nc;
   const int64_t base = (int64_t)tile * kTile;

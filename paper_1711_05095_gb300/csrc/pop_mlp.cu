@@ -28,6 +28,7 @@
 #include <new>
 
 #include "pop.h"
+#include "pop_common.cuh"
 
 namespace popmlp {
 
@@ -104,6 +105,8 @@ __global__ void __launch_bounds__(256) k_forward(Work w) {
   __shared__ float s_phi[8][kRows];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3;
   const int p0 = blockIdx.x * kRows;
+  popgpu::grid_wait();
+  popgpu::grid_release();
   if (blockIdx.x == 0) {  // the sums of k_logits start at zero
     w.dPhi[tid] = 0.0;
     w.dPhi[tid + 256] = 0.0;
@@ -268,13 +271,15 @@ __global__ void __launch_bounds__(kLT) k_logits(Work w, const unsigned long long
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int64_t j_end = min(n, ((int64_t)blockIdx.x + 1) * per_block);
   const int ngr = L >> 2;
-  S.phi[tid] = w.Phi[tid];
-  S.phi[tid + kLT] = w.Phi[tid + kLT];
-  const float c = w.theta[oc];
   for (int b = tid; b < kBins + kPat; b += kLT) {
     S.lo[b] = 0u;
     S.hi[b] = 0;
   }
+  popgpu::grid_wait();
+  popgpu::grid_release();
+  S.phi[tid] = w.Phi[tid];
+  S.phi[tid + kLT] = w.Phi[tid + kLT];
+  const float c = w.theta[oc];
   __syncthreads();
   for (int q = tid; q < kBins; q += kLT)
     S.s4[q] = ((S.phi[q & 511] + S.phi[(q >> 1) & 511]) + S.phi[(q >> 2) & 511]) + S.phi[q >> 3];
@@ -430,6 +435,8 @@ __global__ void __launch_bounds__(256) k_back_patterns(Work w) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3;
   const int p0 = blockIdx.x * kRows;
   float* const part = w.part + blockIdx.x * kPart;
+  popgpu::grid_wait();
+  popgpu::grid_release();
   // B(k, n) = W2[k][n]: pairs along k are two rows
   uint32_t b[2][8][2];
 #pragma unroll
@@ -526,6 +533,8 @@ constexpr int kTileBlocks = (kH / 16) * (kH / 16);
 constexpr int kSmall = 9 * kH + 3 * kH + 2;
 __global__ void __launch_bounds__(256) k_back_weights(Work w, Adam o) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3;
+  popgpu::grid_wait();
+  popgpu::grid_release();
   if (blockIdx.x < kTileBlocks) {
     __shared__ float s_c[8][16][17];
     const int m0 = (blockIdx.x / (kH / 16)) * 16, n0 = (blockIdx.x % (kH / 16)) * 16;
@@ -625,7 +634,7 @@ namespace {
   } while (0)
 
 int forward(pop_mlp_t* h) {
-  k_forward<<<kPB, 256, 0, h->stream>>>(h->w);
+  popgpu::launch_early(k_forward, kPB, 256, 0, h->stream, h->w);
   return cudaGetLastError() == cudaSuccess ? POP_OK : POP_ERR_CUDA;
 }
 
@@ -636,10 +645,10 @@ int backward(pop_mlp_t* h, const uint64_t* d_lat, int32_t W, int32_t L, const ui
   // cost about as much as 64 configurations
   int64_t per = (n + h->logits_blocks - 1) / h->logits_blocks;
   per = (per + 63) / 64 * 64;
-  k_logits<<<(unsigned)((n + per - 1) / per), kLT, sizeof(LogitsSmem), st>>>(
-      h->w, (const unsigned long long*)d_lat, W, L, d_lab, n, per);
-  k_back_patterns<<<kPB, 256, 0, st>>>(h->w);
-  k_back_weights<<<kTileBlocks + (kSmall + 255) / 256, 256, 0, st>>>(h->w, adam);
+  popgpu::launch_early(k_logits, (unsigned)((n + per - 1) / per), kLT, sizeof(LogitsSmem), st, h->w,
+                       (const unsigned long long*)d_lat, W, L, d_lab, n, per);
+  popgpu::launch_early(k_back_patterns, kPB, 256, 0, st, h->w);
+  popgpu::launch_early(k_back_weights, kTileBlocks + (kSmall + 255) / 256, 256, 0, st, h->w, adam);
   return cudaGetLastError() == cudaSuccess ? POP_OK : POP_ERR_CUDA;
 }
 

@@ -97,6 +97,8 @@ __global__ void __launch_bounds__(kThreads) k_sel_range(SelArgs A) {
   __shared__ int s_mn[kWarps], s_mx[kWarps];
   const int tid = threadIdx.x;
   const int64_t base = (int64_t)blockIdx.x * kTile;
+  grid_wait();
+  grid_release();
   for (int b = (int)blockIdx.x * kThreads + tid; b < kKcap; b += A.ntiles * kThreads) A.hist[b] = 0u;
   if (blockIdx.x == 0 && tid == 0) A.st->err = 0;
   int mn = INT_MAX, mx = INT_MIN;
@@ -138,6 +140,9 @@ __global__ void __launch_bounds__(kThreads) k_sel_weights(SelArgs A) {
   const int tid = threadIdx.x;
   const int tile = blockIdx.x;
   const int64_t base = (int64_t)tile * kTile;
+  for (int b = tid; b < kHistSmem; b += kThreads) s_hist[b] = 0u;
+  grid_wait();
+  grid_release();
   int dk[kItems];
 #pragma unroll
   for (int i = 0; i < kItems; ++i) {
@@ -156,7 +161,6 @@ __global__ void __launch_bounds__(kThreads) k_sel_weights(SelArgs A) {
     s_mn[tid >> 5] = mn;
     s_mx[tid >> 5] = mx;
   }
-  for (int b = tid; b < kHistSmem; b += kThreads) s_hist[b] = 0u;
   __syncthreads();
 #pragma unroll
   for (int w = 0; w < kWarps; ++w) {
@@ -203,6 +207,7 @@ __global__ void __launch_bounds__(kThreads) k_sel_ancestors(SelArgs A) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int tile = blockIdx.x;
   const int64_t base = (int64_t)tile * kTile;
+  grid_wait();
   const int kref = A.st->kref;
   const unsigned long long c = 2ull * (unsigned long long)A.st->U + 1ull;
   const uint32_t nc = A.nc;
@@ -336,9 +341,9 @@ extern "C" int pop_select_noalloc(const int32_t* d_dK, int64_t n_clones, double 
       return POP_ERR_CUDA;
     g_tables[dev] = TableKey{true, s, F};
   }
-  k_sel_range<<<A.ntiles, kThreads, 0, stream>>>(A);
-  k_sel_weights<<<A.ntiles, kThreads, 0, stream>>>(A);
-  k_sel_ancestors<<<A.ntiles, kThreads, 0, stream>>>(A);
+  launch_early(k_sel_range, A.ntiles, kThreads, 0, stream, A);
+  launch_early(k_sel_weights, A.ntiles, kThreads, 0, stream, A);
+  launch_early(k_sel_ancestors, A.ntiles, kThreads, 0, stream, A);
   if (cudaGetLastError() != cudaSuccess) return POP_ERR_CUDA;
   SelState out;
   if (cudaMemcpyAsync(&out, A.st, sizeof out, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
