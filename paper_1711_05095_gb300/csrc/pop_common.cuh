@@ -608,9 +608,10 @@ __device__ __forceinline__ void j_lo_run(unsigned long long S0, const unsigned l
 // 128-bit products took about 40 instructions.
 // ---------------------------------------------------------------------------
 #ifndef POP_POS_MARGIN
-#define POP_POS_MARGIN (1ull << 13)  // 2^12 and a factor of two; at most 2^31 (pos_slot)
+#define POP_POS_MARGIN (1ull << 13)  // 2^12 and a factor of two
 #endif
 constexpr unsigned long long kPosMargin = POP_POS_MARGIN;
+static_assert(2ull * kPosMargin < (1ull << 32), "pos_slot compares twice the margin in 32 bits");
 
 struct PosScale {
   unsigned long long m;  // the factor's 53 bits, leading bit at 63

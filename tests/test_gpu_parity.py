@@ -746,3 +746,48 @@ def test_many_one_tile_populations_keep_the_launch_sequence(pg):
 ])
 def test_parity_under_strong_bias(pg, L, nc, s, dt, mode, sel):
     run_parity(pg, [dict(L=L, N=L // 2, n_clones=nc, seed=600 + L, weight_mode=mode, selection=sel)], [s], dt, 3)
+
+
+def test_positions_too_close_to_a_slot_are_settled_exactly(pg, tmp_path):
+    # the cloning stage takes a clone's new slots from 64-bit positions and settles those
+    # within POP_POS_MARGIN of a slot by 128-bit comparisons; by default that is one clone
+    # in 2^28 at N_c = 2^20.  A library built with the margin 2^17 times as wide takes that
+    # path for about a clone in two thousand (four tiles in ten): separate and fused stages against
+    # the per-step calls of the ordinary library, which the oracle tests check
+    import ctypes
+    import subprocess
+    from paper_1711_05095_gb300 import build as b
+    so = str(tmp_path / "libpop_margin.so")
+    subprocess.run([b.nvcc(), "-O3", "-std=c++17", *b.ARCH, "-Xcompiler", "-fPIC", "-shared", "-DPOP_POS_MARGIN=(1ull<<30)",
+                    "-I", b.ROOT + "/include", *b.SOURCES, "-o", so], check=True)
+    pops = [dict(L=50, N=25, n_clones=200 * 1024 + 7, seed=90), dict(L=128, N=64, n_clones=2 ** 20, seed=91),
+            dict(L=30, N=15, n_clones=70 * 1024, seed=92, weight_mode=MOD)]
+    few = [dict(L=40, N=20, n_clones=60 * 1024 + 3, seed=93), dict(L=20, N=10, n_clones=9 * 1024, seed=94)]
+    cases = ((pops, [0.02, 0.001, -0.01]), (few, [0.3, -0.1]))
+    want = []
+    for q, s in cases:
+        a = pg.PopulationBatch(q)
+        for _ in range(4):
+            a.evolve(0.1, s)
+            a.resample()
+        want.append([a.copy_state(p) for p in range(len(q))])
+        a.close()
+    saved, path = pg._lib, pg.LIB_PATH
+    try:
+        pg._lib, pg.LIB_PATH = None, so
+        for (q, s), w in zip(cases, want):
+            for fused in (True, False):
+                a = pg.PopulationBatch(q)
+                if fused:
+                    a.run(0.1, s, 4)
+                else:
+                    for _ in range(4):
+                        a.evolve(0.1, s)
+                        a.resample()
+                for p in range(len(q)):
+                    g = a.copy_state(p)
+                    for key in ("lattice", "K", "anc", "dK"):
+                        assert np.array_equal(g[key], w[p][key]), (p, key, fused)
+                a.close()
+    finally:
+        pg._lib, pg.LIB_PATH = saved, path
