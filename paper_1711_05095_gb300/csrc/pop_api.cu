@@ -198,6 +198,8 @@ struct pop_batch {
   Batch chain[kMaxChains]{};                 // the batch with each chain's own interval counter
   // launch configuration (rule-based at pop_init; pop_autotune or pop_set_tuning may change it)
   int fuse_threads = 128;                    // fused kernel: threads per block (128 or 256)
+  bool one_wave = false;                     // 256 threads in place of the default 128 (size_chains) until
+                                             // pop_set_tuning or pop_autotune sets the configuration
   int fuse_clones = kFuseClones;             // fused kernel: clones per lane (1 or 2)
   int gather_threads = 0;                    // separate cloning stage: 128, 256, or 0 for the rule
   int hist_mode = -1;                        // tile activity histograms: 1 on, 0 off, -1 the rule
@@ -453,7 +455,7 @@ int launch_resample(pop_t* h, cudaStream_t st) {
 // clones per lane, or 256 threads with one.
 template <int W, bool MOD, bool SCAN, bool FULL>
 void launch_fused_form(pop_t* h, unsigned grid, cudaStream_t st, const Batch& Bx, float dt_f, int tile0) {
-  if (h->fuse_threads == 256)
+  if (h->fuse_threads == 256 || h->one_wave)
     k_gather<W, 256, true, MOD, SCAN, 1, FULL><<<grid, 256, 0, st>>>(Bx, dt_f, tile0);
   else if (h->fuse_clones == 2)
     k_gather<W, 128, true, MOD, SCAN, 2, FULL><<<grid, 128, 0, st>>>(Bx, dt_f, tile0);
@@ -566,6 +568,11 @@ int size_chains(pop_t* h) {
     POP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 128, 0));
     POP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     const long long wave = (long long)(per_sm < 1 ? 1 : per_sm) * sms;
+    // a batch within one wave is bound by the latency of a tile: twice the threads, half the
+    // clones each (populations of 16 tiles, L = 50, dt = 0.1; 8, 16, 32 and 64 of them: 23,
+    // 25, 28 and 35 us per interval with 128 threads, 19, 21, 24 and 34 with 256); beyond,
+    // the smaller blocks pack better (256 uneven populations: 474 and 521)
+    h->one_wave = h->lay.ntiles <= wave;
     want = h->lay.ntiles <= 2 * wave || h->lay.P >= kMaxChains ? POP_RUN_CHAINS : POP_RUN_CHAINS_LARGE;
   }
   set_chains(h, want);
@@ -1343,13 +1350,14 @@ int pop_autotune(pop_t* h, double dt, const double* s, int32_t trials, int32_t* 
   if (rc == POP_OK && fusable(h) && !run_small(h)) {
     const int forms[3][2] = {{128, 1}, {128, 2}, {256, 1}};
     const int wants[4] = {1, 2, 4, 8};
-    const int def_threads = h->fuse_threads, def_clones = h->fuse_clones, def_nch = h->nch;
+    const int def_threads = h->one_wave ? 256 : h->fuse_threads, def_clones = h->fuse_clones, def_nch = h->nch;
     const int def_hist = h->hist_mode;
     const bool def_on = h->B.hist_on != 0;
     const bool hist_ok = !h->any_mod && (double)dt_f * h->max_L <= 16.0;
     int bt = def_threads, bc = def_clones, bw = def_nch, bh = def_hist;
     float bms = 1e30f, def_ms = 0.0f;
     int last_nch = -1;
+    h->one_wave = false;
     for (int hm = 0; hm < (hist_ok ? 2 : 1) && rc == POP_OK; ++hm)
     for (int f = 0; f < 3 && rc == POP_OK; ++f) {
       last_nch = -1;
@@ -1498,6 +1506,7 @@ int pop_set_tuning(pop_t* h, const pop_tuning* cfg) {
     return POP_ERR_ARG;
   if (h->phase != kReady) return POP_ERR_STATE;
   set_evolve_grid(h, cfg->evolve_grid);
+  h->one_wave = false;
   h->fuse_threads = cfg->fuse_threads;
   h->fuse_clones = cfg->fuse_clones;
   h->gather_threads = cfg->gather_threads;
