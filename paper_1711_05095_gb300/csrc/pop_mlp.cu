@@ -54,8 +54,8 @@ struct Work {
   double* dc;    // sum over the batch of dL/dz
   double* dPhi;  // [512]
   float* Phi;    // [512]
-  float* Z1;     // [512][128] pre-activations
-  float* Z2;
+  float* G1;     // [512][128] GELU' of the pre-activations of layers 1 and 2
+  float* G2;
   __nv_bfloat16* H1T;   // [128][512] activations of layer 1, hidden unit major
   __nv_bfloat16* H2;    // [512][128]
   __nv_bfloat16* dZ2T;  // [128][512]
@@ -66,11 +66,12 @@ __device__ __forceinline__ float bf(float x) { return __bfloat162float(__float2b
 
 // GELU(x) = x Phi(x) with Phi(x) = erfc(-x / sqrt 2) / 2: the complementary error
 // function keeps the relative accuracy for negative x, where 1 + erf would cancel.
-__device__ __forceinline__ float gelu(float x) {
-  return 0.5f * x * erfcf(x * -0.70710678118654752f);
-}
-__device__ __forceinline__ float gelu_grad(float x) {
-  return 0.5f * erfcf(x * -0.70710678118654752f) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
+// The forward pass takes the derivative along (one erfc for both), so the backward pass,
+// whose blocks wait for one another's results, only loads it.
+__device__ __forceinline__ float gelu(float x, float& grad) {
+  const float c = erfcf(x * -0.70710678118654752f);
+  grad = 0.5f * c + x * expf(-0.5f * x * x) * 0.39894228040143268f;
+  return 0.5f * x * c;
 }
 
 // D += A B for one m16n8k16 tile.  Fragment layout (PTX ISA), g = lane / 4, t = lane % 4:
@@ -138,8 +139,9 @@ __global__ void __launch_bounds__(256) k_forward(Work w) {
 #pragma unroll
       for (int k = 0; k < 9; ++k)
         if ((p >> k) & 1) z += w1[k];
-      w.Z1[p * kH + h] = z;
-      const __nv_bfloat16 hb = __float2bfloat16_rn(gelu(z));
+      float gr;
+      const __nv_bfloat16 hb = __float2bfloat16_rn(gelu(z, gr));
+      w.G1[p * kH + h] = gr;
       s_h1[r0 + r][h] = hb;
       const uint32_t bits = __bfloat16_as_ushort(hb);
       pk[r >> 1] = (r & 1) ? pk[r >> 1] | (bits << 16) : bits;
@@ -165,9 +167,9 @@ __global__ void __launch_bounds__(256) k_forward(Work w) {
     for (int r = 0; r < 2; ++r) {
       const int at = (p0 + g + 8 * r) * kH + n;
       const float z0 = c[nt][2 * r] + bias0, z1 = c[nt][2 * r + 1] + bias1;
-      w.Z2[at] = z0;
-      w.Z2[at + 1] = z1;
-      const float h0 = bf(gelu(z0)), h1 = bf(gelu(z1));
+      float g0, g1;
+      const float h0 = bf(gelu(z0, g0)), h1 = bf(gelu(z1, g1));
+      *reinterpret_cast<float2*>(w.G2 + at) = make_float2(g0, g1);
       *reinterpret_cast<uint32_t*>(w.H2 + at) = pack_bf16(h0, h1);
       dot[r] += h0 * v0 + h1 * v1;
     }
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(256) k_forward(Work w) {
 // FP32 sum.  Non-finite d take a plain FP64 path that gives the same infinities and NaN.
 // A gradient of 16384 configurations of L = 128, its read-back included: 151 us with a
 // thread per configuration and FP32 adds per window (55 us of it here) in nine launches,
-// 69 us now; of 2^20: 493 us, now 120.
+// 56 us now; of 2^20: 493 us, now 108.
 // ---------------------------------------------------------------------------
 constexpr int kLT = 256;                      // threads
 constexpr int kCfg = 8;                       // configurations per thread and chunk
@@ -461,7 +463,7 @@ __global__ void __launch_bounds__(256) k_back_patterns(Work w) {
     for (int r = 0; r < 8; ++r) {
       const int at = (p0 + r0 + r) * kH + h;
       const float dphi = s_dphi[r0 + r];
-      const float dz = dphi * w3 * gelu_grad(w.Z2[at]);
+      const float dz = dphi * w3 * w.G2[at];
       s2 += dz;
       s3 += __bfloat162float(w.H2[at]) * dphi;
       const __nv_bfloat16 db = __float2bfloat16_rn(dz);
@@ -494,8 +496,8 @@ __global__ void __launch_bounds__(256) k_back_patterns(Work w) {
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int n = wid * 16 + nt * 8 + 2 * t + q;
-      const float lo = c[nt][q] * gelu_grad(w.Z1[(p0 + g) * kH + n]);
-      const float up = c[nt][2 + q] * gelu_grad(w.Z1[(p0 + g + 8) * kH + n]);
+      const float lo = c[nt][q] * w.G1[(p0 + g) * kH + n];
+      const float up = c[nt][2 + q] * w.G1[(p0 + g + 8) * kH + n];
       const float all = sum_rows(lo + up), bit3 = sum_rows(up);
       float bit[3];
 #pragma unroll
@@ -588,7 +590,7 @@ __global__ void __launch_bounds__(256) k_back_weights(Work w, Adam o) {
 size_t align256(size_t x) { return (x + 255u) & ~(size_t)255u; }
 
 struct Layout {
-  size_t theta, m, v, loss, grad, dc, dPhi, Phi, Z1, Z2, H1T, H2, dZ2T, part, total;
+  size_t theta, m, v, loss, grad, dc, dPhi, Phi, G1, G2, H1T, H2, dZ2T, part, total;
 };
 
 Layout layout() {
@@ -603,8 +605,8 @@ Layout layout() {
   l.dc = take(8);
   l.dPhi = take(kPat * 8);
   l.Phi = take(kPat * 4);
-  l.Z1 = take(kPat * kH * 4);
-  l.Z2 = take(kPat * kH * 4);
+  l.G1 = take(kPat * kH * 4);
+  l.G2 = take(kPat * kH * 4);
   l.H1T = take(kPat * kH * 2);
   l.H2 = take(kPat * kH * 2);
   l.dZ2T = take(kPat * kH * 2);
@@ -641,10 +643,13 @@ int forward(pop_mlp_t* h) {
 int backward(pop_mlp_t* h, const uint64_t* d_lat, int32_t W, int32_t L, const uint8_t* d_lab,
              int64_t n, const Adam& adam) {
   cudaStream_t st = h->stream;
-  // an even split of the configurations, at least 64 to a block: the tables a block builds
-  // cost about as much as 64 configurations
-  int64_t per = (n + h->logits_blocks - 1) / h->logits_blocks;
-  per = (per + 63) / 64 * 64;
+  // an even split of the configurations.  A block's tables cost as much as hundreds of
+  // configurations, and its threads take one each side by side: at least 256 to a block,
+  // and up to 1024 before an SM gets a second one (16384 configurations: 40 us per step with
+  // 64 to a block, 32 with 256)
+  const int64_t sms = h->logits_blocks / 4;
+  int64_t per = n <= 1024 * sms ? (n + sms - 1) / sms : (n + h->logits_blocks - 1) / h->logits_blocks;
+  per = (per + 255) / 256 * 256;
   popgpu::launch_early(k_logits, (unsigned)((n + per - 1) / per), kLT, sizeof(LogitsSmem), st, h->w,
                        (const unsigned long long*)d_lat, W, L, d_lab, n, per);
   popgpu::launch_early(k_back_patterns, kPB, 256, 0, st, h->w);
@@ -684,8 +689,8 @@ int pop_mlp_init(pop_mlp_t** out, const float* h_theta, void* d_workspace, size_
   w.dc = (double*)(h->ws + l.dc);
   w.dPhi = (double*)(h->ws + l.dPhi);
   w.Phi = (float*)(h->ws + l.Phi);
-  w.Z1 = (float*)(h->ws + l.Z1);
-  w.Z2 = (float*)(h->ws + l.Z2);
+  w.G1 = (float*)(h->ws + l.G1);
+  w.G2 = (float*)(h->ws + l.G2);
   w.H1T = (__nv_bfloat16*)(h->ws + l.H1T);
   w.H2 = (__nv_bfloat16*)(h->ws + l.H2);
   w.dZ2T = (__nv_bfloat16*)(h->ws + l.dZ2T);
