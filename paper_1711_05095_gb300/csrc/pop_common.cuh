@@ -4,16 +4,16 @@
 // kernels over a batch of populations laid out back to back in "slots" (every
 // population starts on a 1024-slot tile):
 //   k_evolve   dynamical stage (Sec. 4: BKL continuous-time Monte Carlo of the SSEP,
-//              Sec. 3.1 rates).  A persistent grid; each block owns an equal range of
-//              256-slot units, stages the clones in shared memory and advances them in
-//              rounds of one BKL step per running clone, compacting the running clones
-//              after each round so that every lane does useful work.  Epilogue: the
-//              per-population min/max of the interval activity.
+//              Sec. 3.1 rates).  A persistent grid; each warp has an even share of the
+//              slots, holds its clones in registers and advances them two predicated BKL
+//              steps per Philox draw, a lane whose clone ended taking the share's next one.
+//              Epilogue: the per-population min/max of the interval activity.
 //   k_weights  fixed-point weights exp(-s dK) (64-bit), their per-tile sums and the
 //              histogram of the interval activity.
 //   k_gather   per tile: the exclusive prefix sums of the weights (tile sums, then a
 //              block scan), [eq] selection (Sec. 4.1, eq. alpha-Ups) inverted per old
-//              clone in exact integers, and a pull copy of lattices and carried
+//              clone (fixed-point positions, exact integers where one is too close to
+//              call), and a pull copy of lattices and carried
 //              activities (eq. khat) staged through shared memory.  The first tile of
 //              each population adds the psi term of eq. (psihat).
 // All arithmetic that decides an integer result (waiting times, bond choice,
