@@ -11,8 +11,8 @@
 //
 // One interval = k_evolve, k_weights, k_gather on the caller's stream.  pop_run fuses
 // the cloning stage of each interval with the dynamical stage of the next where it can
-// (k_gather<FUSE>), captures kGraphIntervals of its repeated part into a CUDA graph once
-// (on a private capture stream) and replays it on the caller's stream; the kernels read
+// (k_gather<FUSE>), captures kGraphIntervals of the repeated part of each chain into a CUDA
+// graph once (on a private capture stream) and replays it on the chain's stream; the kernels read
 // the interval number and every other changing quantity from device memory, so replays
 // need no new arguments.  The evolved lattices, K, dK and A are double-buffered by the
 // parity of the interval, so one interval's dynamical stage never overwrites the
@@ -209,7 +209,9 @@ struct pop_batch {
   bool hist_pending = false;
   int graph_hist = -1;                       // hist_on of the captured graph
   float tuned_default_us = 0.0f, tuned_us = 0.0f;
-  cudaGraphExec_t graph = nullptr;
+  // pop_run's captured intervals: one graph per chain, or graph[0] for a batch that does not
+  // fuse; all null or all of the same dt and hist_on
+  cudaGraphExec_t graph[kMaxChains] = {};
   float graph_dt = 0.0f;
   unsigned char* ws = nullptr;
   Batch B{};
@@ -658,6 +660,38 @@ int launch_small(pop_t* h, cudaStream_t st, float dt_f, uint32_t beta0, int64_t 
   return lr;
 }
 
+cudaStream_t chain_stream(pop_t* h, int c) { return c == 0 ? h->stream : h->aux_stream[c - 1]; }
+
+// The auxiliary streams of the chains start after what st holds, and st goes on after them.
+cudaError_t fork_chains(pop_t* h, cudaStream_t st) {
+  if (h->nch == 1) return cudaSuccess;
+  cudaError_t e = cudaEventRecord(h->ev_fork, st);
+  for (int c = 0; c + 1 < h->nch && e == cudaSuccess; ++c) e = cudaStreamWaitEvent(h->aux_stream[c], h->ev_fork, 0);
+  return e;
+}
+cudaError_t join_chains(pop_t* h, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  for (int c = 0; c + 1 < h->nch && e == cudaSuccess; ++c) {
+    e = cudaEventRecord(h->ev_join[c], h->aux_stream[c]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_join[c], 0);
+  }
+  return e;
+}
+
+// One fused interval of chain c on st.
+int launch_chain(pop_t* h, cudaStream_t st, float dt_f, int c, bool after_fused) {
+  return launch_resample_evolve_range(h, st, dt_f, h->chain[c], h->chain_tile[c],
+                                      h->chain_tile[c + 1] - h->chain_tile[c], h->chain_pop[c], h->chain_pop[c + 1],
+                                      after_fused);
+}
+
+void drop_graphs(pop_t* h) {
+  for (cudaGraphExec_t& g : h->graph) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  }
+}
+
 // n fused intervals over the chains: chain 0 on st, the others on the auxiliary
 // streams forked from st and joined back into it, each chain with its own interval
 // counter (copy_chain_counters brings them in line with the batch's counter before and
@@ -665,31 +699,15 @@ int launch_small(pop_t* h, cudaStream_t st, float dt_f, uint32_t beta0, int64_t 
 // was itself a fused one (its tile histograms are pending).
 int run_chains(pop_t* h, cudaStream_t st, float dt_f, int64_t n, bool after_fused) {
   if (n > 0) h->hist_pending = h->B.hist_on != 0;
-  if (h->nch == 1) {
-    int lr = POP_OK;
-    for (int64_t i = 0; i < n && lr == POP_OK; ++i) {
-      if (h->timer_base >= 0) h->timer_interval = h->timer_base + (int)i;
-      lr = launch_resample_evolve_range(h, st, dt_f, h->chain[0], 0, h->lay.ntiles, 0, h->lay.P,
-                                        after_fused || i > 0);
-    }
-    return lr;
-  }
-  if (cudaEventRecord(h->ev_fork, st) != cudaSuccess) return POP_ERR_CUDA;
-  for (int c = 0; c + 1 < h->nch; ++c)
-    if (cudaStreamWaitEvent(h->aux_stream[c], h->ev_fork, 0) != cudaSuccess) return POP_ERR_CUDA;
+  if (fork_chains(h, st) != cudaSuccess) return POP_ERR_CUDA;
   int lr = POP_OK;
   for (int64_t i = 0; i < n && lr == POP_OK; ++i)
     for (int c = 0; c < h->nch && lr == POP_OK; ++c) {
       if (h->timer_base >= 0) h->timer_interval = h->timer_base + (int)i;
-      lr = launch_resample_evolve_range(h, c == 0 ? st : h->aux_stream[c - 1], dt_f, h->chain[c],
-                                        h->chain_tile[c], h->chain_tile[c + 1] - h->chain_tile[c],
-                                        h->chain_pop[c], h->chain_pop[c + 1], after_fused || i > 0);
+      lr = launch_chain(h, c == 0 ? st : h->aux_stream[c - 1], dt_f, c, after_fused || i > 0);
     }
   // the joins are made even after a failed launch, so a capture can end cleanly
-  for (int c = 0; c + 1 < h->nch; ++c)
-    if (cudaEventRecord(h->ev_join[c], h->aux_stream[c]) != cudaSuccess ||
-        cudaStreamWaitEvent(st, h->ev_join[c], 0) != cudaSuccess)
-      return POP_ERR_CUDA;
+  if (join_chains(h, st) != cudaSuccess) return POP_ERR_CUDA;
   return lr;
 }
 
@@ -961,64 +979,74 @@ int pop_run(pop_t* h, double dt, const double* s, int64_t n_intervals) {
     return POP_OK;
   }
   // fused: evolve, then (n - 1) x [weights, gather + next evolve] over the chains, then
-  // weights, gather; otherwise n x [evolve, weights, gather].  The graph holds
+  // weights, gather; otherwise n x [evolve, weights, gather].  A graph holds
   // kGraphIntervals of the repeated part.  The first fused interval follows the
-  // separate dynamical stage, so it runs before the graph, whose intervals all follow
+  // separate dynamical stage, so it runs before the graphs, whose intervals all follow
   // a fused one (with tile histograms, their weights come from those).
   const bool fuse = fusable(h);
   set_hist(h, dt_f);
-  if (fuse) {
-    rc = launch_evolve(h, h->stream, dt_f);
-    if (rc != POP_OK) return rc;
-    POP_CUDA(copy_chain_counters(h, true));
-    if (n_intervals > 1) {
-      rc = run_chains(h, h->stream, dt_f, 1, false);
-      if (rc != POP_OK) return rc;
-    }
-  }
   const int64_t n_rep = fuse ? (n_intervals > 1 ? n_intervals - 2 : 0) : n_intervals;
   const int64_t n_graph = n_rep / kGraphIntervals;
   const int64_t n_rest = n_rep % kGraphIntervals;
-  auto block = [&](cudaStream_t st, int64_t n) {
-    if (fuse) return run_chains(h, st, dt_f, n, true);
+  const int ngr = fuse ? h->nch : 1;
+  // n of the repeated intervals of chain c (all of a batch that does not fuse) on st
+  auto repeat = [&](cudaStream_t st, int c, int64_t n, bool after_fused) {
     int lr = POP_OK;
     for (int64_t i = 0; i < n && lr == POP_OK; ++i) {
-      lr = launch_evolve(h, st, dt_f);
-      if (lr == POP_OK) lr = launch_resample(h, st);
+      if (fuse) {
+        lr = launch_chain(h, st, dt_f, c, after_fused || i > 0);
+      } else {
+        lr = launch_evolve(h, st, dt_f);
+        if (lr == POP_OK) lr = launch_resample(h, st);
+      }
     }
     return lr;
   };
-  if (n_graph > 0 && (h->graph == nullptr || h->graph_dt != dt_f || h->graph_hist != h->B.hist_on)) {
-    if (h->graph != nullptr) {
-      cudaGraphExecDestroy(h->graph);
-      h->graph = nullptr;
-    }
-    cudaGraph_t g = nullptr;
-    POP_CUDA(cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal));
+  if (n_graph > 0 && (h->graph[0] == nullptr || h->graph_dt != dt_f || h->graph_hist != h->B.hist_on)) {
+    drop_graphs(h);
     for (uint64_t& c : h->graph_counts) c = 0;
-    h->count = h->graph_counts;
-    const int lr = block(h->capture_stream, kGraphIntervals);
-    h->count = h->launches;
-    const cudaError_t ec = cudaStreamEndCapture(h->capture_stream, &g);
-    if (lr != POP_OK || ec != cudaSuccess) {
+    for (int c = 0; c < ngr; ++c) {
+      cudaGraph_t g = nullptr;
+      if (cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+        drop_graphs(h);
+        return POP_ERR_CUDA;
+      }
+      h->count = h->graph_counts;
+      const int lr = repeat(h->capture_stream, c, kGraphIntervals, true);
+      h->count = h->launches;
+      const cudaError_t ec = cudaStreamEndCapture(h->capture_stream, &g);
+      const bool ok = lr == POP_OK && ec == cudaSuccess && cudaGraphInstantiate(&h->graph[c], g, 0) == cudaSuccess;
       if (g) cudaGraphDestroy(g);
-      return POP_ERR_CUDA;
-    }
-    const cudaError_t ei = cudaGraphInstantiate(&h->graph, g, 0);
-    cudaGraphDestroy(g);
-    if (ei != cudaSuccess) {
-      h->graph = nullptr;
-      return POP_ERR_CUDA;
+      if (!ok) {
+        h->graph[c] = nullptr;
+        drop_graphs(h);
+        return POP_ERR_CUDA;
+      }
     }
     h->graph_dt = dt_f;
     h->graph_hist = h->B.hist_on;
   }
-  for (int64_t i = 0; i < n_graph; ++i) {
-    POP_CUDA(cudaGraphLaunch(h->graph, h->stream));
-    for (int k = 0; k < POP_NKINDS; ++k) h->launches[k] += h->graph_counts[k];
+  if (fuse) {
+    rc = launch_evolve(h, h->stream, dt_f);
+    if (rc != POP_OK) return rc;
+    POP_CUDA(copy_chain_counters(h, true));
   }
-  if (n_rest > 0) {
-    rc = block(h->stream, n_rest);
+  if (n_intervals > 1 || !fuse) {
+    // each chain runs all of its intervals on its own stream and is joined once, at the end
+    // (one graph of all chains joins and drains them every kGraphIntervals intervals: the
+    // s-sweep 34.3 us per interval, 33.6 so; the study at dt = 10 2239 and 2177)
+    if (fuse) h->hist_pending = h->B.hist_on != 0;
+    POP_CUDA(fork_chains(h, h->stream));
+    if (fuse)
+      for (int c = 0; c < ngr && rc == POP_OK; ++c) rc = repeat(chain_stream(h, c), c, 1, false);
+    for (int64_t i = 0; i < n_graph && rc == POP_OK; ++i) {
+      for (int c = 0; c < ngr && rc == POP_OK; ++c)
+        rc = cuda_status(cudaGraphLaunch(h->graph[c], chain_stream(h, c)));
+      for (int k = 0; k < POP_NKINDS; ++k) h->launches[k] += h->graph_counts[k];
+    }
+    for (int64_t i = 0; i < n_rest && rc == POP_OK; ++i)
+      for (int c = 0; c < ngr && rc == POP_OK; ++c) rc = repeat(chain_stream(h, c), c, 1, true);
+    POP_CUDA(join_chains(h, h->stream));  // also after a failed launch
     if (rc != POP_OK) return rc;
   }
   if (fuse) {
@@ -1473,10 +1501,7 @@ int pop_autotune(pop_t* h, double dt, const double* s, int32_t trials, int32_t* 
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   for (int k = 0; k < POP_NKINDS; ++k) h->launches[k] = launches_before[k];
-  if (h->graph != nullptr) {  // a captured graph holds the old launch configuration
-    cudaGraphExecDestroy(h->graph);
-    h->graph = nullptr;
-  }
+  drop_graphs(h);  // captured graphs hold the old launch configuration
   if (!restore()) return POP_ERR_CUDA;
   if (rc != POP_OK) return rc;
   if (h_evolve_grid) *h_evolve_grid = best;
@@ -1512,10 +1537,7 @@ int pop_set_tuning(pop_t* h, const pop_tuning* cfg) {
   h->gather_threads = cfg->gather_threads;
   h->hist_mode = cfg->hist_mode;
   set_chains(h, cfg->chains);
-  if (h->graph != nullptr) {  // the captured graph holds the old launch configuration
-    cudaGraphExecDestroy(h->graph);
-    h->graph = nullptr;
-  }
+  drop_graphs(h);  // captured graphs hold the old launch configuration
   return POP_OK;
 }
 
@@ -1566,7 +1588,7 @@ const char* pop_strerror(int status) {
 
 void pop_free(pop_t* h) {
   if (h == nullptr) return;
-  if (h->graph) cudaGraphExecDestroy(h->graph);
+  drop_graphs(h);
   if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
   for (int c = 0; c + 1 < kMaxChains; ++c) {
     if (h->aux_stream[c]) cudaStreamDestroy(h->aux_stream[c]);
