@@ -347,8 +347,8 @@ int pop_events(pop_t* pop, uint64_t* h_events);
 
 /*
  * Measurement.  Advances the batch by n_intervals >= 1 intervals with the launches
- * pop_run makes (per_step = 0: the same chains on the same streams, the intervals after
- * the first fused one as one captured graph, as pop_run replays them) or those of
+ * pop_run makes (per_step = 0: the same chains on streams of their own, the intervals
+ * after the first fused one from a captured graph, as pop_run replays them) or those of
  * pop_evolve + pop_resample (per_step = 1: the separate dynamical and cloning stages,
  * launched one by one), in the same order and so with the same results, with a CUDA
  * event recorded before and after every launch on its own stream (an event-record node

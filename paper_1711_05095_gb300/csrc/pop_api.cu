@@ -1099,8 +1099,9 @@ int pop_kernel_times(pop_t* h, double dt, const double* s, int64_t n_intervals, 
     rc = launch_evolve(h, h->stream, dt_f);
     if (rc == POP_OK) rc = total_hops(&hops1);
     if (rc == POP_OK) rc = copy_chain_counters(h, true) == cudaSuccess ? POP_OK : POP_ERR_CUDA;
-    // the first fused interval as pop_run launches it; the others as one captured graph
-    // of run_chains, as pop_run replays them, with event-record nodes around each launch
+    // the first fused interval as pop_run launches it; the others captured and replayed as
+    // pop_run does (there a graph per chain, here one of all chains on their streams), with
+    // event-record nodes around each launch
     if (n_intervals > 1 && rc == POP_OK) {
       h->timer_interval = 1;
       rc = run_chains(h, h->stream, dt_f, 1, false);

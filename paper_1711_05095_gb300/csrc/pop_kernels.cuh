@@ -119,12 +119,12 @@ __device__ __forceinline__ bool bkl_step_pred(uint32_t (&u)[2 * W], float& t, fl
 // no shared counter.  Clones go from global memory to registers and back.
 // Bound by ALU issue.  An interval of 2^22 clones of L = 128, dt = 0.05 by the per-step
 // calls took 288 us with clones staged in shared memory, diverging steps and a counter per
-// block, and 240 us with this form (the cloning stage unchanged); 2^21 clones of L = 50,
-// dt = 1, [iid]: 520 and 462 us.
+// block, and 240 us with this form (the cloning stage unchanged; 205 us with what followed
+// there and in the step); 2^21 clones of L = 50, dt = 1, [iid]: 520 and 462 us.
 // Wide rings: about 250 instructions per step and warp for 32 / G clones, where a whole
 // warp per clone took 225 for one (2^16 clones of L = 256, dt = 0.05, with the cloning
 // stage: 301 us per interval with a warp per clone and a block's own copy of its tile,
-// 51 us now).
+// 46 us now).
 // ---------------------------------------------------------------------------
 constexpr int kEvolveThreads = 128;
 constexpr int kEvolveWarps = kEvolveThreads / 32;
@@ -1644,7 +1644,7 @@ __device__ __forceinline__ float i64_to_float_rn(long long v) {
 // Bound by issue and by the latency of the table loads.  32 populations of 2^14 clones,
 // L = 128, dt = 0.05: 405 us per interval with a block's share of at most a tile (one
 // clone per lane and no refill for this batch: 13.4 of 32 lanes), windows cut from the
-// lattice words and each of the 19 bonds re-rated before and after the hop; 230 us now.
+// lattice words and each of the 19 bonds re-rated before and after the hop; 225 us now.
 #ifndef POP_GUIDE_MIN_BLOCKS
 #define POP_GUIDE_MIN_BLOCKS 8   // 64 registers, 32 warps per SM
 #endif
