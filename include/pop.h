@@ -225,7 +225,7 @@ typedef struct pop_tuning {
  * Choose the launch configuration by timing on this batch's own shape.  Times `trials`
  * launches of the dynamical stage of the first interval for every candidate persistent
  * grid (1 .. the resident blocks per SM, times the SM count); for a batch that fuses,
- * three replays of `trials` fused intervals captured as a CUDA graph (as pop_run runs
+ * eight replays of `trials` fused intervals captured as CUDA graphs (as pop_run runs
  * them) for each fused-kernel form (128 threads with one or two clones per lane, 256
  * threads with one) and each chain split (up to 1, 2, 4, 8), with and without the
  * per-tile activity counts where dt * (largest L) <= 16 and no weights are MODIFIED

@@ -1398,38 +1398,46 @@ int pop_autotune(pop_t* h, double dt, const double* s, int32_t trials, int32_t* 
         set_hist(h, dt_f);
         if (h->nch == last_nch) continue;  // the same split as the smaller want
         last_nch = h->nch;
-        // `trials` fused intervals captured as a graph, as pop_run replays them (launched
-        // one by one, many short chains would be timed by their launch overhead); each
-        // follows a fused interval, as in pop_run's graph
-        cudaGraph_t g = nullptr;
-        cudaGraphExec_t ge = nullptr;
-        if (cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-          rc = POP_ERR_CUDA;
-          break;
-        }
+        // `trials` fused intervals of each chain captured as a graph and replayed on the
+        // chain's stream, joined at the end, as pop_run does (launched one by one, many
+        // short chains would be timed by their launch overhead; joined after every replay,
+        // by their drains); each follows a fused interval, as in pop_run's graphs
+        cudaGraphExec_t ge[kMaxChains] = {};
         uint64_t* const count = h->count;
         h->count = h->graph_counts;  // launches made while tuning are not the batch's
-        const int lc = run_chains(h, h->capture_stream, dt_f, trials, true);
-        h->count = count;
-        const cudaError_t ec = cudaStreamEndCapture(h->capture_stream, &g);
-        if (lc != POP_OK || ec != cudaSuccess || cudaGraphInstantiate(&ge, g, 0) != cudaSuccess) {
+        for (int c = 0; c < h->nch && rc == POP_OK; ++c) {
+          cudaGraph_t g = nullptr;
+          if (cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+            rc = POP_ERR_CUDA;
+            break;
+          }
+          int lc = POP_OK;
+          for (int i = 0; i < trials && lc == POP_OK; ++i) lc = launch_chain(h, h->capture_stream, dt_f, c, true);
+          const cudaError_t ec = cudaStreamEndCapture(h->capture_stream, &g);
+          if (lc != POP_OK || ec != cudaSuccess || cudaGraphInstantiate(&ge[c], g, 0) != cudaSuccess) rc = POP_ERR_CUDA;
           if (g) cudaGraphDestroy(g);
-          rc = POP_ERR_CUDA;
-          break;
         }
-        cudaGraphDestroy(g);
+        h->count = count;
+        constexpr int kReplays = 8;
         float ms = 0.0f;
-        rc = timed([&](bool first) {
-              int lr = POP_OK;
-              if (first) {  // as pop_run: the first fused interval follows the dynamical stage
-                lr = launch_evolve(h, h->stream, dt_f);
-                if (lr == POP_OK && copy_chain_counters(h, true) != cudaSuccess) lr = POP_ERR_CUDA;
-                if (lr == POP_OK) lr = run_chains(h, h->stream, dt_f, 1, false);
-              }
-              if (lr == POP_OK && cudaGraphLaunch(ge, h->stream) != cudaSuccess) lr = POP_ERR_CUDA;
-              return lr;
-            }, 3, &ms);
-        cudaGraphExecDestroy(ge);
+        if (rc == POP_OK)
+          rc = timed([&](bool first) {
+                int lr = POP_OK;
+                if (first) {  // as pop_run: the first fused interval follows the dynamical stage
+                  lr = launch_evolve(h, h->stream, dt_f);
+                  if (lr == POP_OK && copy_chain_counters(h, true) != cudaSuccess) lr = POP_ERR_CUDA;
+                  if (lr == POP_OK) lr = run_chains(h, h->stream, dt_f, 1, false);
+                  return lr;
+                }
+                if (fork_chains(h, h->stream) != cudaSuccess) return (int)POP_ERR_CUDA;
+                for (int r = 0; r < kReplays && lr == POP_OK; ++r)
+                  for (int c = 0; c < h->nch && lr == POP_OK; ++c)
+                    lr = cuda_status(cudaGraphLaunch(ge[c], chain_stream(h, c)));
+                return join_chains(h, h->stream) == cudaSuccess ? lr : (int)POP_ERR_CUDA;
+              }, 1, &ms);
+        for (cudaGraphExec_t& e : ge)
+          if (e) cudaGraphExecDestroy(e);
+        ms /= (float)kReplays;
         ms /= (float)trials;
         if (rc != POP_OK) break;
         if (forms[f][0] == def_threads && forms[f][1] == def_clones && h->nch == def_nch &&
