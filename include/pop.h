@@ -202,7 +202,8 @@ int pop_copy_state(pop_t* pop, int32_t p, uint64_t* h_lattice, int32_t* h_K,
  *                   counts the new clones' activities per tile, so that the next
  *                   interval's tile weight sums and activity histogram come from those
  *                   counts instead of a pass over every clone: 1 on, 0 off, -1 the rule
- *                   (on when every population has more than 64 tiles of 1024 clones and
+ *                   (on when every population has more than 64 tiles of 1024 clones, or the
+ *                   batch more than 4096 and 16 per population on average, and
  *                   dt * (largest L) <= 16, where an activity of 64 or more in one
  *                   interval is very unlikely; such an activity is still handled, by a
  *                   slower pass over the population's clones)

@@ -545,6 +545,12 @@ void set_chains(pop_t* h, int want) {
 void set_hist(pop_t* h, float dt_f) {
   bool many_tiles = true;
   for (const PopDesc& d : h->desc) many_tiles = many_tiles && d.ntiles > kScanTiles;
+  // ... or in a large batch of populations of 16 tiles and more on average: there one scan
+  // block per population keeps up with k_weights, and the pass over every clone is what
+  // costs (8192 tiles, L = 50, dt = 0.1; populations of 8, 16, 32 and 64 tiles: 229, 227, 226
+  // and 227 us per interval with k_weights, 234, 223, 219 and 218 with the counts; 256 uneven
+  // populations, 10911 tiles: 448 and 437.  4096 tiles, L = 100: 182 and 184)
+  many_tiles = many_tiles || (h->lay.ntiles > 4096 && h->lay.ntiles >= 16 * (int64_t)h->lay.P);
   const bool on = fusable(h) && !h->any_mod &&
                   (h->hist_mode == 1 ||
                    (h->hist_mode == -1 && many_tiles && (double)dt_f * h->max_L <= 16.0));
