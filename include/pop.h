@@ -146,7 +146,8 @@ int pop_resample(pop_t* pop);
  * joined back into the handle's stream (the chains share no data; results are the
  * same bit for bit); pop_run_chains gives the split.  A batch that fuses and whose
  * populations hold at most 1024 clones each (and are not many more than the device's SMs)
- * runs up to 1024 intervals per launch instead, one block per population (a launch of the
+ * runs up to 1024 intervals per launch instead (fewer of long intervals: a launch ends
+ * within tens of milliseconds), one block per population (a launch of the
  * kind POP_K_GATHER_EVOLVE); the launch configuration does not apply to it.
  */
 int pop_run(pop_t* pop, double dt, const double* s, int64_t n_intervals);

@@ -648,13 +648,28 @@ int launch_small_form(pop_t* h, cudaStream_t st, float dt_f, uint32_t beta0, int
   return cuda_status(cudaGetLastError());
 }
 
-// n intervals of a batch of one-tile populations, the first of them interval beta0;
-// kSmallIntervals to a launch.
+// Intervals of one launch of k_run_small: 1024, fewer where the interval is long, so that a
+// launch makes some kSmallDraws draws of about a microsecond each and ends within tens of
+// milliseconds.  A ring of N particles on L sites has at most 2 min(N, L - N) active bonds,
+// each with a hop of rate 1 (MODIFIED: e^-s), and a draw makes two hops.
 constexpr int kSmallIntervals = 1024;
+constexpr double kSmallDraws = 32768.0;
+int small_intervals(const pop_t* h, float dt_f) {
+  double rate = 0.0;
+  for (const PopDesc& d : h->desc) {
+    const double r = 2.0 * (double)std::min(d.N, d.L - d.N);
+    rate = std::max(rate, d.modified ? r * std::exp(-d.s) : r);
+  }
+  const double n = kSmallDraws / (0.5 * rate * (double)dt_f + 1.0);
+  return n >= kSmallIntervals ? kSmallIntervals : (n >= 1.0 ? (int)n : 1);
+}
+
+// n intervals of a batch of one-tile populations, the first of them interval beta0.
 int launch_small(pop_t* h, cudaStream_t st, float dt_f, uint32_t beta0, int64_t n) {
   int lr = POP_OK;
-  for (int64_t at = 0; at < n && lr == POP_OK; at += kSmallIntervals) {
-    const int k = (int)std::min<int64_t>(n - at, kSmallIntervals);
+  const int most = small_intervals(h, dt_f);
+  for (int64_t at = 0; at < n && lr == POP_OK; at += most) {
+    const int k = (int)std::min<int64_t>(n - at, most);
     const uint32_t b = beta0 + (uint32_t)at;
     if (h->lay.W == 1)
       lr = h->any_mod ? launch_small_form<1, true>(h, st, dt_f, b, k)

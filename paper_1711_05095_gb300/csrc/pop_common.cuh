@@ -47,7 +47,10 @@ constexpr int kScanTiles = POP_SCAN_TILES; // fused stage: k_tile_scan when ever
 constexpr int kMaxL = 128;                // one clone per lane: W <= 2 words
 constexpr int kMaxLWide = 4096;           // 1 to 16 lanes per clone, 256 sites each
 constexpr int kInvStride = kMaxLWide + 1; // per-population 1/r table stride
-constexpr uint32_t kStepLimit = 1u << 24; // BKL steps per clone per interval
+#ifndef POP_STEP_LIMIT
+#define POP_STEP_LIMIT (1u << 24)
+#endif
+constexpr uint32_t kStepLimit = POP_STEP_LIMIT; // BKL steps per clone per interval
 
 constexpr int32_t kErrRange = -3;
 
@@ -97,6 +100,7 @@ struct PopState {
   unsigned long long T;        // total weight of this interval (k_tile_scan or k_gather)
   unsigned long long pos_m;    // PosScale of T (k_tile_scan)
   int32_t pos_sh;
+  int32_t stuck;               // k_run_small reached the step limit: its later launches run no interval
 };
 
 struct Batch {

@@ -1221,6 +1221,9 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
 // L = 128, dt = 0.1, 13.7 and 40.3.
 // The psi terms need FP64 logarithms, slow on one thread: warp 0 keeps what they are
 // formed from and takes 32 of them at once, one per lane, then adds them in order.
+// An interval that reaches the step limit is the population's last here: the block leaves
+// the loop after it and later launches return at once, so no launch spins through the
+// limit more than once.
 // ---------------------------------------------------------------------------
 constexpr int kSmallThreads = kTile;
 template <int W>
@@ -1255,6 +1258,11 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
   const uint32_t nc = (uint32_t)n;
   const bool valid = tid < n;
   const unsigned long long* const wt = B.wtab + (size_t)p * kKcap;
+  const uint32_t beta_end = beta0 + (uint32_t)n_int;
+  if (st->stuck) {
+    if (p == 0 && tid == 0) *B.beta = beta_end;
+    return;
+  }
   for (int r = tid; r <= kMaxL; r += (int)blockDim.x)  // inv[0] = NaN: see bkl_step_pred
     S.inv[r] = r == 0 ? __int_as_float(0x7fffffff) : (r <= d.L) ? B.inv_rate[(size_t)p * kInvStride + r] : 0.0f;
   build_hop_table<2 * W>(S.hop, (uint32_t)d.L, tid, (int)blockDim.x);
@@ -1295,7 +1303,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
     pad_fill<2 * W>(u, S.hop[kPadEntry]);
     float t = 0.0f, acc = 0.0f;
     h = 0;
-    bool run = valid;
+    bool run = valid, stuck = false;
     for (uint32_t q = 0u; __ballot_sync(0xffffffffu, run) != 0u; ++q) {
       const uint4 d4 = philox4x32_10_rk(make_uint4(q, beta, (uint32_t)tid, kTagEvolve), S.keys);
       const float E1 = neg_ln_u(d4.x, S.logtab), E2 = neg_ln_u(d4.z, S.logtab);
@@ -1303,7 +1311,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
       run = bkl_step_pred<W, MOD>(u, t, acc, S.inv, E2, d4.w, dt_f, h1, kth8, S.hop);
       h += (int)h1 + (int)run;
       if (q + 1u >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
-        if (run) st->err = kErrRange;
+        stuck = run;
         run = false;
       }
     }
@@ -1331,7 +1339,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
         S.amx[wid] = amx;
       }
     }
-    __syncthreads();
+    const bool last = __syncthreads_or(stuck) != 0 || it == n_int - 1;
     mn = __reduce_min_sync(0xffffffffu, lane < nwarps ? S.mn[lane] : INT_MAX);
     mx = __reduce_max_sync(0xffffffffu, lane < nwarps ? S.mx[lane] : INT_MIN);
     if (MOD) {
@@ -1416,7 +1424,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
           S.pend_k[slot] = kref;
         }
       }
-      if (slot == 31 || it == n_int - 1) {
+      if (slot == 31 || last) {
         __syncwarp();
         double term = 0.0;
         if (lane <= slot) {
@@ -1434,8 +1442,13 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
         for (int e = 0; e <= slot; ++e) psi += __shfl_sync(0xffffffffu, term, e);
       }
     }
+    if (stuck) {
+      st->err = kErrRange;
+      st->stuck = 1;
+    }
     __syncthreads();
     cur ^= 1;
+    if (last) break;
   }
   // the population after the last cloning stage, its ancestors and activities
   if (valid) {
@@ -1447,13 +1460,13 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
     store_lat<W>(B.Y, slot, x);
     B.KY[slot] = S.K[cur][a];
     B.anc[slot] = a;
-    B.dKb[(beta0 + (uint32_t)n_int - 1u) & 1u][slot] = h;
+    B.dKb[(beta_end - 1u) & 1u][slot] = h;
   }
   ev = warp_sum_u64(ev);
   if (lane == 0) atomicAdd(&st->events, ev);
   if (tid == 0) {
     st->psi_acc = psi;
-    if (p == 0) *B.beta = beta0 + (uint32_t)n_int;  // beta0 came with the launch: no block reads the counter
+    if (p == 0) *B.beta = beta_end;  // beta0 came with the launch: no block reads the counter
   }
 }
 

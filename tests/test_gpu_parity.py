@@ -791,3 +791,34 @@ def test_positions_too_close_to_a_slot_are_settled_exactly(pg, tmp_path):
                 a.close()
     finally:
         pg._lib, pg.LIB_PATH = saved, path
+
+
+def test_one_tile_launches_are_bounded_and_stop_at_the_step_limit(pg):
+    # 64 active bonds at rate 1 or so for dt = 100: some thousands of draws per clone and
+    # interval, so a launch takes five intervals (32768 draws over 0.5 x 128 x 100 + 1)
+    a = pg.PopulationBatch([dict(L=128, N=64, n_clones=40, seed=70)])
+    a.run(100.0, [0.0], 11)
+    assert a.launch_count()["gather_evolve"] == 3
+    b = pg.PopulationBatch([dict(L=128, N=64, n_clones=40, seed=70)])
+    for _ in range(11):
+        b.evolve(100.0, [0.0])
+        b.resample()
+    for key in ("lattice", "K", "anc", "dK"):
+        assert np.array_equal(a.copy_state(0)[key], b.copy_state(0)[key]), key
+    # intervals that only the step limit ends: the first is reported and the others are not
+    # run, so sixteen take the time of one (and not sixteen times that)
+    import time
+
+    def seconds(n):
+        c = pg.PopulationBatch([dict(L=128, N=1, n_clones=1, seed=71)])
+        t = time.perf_counter()
+        c.run(1e7, [0.0], n)
+        with pytest.raises(pg.PopError) as e:
+            c.events()
+        assert e.value.status == pg.POP_ERR_RANGE
+        t = time.perf_counter() - t
+        c.close()
+        return t
+
+    one = seconds(1)
+    assert seconds(16) < 4.0 * one
