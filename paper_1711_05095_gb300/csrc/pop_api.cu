@@ -641,9 +641,9 @@ int size_small(pop_t* h) {
 }
 
 template <int W, bool MOD>
-int launch_small_form(pop_t* h, cudaStream_t st, float dt_f, uint32_t beta0, int n) {
+int launch_small_form(pop_t* h, cudaStream_t st, float dt_f, int n) {
   kernel_begin(h, st, POP_K_GATHER_EVOLVE);
-  k_run_small<W, MOD><<<(unsigned)h->lay.P, (unsigned)h->small_threads, sizeof(SmallSmem<W>), st>>>(h->B, dt_f, beta0, n);
+  k_run_small<W, MOD><<<(unsigned)h->lay.P, (unsigned)h->small_threads, sizeof(SmallSmem<W>), st>>>(h->B, dt_f, n);
   kernel_end(h, st);
   return cuda_status(cudaGetLastError());
 }
@@ -664,19 +664,18 @@ int small_intervals(const pop_t* h, float dt_f) {
   return n >= kSmallIntervals ? kSmallIntervals : (n >= 1.0 ? (int)n : 1);
 }
 
-// n intervals of a batch of one-tile populations, the first of them interval beta0.
-int launch_small(pop_t* h, cudaStream_t st, float dt_f, uint32_t beta0, int64_t n) {
+// n intervals of a batch of one-tile populations.
+int launch_small(pop_t* h, cudaStream_t st, float dt_f, int64_t n) {
   int lr = POP_OK;
   const int most = small_intervals(h, dt_f);
   for (int64_t at = 0; at < n && lr == POP_OK; at += most) {
     const int k = (int)std::min<int64_t>(n - at, most);
-    const uint32_t b = beta0 + (uint32_t)at;
     if (h->lay.W == 1)
-      lr = h->any_mod ? launch_small_form<1, true>(h, st, dt_f, b, k)
-                      : launch_small_form<1, false>(h, st, dt_f, b, k);
+      lr = h->any_mod ? launch_small_form<1, true>(h, st, dt_f, k)
+                      : launch_small_form<1, false>(h, st, dt_f, k);
     else
-      lr = h->any_mod ? launch_small_form<2, true>(h, st, dt_f, b, k)
-                      : launch_small_form<2, false>(h, st, dt_f, b, k);
+      lr = h->any_mod ? launch_small_form<2, true>(h, st, dt_f, k)
+                      : launch_small_form<2, false>(h, st, dt_f, k);
   }
   return lr;
 }
@@ -993,7 +992,7 @@ int pop_run(pop_t* h, double dt, const double* s, int64_t n_intervals) {
   if (n_intervals == 0) return POP_OK;
   const float dt_f = (float)dt;
   if (run_small(h)) {
-    rc = launch_small(h, h->stream, dt_f, (uint32_t)(h->intervals + 1), n_intervals);
+    rc = launch_small(h, h->stream, dt_f, n_intervals);
     if (rc != POP_OK) return rc;
     h->intervals += n_intervals;
     h->t_obs += (double)n_intervals * dt;
@@ -1114,7 +1113,7 @@ int pop_kernel_times(pop_t* h, double dt, const double* s, int64_t n_intervals, 
   // the same launches, in the same order and on the same streams, as pop_run (or the
   // per-step calls), each interval's launches tagged with its index
   if (small) {
-    rc = launch_small(h, h->stream, dt_f, (uint32_t)(h->intervals + 1), n_intervals);
+    rc = launch_small(h, h->stream, dt_f, n_intervals);
     hops1 = hops0;
   } else if (fuse) {
     rc = launch_evolve(h, h->stream, dt_f);
@@ -1523,7 +1522,7 @@ int pop_autotune(pop_t* h, double dt, const double* s, int32_t trials, int32_t* 
     POP_CUDA(cudaMemcpyAsync(h->B.Xb[0], h->B.Y, lat, cudaMemcpyDeviceToDevice, h->stream));
     POP_CUDA(cudaMemcpyAsync(h->B.KXb[0], h->B.KY, ks, cudaMemcpyDeviceToDevice, h->stream));
     float ms = 0.0f;
-    rc = timed([&](bool) { return launch_small(h, h->stream, dt_f, 1u, trials); }, 3, &ms);
+    rc = timed([&](bool) { return launch_small(h, h->stream, dt_f, trials); }, 3, &ms);
     POP_CUDA(cudaMemcpyAsync(h->B.Y, h->B.Xb[0], lat, cudaMemcpyDeviceToDevice, h->stream));
     POP_CUDA(cudaMemcpyAsync(h->B.KY, h->B.KXb[0], ks, cudaMemcpyDeviceToDevice, h->stream));
     h->tuned_default_us = h->tuned_us = 1e3f * ms / (float)trials;

@@ -1211,7 +1211,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
 
 // ---------------------------------------------------------------------------
 // Whole intervals of populations of at most one tile, one block per population and one
-// clone per thread: n_int intervals, beta0 the first, in one launch.  Lattices and
+// clone per thread: n_int intervals in one launch.  Lattices and
 // cumulative activities stay in shared memory (two buffers; a new clone starts from its
 // ancestor's in the other one, so the gather is part of taking the clone); three barriers
 // per interval.  The arithmetic is that of the separate stages, with the exact j_lo.
@@ -1224,6 +1224,8 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
 // An interval that reaches the step limit is the population's last here: the block leaves
 // the loop after it and later launches return at once, so no launch spins through the
 // limit more than once.
+// The first interval is read from the device's counter, so a captured launch goes on from
+// wherever the population is when it is replayed; the last block to end advances it.
 // ---------------------------------------------------------------------------
 constexpr int kSmallThreads = kTile;
 template <int W>
@@ -1247,7 +1249,7 @@ struct SmallSmem {
 };
 
 template <int W, bool MOD>
-__global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float dt_f, uint32_t beta0, int n_int) {
+__global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float dt_f, int n_int) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmallSmem<W>& S = *reinterpret_cast<SmallSmem<W>*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarps = (int)blockDim.x >> 5;
@@ -1258,9 +1260,15 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
   const uint32_t nc = (uint32_t)n;
   const bool valid = tid < n;
   const unsigned long long* const wt = B.wtab + (size_t)p * kKcap;
-  const uint32_t beta_end = beta0 + (uint32_t)n_int;
+  const uint32_t beta0 = *B.beta, beta_end = beta0 + (uint32_t)n_int;
+  auto leave = [&]() {  // the block's last act: every block has read the counter before
+    if (atomicAdd(&B.st->done, 1u) == gridDim.x - 1u) {
+      B.st->done = 0u;
+      *B.beta = beta_end;
+    }
+  };
   if (st->stuck) {
-    if (p == 0 && tid == 0) *B.beta = beta_end;
+    if (tid == 0) leave();
     return;
   }
   for (int r = tid; r <= kMaxL; r += (int)blockDim.x)  // inv[0] = NaN: see bkl_step_pred
@@ -1466,7 +1474,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
   if (lane == 0) atomicAdd(&st->events, ev);
   if (tid == 0) {
     st->psi_acc = psi;
-    if (p == 0) *B.beta = beta_end;  // beta0 came with the launch: no block reads the counter
+    leave();
   }
 }
 

@@ -822,3 +822,31 @@ def test_one_tile_launches_are_bounded_and_stop_at_the_step_limit(pg):
 
     one = seconds(1)
     assert seconds(16) < 4.0 * one
+
+
+@pytest.mark.parametrize("pops", [[dict(L=30, N=15, n_clones=300, seed=73), dict(L=20, N=10, n_clones=1024, seed=74)],
+                                  [dict(L=30, N=15, n_clones=3000, seed=75)]])
+def test_a_captured_run_goes_on_from_the_population_when_replayed(pg, pops):
+    # the interval number is the device's, not one fixed when the call was captured: two
+    # intervals replayed three times after a first are intervals 2 .. 7, and the next call is
+    # the eighth (one-tile populations, and the fused launches)
+    import torch
+    s = [0.02] * len(pops)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        a = pg.PopulationBatch(pops)
+        a.run(0.1, s, 1)
+        g = torch.cuda.CUDAGraph()
+        st.synchronize()
+        with torch.cuda.graph(g, stream=st):
+            a.run(0.1, s, 2)
+        for _ in range(3):
+            g.replay()
+        a.run(0.1, s, 1)
+        b = pg.PopulationBatch(pops)
+        b.run(0.1, s, 8)
+        st.synchronize()
+    np.testing.assert_array_equal(a.events(), b.events())
+    for p in range(len(pops)):
+        for key in ("lattice", "K", "anc", "dK"):
+            assert np.array_equal(a.copy_state(p)[key], b.copy_state(p)[key]), (p, key)
