@@ -1246,6 +1246,7 @@ struct SmallSmem {
   unsigned int hist[kHistSmem];
   int32_t mn[32], mx[32], amn[32], amx[32];
   uint32_t U[32];                     // [eq] offset words of 32 intervals
+  int32_t stuck;                      // a clone reached the step limit
 };
 
 template <int W, bool MOD>
@@ -1292,7 +1293,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
   }
   S.src[tid] = (uint16_t)tid;
   double psi = 0.0;  // thread 0: the population's accumulator
-  if (tid == 0) psi = st->psi_acc;
+  if (tid == 0) {
+    psi = st->psi_acc;
+    S.stuck = 0;
+  }
   __syncthreads();
   const uint8_t* const kth8 = reinterpret_cast<const uint8_t*>(S.kth8);
   unsigned long long ev = 0ull;
@@ -1311,7 +1315,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
     pad_fill<2 * W>(u, S.hop[kPadEntry]);
     float t = 0.0f, acc = 0.0f;
     h = 0;
-    bool run = valid, stuck = false;
+    bool run = valid;
     for (uint32_t q = 0u; __ballot_sync(0xffffffffu, run) != 0u; ++q) {
       const uint4 d4 = philox4x32_10_rk(make_uint4(q, beta, (uint32_t)tid, kTagEvolve), S.keys);
       const float E1 = neg_ln_u(d4.x, S.logtab), E2 = neg_ln_u(d4.z, S.logtab);
@@ -1319,7 +1323,11 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
       run = bkl_step_pred<W, MOD>(u, t, acc, S.inv, E2, d4.w, dt_f, h1, kth8, S.hop);
       h += (int)h1 + (int)run;
       if (q + 1u >= kStepLimit / 2u) {  // guard: an interval must end; report, never spin
-        stuck = run;
+        if (run) {
+          st->err = kErrRange;
+          st->stuck = 1;
+          S.stuck = 1;
+        }
         run = false;
       }
     }
@@ -1347,7 +1355,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
         S.amx[wid] = amx;
       }
     }
-    const bool last = __syncthreads_or(stuck) != 0 || it == n_int - 1;
+    __syncthreads();
+    const bool stop = S.stuck != 0;  // read between barriers: set before this one at the latest
     mn = __reduce_min_sync(0xffffffffu, lane < nwarps ? S.mn[lane] : INT_MAX);
     mx = __reduce_max_sync(0xffffffffu, lane < nwarps ? S.mx[lane] : INT_MIN);
     if (MOD) {
@@ -1432,7 +1441,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
           S.pend_k[slot] = kref;
         }
       }
-      if (slot == 31 || last) {
+      if (slot == 31 || it == n_int - 1) {
         __syncwarp();
         double term = 0.0;
         if (lane <= slot) {
@@ -1450,13 +1459,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_run_small(Batch B, float d
         for (int e = 0; e <= slot; ++e) psi += __shfl_sync(0xffffffffu, term, e);
       }
     }
-    if (stuck) {
-      st->err = kErrRange;
-      st->stuck = 1;
-    }
     __syncthreads();
     cur ^= 1;
-    if (last) break;
+    if (stop) break;
   }
   // the population after the last cloning stage, its ancestors and activities
   if (valid) {
