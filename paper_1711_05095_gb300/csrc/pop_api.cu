@@ -378,14 +378,50 @@ EvolveKernel evolve_kernel_of(const pop_t* h) {
   }
 }
 
-EvolveKernel evolve_kernel(const pop_t* h) {
+// The largest rate of a clone: a ring of N particles on L sites has at most 2 min(N, L - N)
+// active bonds, each with hops of rate 1 (MODIFIED: e^-s).
+double largest_rate(const pop_t* h) {
+  double rate = 0.0;
+  for (const PopDesc& d : h->desc) {
+    const double r = 2.0 * (double)std::min(d.N, d.L - d.N);
+    rate = std::max(rate, d.modified ? r * std::exp(-d.s) : r);
+  }
+  return rate;
+}
+
+// Whether the hops of a warp's share may not fit 32 bits: they are at most a Poisson number
+// of mean share * rate * dt, which does not reach 2^32 from a mean below 2^30 (the exponent
+// of its probability is -2^30 (4 ln 4 - 3)).  From about 2^23 hops per clone on, time in FP32
+// may stand still and hops no longer follow that law.
+bool many_hops(const pop_t* h, float dt_f) {
+  const double share = (double)(h->B.unit_q + 1) * (32 / evolve_lanes(h));
+  const double hops = largest_rate(h) * (double)dt_f;
+  return !(hops < 1048576.0 && share * hops < 1073741824.0);
+}
+
+// Counting in 64 bits: for MODIFIED populations and plain ones (whose A is not read), and
+// for rings that fill their words and others.
+EvolveKernel evolve_kernel_count64(const pop_t* h) {
+  if (h->lay.W == 1) return k_evolve<2, 1, true, false, true>;
+  if (h->lay.W == 2) return k_evolve<4, 1, true, false, true>;
+  switch (evolve_lanes(h)) {
+    case 1: return k_evolve<8, 1, true, false, true>;
+    case 2: return k_evolve<8, 2, true, false, true>;
+    case 4: return k_evolve<8, 4, true, false, true>;
+    case 8: return k_evolve<8, 8, true, false, true>;
+    default: return k_evolve<8, 16, true, false, true>;
+  }
+}
+
+EvolveKernel evolve_kernel(const pop_t* h, float dt_f) {
   if (h->guided) return h->lay.W == 1 ? k_evolve_guided<1> : k_evolve_guided<2>;
+  if (many_hops(h, dt_f)) return evolve_kernel_count64(h);
   return h->any_mod ? evolve_kernel_of<true>(h) : evolve_kernel_of<false>(h);
 }
 
 int launch_evolve(pop_t* h, cudaStream_t st, float dt_f) {
   kernel_begin(h, st, POP_K_EVOLVE);
-  evolve_kernel(h)<<<(unsigned)h->evolve_grid, kEvolveThreads, 0, st>>>(h->B, dt_f);
+  evolve_kernel(h, dt_f)<<<(unsigned)h->evolve_grid, kEvolveThreads, 0, st>>>(h->B, dt_f);
   kernel_end(h, st);
   return cuda_status(cudaGetLastError());
 }
@@ -602,7 +638,7 @@ void set_evolve_grid(pop_t* h, int grid) {
 // As many blocks as fit on the device at once (or as there are chunks for).
 int size_evolve_grid(pop_t* h) {
   int per_sm = 0, sms = 0;
-  POP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evolve_kernel(h), kEvolveThreads, 0));
+  POP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evolve_kernel(h, 0.0f), kEvolveThreads, 0));
   POP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
   set_evolve_grid(h, (per_sm < 1 ? 1 : per_sm) * sms);
   h->evolve_grid_cap = h->evolve_grid;
@@ -649,18 +685,12 @@ int launch_small_form(pop_t* h, cudaStream_t st, float dt_f, int n) {
 }
 
 // Intervals of one launch of k_run_small: 1024, fewer where the interval is long, so that a
-// launch makes some kSmallDraws draws of about a microsecond each and ends within tens of
-// milliseconds.  A ring of N particles on L sites has at most 2 min(N, L - N) active bonds,
-// each with a hop of rate 1 (MODIFIED: e^-s), and a draw makes two hops.
+// launch makes some kSmallDraws draws (two hops each) of about a microsecond and ends
+// within tens of milliseconds.
 constexpr int kSmallIntervals = 1024;
 constexpr double kSmallDraws = 32768.0;
 int small_intervals(const pop_t* h, float dt_f) {
-  double rate = 0.0;
-  for (const PopDesc& d : h->desc) {
-    const double r = 2.0 * (double)std::min(d.N, d.L - d.N);
-    rate = std::max(rate, d.modified ? r * std::exp(-d.s) : r);
-  }
-  const double n = kSmallDraws / (0.5 * rate * (double)dt_f + 1.0);
+  const double n = kSmallDraws / (0.5 * largest_rate(h) * (double)dt_f + 1.0);
   return n >= kSmallIntervals ? kSmallIntervals : (n >= 1.0 ? (int)n : 1);
 }
 

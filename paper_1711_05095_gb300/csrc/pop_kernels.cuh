@@ -2,6 +2,8 @@
 // interval structure, the data layout and the arithmetic they share.
 #pragma once
 
+#include <type_traits>
+
 #include "pop_common.cuh"
 
 namespace popgpu {
@@ -212,9 +214,13 @@ __device__ __forceinline__ bool wide_step_pred(uint32_t (&u)[8], float& t, float
 }
 
 // FULL: every ring fills the words (L = 32 NW), so there is no padding to keep.
-template <int NW, int G, bool MOD, bool FULL>
+// COUNT64: the hops of a lane's share are counted in 64 bits, where they may not fit 32 (the
+// host's rule; beside the steps that costs a register, 2.5 % of the [iid] study's time, and
+// so did a second count behind the loop).
+template <int NW, int G, bool MOD, bool FULL, bool COUNT64 = false>
 __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_BLOCKS) k_evolve(Batch B, float dt_f) {
   static_assert(NW == 8 || G == 1, "one lane for up to four words");
+  using Count = std::conditional_t<COUNT64, unsigned long long, unsigned int>;
   constexpr int W64 = NW / 2;                        // 64-bit words per lane
   __shared__ float2 s_tab[64];
   __shared__ __align__(16) uint32_t s_kth8[512];
@@ -263,7 +269,7 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
     uint32_t q = 0u, u[NW];
     float t = 0.0f, acc = 0.0f;
     int hmin = INT_MAX, hmax = INT_MIN, amin = INT_MAX, amax = INT_MIN;
-    unsigned int ev = 0u;
+    Count ev = 0;
 #pragma unroll
     for (int j = 0; j < NW; ++j) u[j] = 0u;
     for (;;) {
@@ -338,14 +344,15 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
           }
           hmin = min(hmin, h);
           hmax = max(hmax, h);
-          ev += (unsigned int)h;
+          ev += (Count)h;
         }
         cl = -1;
       }
     }
     hmin = __reduce_min_sync(0xffffffffu, hmin);
     hmax = __reduce_max_sync(0xffffffffu, hmax);
-    ev = __reduce_add_sync(0xffffffffu, ev);
+    if constexpr (COUNT64) ev = warp_sum_u64(ev);
+    else ev = __reduce_add_sync(0xffffffffu, ev);
     if (MOD) {
       amin = __reduce_min_sync(0xffffffffu, amin);
       amax = __reduce_max_sync(0xffffffffu, amax);
@@ -1759,7 +1766,7 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
     unsigned long long R = 0ull;
     float t = 0.0f, a_r = 0.0f, a_h = 0.0f;
     int hmin = INT_MAX, hmax = INT_MIN, xmin = INT_MAX, xmax = INT_MIN;
-    unsigned int ev = 0u;
+    unsigned long long ev = 0ull;
 #pragma unroll
     for (int j = 0; j < NW; ++j) u[j] = 0u;
     for (;;) {
@@ -1898,7 +1905,7 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
           B.Ab[par][slot] = X;
           hmin = min(hmin, h);
           hmax = max(hmax, h);
-          ev += (unsigned int)h;
+          ev += (unsigned long long)h;
           xmin = min(xmin, float_order(X));
           xmax = max(xmax, float_order(X));
           cl = -1;
@@ -1908,14 +1915,14 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
     }
     hmin = __reduce_min_sync(0xffffffffu, hmin);
     hmax = __reduce_max_sync(0xffffffffu, hmax);
-    ev = __reduce_add_sync(0xffffffffu, ev);
+    ev = warp_sum_u64(ev);
     xmin = __reduce_min_sync(0xffffffffu, xmin);
     xmax = __reduce_max_sync(0xffffffffu, xmax);
     if (lane == 0 && n > 0) {
       PopState* st = B.st + p;
       atomicMin(&st->dk_min[par], hmin);
       atomicMax(&st->dk_max[par], hmax);
-      atomicAdd(&st->events, (unsigned long long)ev);
+      atomicAdd(&st->events, ev);
       atomicMin(&st->a_min[par], xmin);
       atomicMax(&st->a_max[par], xmax);
     }

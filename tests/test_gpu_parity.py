@@ -850,3 +850,32 @@ def test_a_captured_run_goes_on_from_the_population_when_replayed(pg, pops):
     for p in range(len(pops)):
         for key in ("lattice", "K", "anc", "dK"):
             assert np.array_equal(a.copy_state(p)[key], b.copy_state(p)[key]), (p, key)
+
+
+def test_events_of_a_share_of_more_than_2_to_the_32_hops(pg):
+    # one block: 32768 clones to a warp, some 139800 hops each (4300 x 32.5), 4.6e9 > 2^32
+    b = pg.PopulationBatch([dict(L=64, N=32, n_clones=2 ** 17, seed=76)])
+    b.set_tuning(evolve_grid=1)
+    b.evolve(4300.0, [0.0])
+    hops = int(b.copy_state(0)["dK"].astype(np.int64).sum())
+    assert hops > 4 * 2 ** 32
+    assert int(b.events()[0]) == hops
+
+
+@pytest.mark.parametrize("L", [40, 64, 100, 200, 400, 1000, 2000, 3000])
+@pytest.mark.parametrize("mode", [0, MOD])
+def test_long_intervals_counted_in_64_bits_match_oracle(pg, L, mode):
+    # from 2^20 hops per clone on the dynamical stage counts in 64 bits, in kernels of its own
+    # (two active bonds for dt = 530000; e^-s nearly 1); a short ring beside the others
+    pops = [dict(L=L, N=1, n_clones=5 if L <= 128 else 1, seed=400 + L, weight_mode=mode), dict(L=9, N=1, n_clones=2, seed=401 + L)]
+    s = [-1e-6, 0.0]
+    b = pg.PopulationBatch(pops)
+    b.evolve(530000.0, s)
+    events = b.events()
+    for p, q in enumerate(pops):
+        o = oracle.Population(q["L"], q["N"], q["n_clones"], q["seed"], modified=q.get("weight_mode", 0) == MOD)
+        o.evolve(530000.0, s[p])
+        g = b.copy_state(p)
+        assert np.array_equal(g["lattice"], oracle.sites_to_words(o.sites, b.W)), p
+        assert np.array_equal(g["K"], o.K) and np.array_equal(g["dK"], o.dK), p
+        assert int(events[p]) == int(o.dK.astype(np.int64).sum()), p
