@@ -199,11 +199,17 @@ __global__ void __launch_bounds__(256) k_forward(Work w) {
 // one of 4096 bins per four windows and the bins are folded onto the 512 patterns at the
 // end.  (The last L mod 4 windows use the 512-entry tables.)  Shared-memory FP32 adds are
 // compare-and-swap loops, so the bins are integers: d is held as a 31-bit fixed-point
-// number relative to the largest |d| of the block's chunk, split into 16 low bits
-// (unsigned) and the rest (signed), one native 32-bit add each.  A chunk has at most
-// kChunkCfg configurations of at most 32 groups, so no bin leaves 32 bits; its sums are
-// exact, and a term's rounding is at most 2^-31 of the largest term, below that of an
-// FP32 sum.  Non-finite d take a plain FP64 path that gives the same infinities and NaN.
+// number, split into 16 low bits (unsigned) and the rest (signed), one native 32-bit add
+// each.  A chunk has at most kChunkCfg configurations of at most 32 groups, so no bin
+// leaves 32 bits.  The scale takes the largest |d| of the block's chunk into [2^29, 2^30);
+// the terms of its binary order and the six below keep 24 bits or more, as in an FP32 sum,
+// and are added; those below them are left to a pass of their own, scaled by the largest
+// of them, and so on: a network near its start needs one pass, one that is sure of many
+// configurations several (2^18 configurations of L = 128, the initial network's last layer
+// 10 and 30 times as large: 88 and 95 us per gradient, 82 as it is; in one pass, 83 for all
+// of them, small terms beside a large one lost their digits).  So a term's rounding is at most 2^-24 of
+// it, and the sums of a pass are exact.  Non-finite d take a plain FP64 path that gives the
+// same infinities and NaN.
 // A gradient of 16384 configurations of L = 128, its read-back included: 151 us with a
 // thread per configuration and FP32 adds per window (55 us of it here) in nine launches,
 // 56 us now; of 2^20: 493 us, now 108.
@@ -219,7 +225,7 @@ struct LogitsSmem {
   uint32_t lo[kBins + kPat];
   int32_t hi[kBins + kPat];
   double red[2][kLT / 32];
-  uint32_t mx[kLT / 32];
+  uint32_t mx[2][kLT / 32];
 };
 
 // Bits t = 0 .. L + 10 of e are the sites t - 4 (mod L) of a configuration, so window i
@@ -314,25 +320,52 @@ __global__ void __launch_bounds__(kLT) k_logits(Work w, const unsigned long long
       for (int k = 0; k < kCfg; ++k) d[k] = k == r ? dv : d[k];
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
-    if (lane == 0) S.mx[wid] = mx;
+    if (lane == 0) S.mx[0][wid] = mx;
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < kLT / 32; ++q) mx = max(mx, S.mx[q]);
-    const bool finite = mx < 0x7f800000u;
-    // the scale 2^x that takes the largest |d| into [2^29, 2^30)
-    const int x = 29 - max((int)(mx >> 23) - 127, -90);
-    const float scale = __uint_as_float((uint32_t)(x + 127) << 23);
+    for (int q = 0; q < kLT / 32; ++q) mx = max(mx, S.mx[0][q]);
+    if (mx >= 0x7f800000u) {  // not finite
 #pragma unroll 1
-    for (int r = 0; r < kCfg; ++r) {
-      const int64_t j = j0 + r * kLT + tid;
-      if (j >= j_end) break;
-      float dv = 0.f;
+      for (int r = 0; r < kCfg; ++r) {
+        const int64_t j = j0 + r * kLT + tid;
+        if (j >= j_end) break;
+        float dv = 0.f;
 #pragma unroll
-      for (int k = 0; k < kCfg; ++k) dv = k == r ? d[k] : dv;
-      uint32_t e[5];
-      extend(lat, W, L, j, e);
-      if (finite) {
-        const int v = __float2int_rn(dv * scale);
+        for (int k = 0; k < kCfg; ++k) dv = k == r ? d[k] : dv;
+        uint32_t e[5];
+        extend(lat, W, L, j, e);
+        for (int i = 0; i < L; ++i) atomicAdd(&w.dPhi[window9(e, i)], (double)dv * (0.5 / (double)n));
+      }
+      __syncthreads();
+      continue;
+    }
+    uint32_t top = 0x7f800000u;  // the terms from here on have been added
+    for (int pass = 1;; ++pass) {
+      // mx: the largest |d| below top; this pass adds the terms of its binary order and the
+      // six below, in units of 2^-x
+      const int order = max((int)(mx >> 23), 1);
+      const uint32_t low = order > 7 ? (uint32_t)(order - 6) << 23 : 0u;
+      const int x = 29 + 127 - order;  // 21 .. 155
+      const float scale1 = __uint_as_float((uint32_t)((x >> 1) + 127) << 23);
+      const float scale2 = __uint_as_float((uint32_t)(x - (x >> 1) + 127) << 23);
+      uint32_t rest = 0u;
+#pragma unroll
+      for (int k = 0; k < kCfg; ++k) {
+        const uint32_t m = __float_as_uint(fabsf(d[k]));
+        rest = m < low ? max(rest, m) : rest;
+      }
+#pragma unroll 1
+      for (int r = 0; r < kCfg; ++r) {
+        const int64_t j = j0 + r * kLT + tid;
+        if (j >= j_end) break;
+        float dv = 0.f;
+#pragma unroll
+        for (int k = 0; k < kCfg; ++k) dv = k == r ? d[k] : dv;
+        const uint32_t m = __float_as_uint(fabsf(dv));
+        if (m < low || m >= top) continue;
+        uint32_t e[5];
+        extend(lat, W, L, j, e);
+        const int v = __float2int_rn(dv * scale1 * scale2);
         const uint32_t vl = (uint32_t)v & 0xffffu;
         const int vh = v >> 16;
 #pragma unroll
@@ -347,12 +380,14 @@ __global__ void __launch_bounds__(kLT) k_logits(Work w, const unsigned long long
           atomicAdd(&S.lo[b], vl);
           atomicAdd(&S.hi[b], vh);
         }
-      } else {
-        for (int i = 0; i < L; ++i) atomicAdd(&w.dPhi[window9(e, i)], (double)dv * (0.5 / (double)n));
       }
-    }
-    __syncthreads();
-    if (finite) {
+      rest = __reduce_max_sync(0xffffffffu, rest);
+      if (lane == 0) S.mx[pass & 1][wid] = rest;
+      __syncthreads();
+      mx = 0u;
+#pragma unroll
+      for (int q = 0; q < kLT / 32; ++q) mx = max(mx, S.mx[pass & 1][q]);
+      top = low;
       // window o (0 .. 3) of the group q is (q >> o) & 511
       const double unit = exp2((double)-x);
 #pragma unroll 1
@@ -389,15 +424,15 @@ __global__ void __launch_bounds__(kLT) k_logits(Work w, const unsigned long long
         if (k == 0) acc[0] += add;
         else acc[1] += add;
       }
-      if (j0 + kChunkCfg < j_end) {  // the next chunk starts from empty bins
-        __syncthreads();
-        for (int b = tid; b < kBins + kPat; b += kLT) {
-          S.lo[b] = 0u;
-          S.hi[b] = 0;
-        }
+      if (mx == 0u && j0 + kChunkCfg >= j_end) break;
+      __syncthreads();  // the next pass or chunk starts from empty bins
+      for (int b = tid; b < kBins + kPat; b += kLT) {
+        S.lo[b] = 0u;
+        S.hi[b] = 0;
       }
+      __syncthreads();
+      if (mx == 0u) break;
     }
-    __syncthreads();
   }
   if (acc[0] != 0.0) atomicAdd(&w.dPhi[tid], acc[0] * (0.5 / (double)n));
   if (acc[1] != 0.0) atomicAdd(&w.dPhi[tid + kLT], acc[1] * (0.5 / (double)n));

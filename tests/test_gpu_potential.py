@@ -159,3 +159,26 @@ def test_gradient_of_a_network_that_is_not_finite(env):
     loss, grad = tr.grad(torch.from_numpy(words.view(np.int64)).cuda(), torch.from_numpy(labels).cuda(), 20)
     assert np.isnan(loss) and np.isnan(grad[-1]) and np.isnan(grad[128 * 9 + 128:128 * 9 + 128 + 128 * 128]).all()
     tr.close()
+
+
+@pytest.mark.parametrize("L,n,c", [(20, 300, -5.0), (20, 300, -14.0), (30, 3000, -23.0), (70, 200, -23.0), (128, 300, -60.0)])
+def test_gradient_of_confident_configurations_beside_a_wrong_one(env, L, n, c):
+    # one empty ring (only window 0, which has no input set and so no part in dW1) that the
+    # network takes for the wrong class, d = -1, beside configurations it is sure of, d about
+    # e^c: every element of the gradient within the FP32 / BF16 tolerance, those that only
+    # the small terms reach included
+    torch, pg, potential = env
+    theta = potential.init_params(13)
+    theta[-1] = c
+    words, labels = batch(n, L, 200 + L)
+    labels[:] = 0
+    words[7], labels[7] = 0, 1
+    tr = potential.Trainer(theta=theta)
+    loss, grad = tr.grad(torch.from_numpy(words.view(np.int64)).cuda(), torch.from_numpy(labels).cuda(), L)
+    want_loss, want_grad = mlp.loss_and_grad(theta, words, labels, L, bf=True)
+    tol_loss, tol = mlp.grad_tolerance(theta, words, labels, L)
+    assert abs(loss - want_loss) <= tol_loss
+    assert np.all(np.abs(grad - want_grad) <= tol)
+    # the bound tells a lost term: most of dW1 is several times its tolerance
+    assert np.median(np.abs(want_grad[:128 * 9]) / tol[:128 * 9]) > 5.0
+    tr.close()
