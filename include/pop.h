@@ -190,11 +190,11 @@ int pop_copy_state(pop_t* pop, int32_t p, uint64_t* h_lattice, int32_t* h_K,
  * counts).  Every choice changes only speed, never a result:
  *   evolve_grid     persistent grid of the separate dynamical stage (the first interval
  *                   of a fused run; every interval of a batch that does not fuse)
- *   fuse_threads    threads per block of the fused cloning + dynamical stage: 128 or 256
- *                   (pop_init's 128 stands for 256 in a batch whose tiles are resident all
- *                   at once, until pop_set_tuning or pop_autotune sets the configuration)
+ *   fuse_threads    threads per block of the fused cloning + dynamical stage: 128, 256, or
+ *                   0 for the rule (pop_init's: 256 for a batch whose tiles are resident
+ *                   all at once and one clone to a lane, else 128)
  *   fuse_clones     clones each lane of the fused stage advances together: 1 or 2
- *                   (2 only with 128 threads)
+ *                   (2 not with fuse_threads 256)
  *   chains          chains of pop_run (1 .. 8; the split actually used may have fewer,
  *                   see pop_run_chains)
  *   gather_threads  threads per block of the separate cloning stage: 128, 256, or 0 for

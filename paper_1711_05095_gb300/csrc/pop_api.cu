@@ -197,9 +197,8 @@ struct pop_batch {
   cudaEvent_t ev_join[kMaxChains - 1] = {};
   Batch chain[kMaxChains]{};                 // the batch with each chain's own interval counter
   // launch configuration (rule-based at pop_init; pop_autotune or pop_set_tuning may change it)
-  int fuse_threads = 128;                    // fused kernel: threads per block (128 or 256)
-  bool one_wave = false;                     // 256 threads in place of the default 128 (size_chains) until
-                                             // pop_set_tuning or pop_autotune sets the configuration
+  int fuse_threads = 0;                      // fused kernel: threads per block, 128, 256, or 0 for the rule
+  bool one_wave = false;                     // the rule's 256 threads instead of 128 (size_chains)
   int fuse_clones = kFuseClones;             // fused kernel: clones per lane (1 or 2)
   int gather_threads = 0;                    // separate cloning stage: 128, 256, or 0 for the rule
   int hist_mode = -1;                        // tile activity histograms: 1 on, 0 off, -1 the rule
@@ -491,9 +490,14 @@ int launch_resample(pop_t* h, cudaStream_t st) {
 
 // The fused kernel in the handle's configuration: 128 threads per block with one or two
 // clones per lane, or 256 threads with one.
+int fused_threads(const pop_t* h) {
+  if (h->fuse_threads != 0) return h->fuse_threads;
+  return h->one_wave && h->fuse_clones == 1 ? 256 : 128;
+}
+
 template <int W, bool MOD, bool SCAN, bool FULL>
 void launch_fused_form(pop_t* h, unsigned grid, cudaStream_t st, const Batch& Bx, float dt_f, int tile0) {
-  if (h->fuse_threads == 256 || h->one_wave)
+  if (fused_threads(h) == 256)
     k_gather<W, 256, true, MOD, SCAN, 1, FULL><<<grid, 256, 0, st>>>(Bx, dt_f, tile0);
   else if (h->fuse_clones == 2)
     k_gather<W, 128, true, MOD, SCAN, 2, FULL><<<grid, 128, 0, st>>>(Bx, dt_f, tile0);
@@ -1429,14 +1433,13 @@ int pop_autotune(pop_t* h, double dt, const double* s, int32_t trials, int32_t* 
   if (rc == POP_OK && fusable(h) && !run_small(h)) {
     const int forms[3][2] = {{128, 1}, {128, 2}, {256, 1}};
     const int wants[4] = {1, 2, 4, 8};
-    const int def_threads = h->one_wave ? 256 : h->fuse_threads, def_clones = h->fuse_clones, def_nch = h->nch;
+    const int def_threads = fused_threads(h), def_clones = h->fuse_clones, def_nch = h->nch;
     const int def_hist = h->hist_mode;
     const bool def_on = h->B.hist_on != 0;
     const bool hist_ok = !h->any_mod && (double)dt_f * h->max_L <= 16.0;
     int bt = def_threads, bc = def_clones, bw = def_nch, bh = def_hist;
     float bms = 1e30f, def_ms = 0.0f;
     int last_nch = -1;
-    h->one_wave = false;
     for (int hm = 0; hm < (hist_ok ? 2 : 1) && rc == POP_OK; ++hm)
     for (int f = 0; f < 3 && rc == POP_OK; ++f) {
       last_nch = -1;
@@ -1582,7 +1585,7 @@ int pop_get_tuning(pop_t* h, pop_tuning* out) {
 
 int pop_set_tuning(pop_t* h, const pop_tuning* cfg) {
   if (h == nullptr || cfg == nullptr) return POP_ERR_ARG;
-  if (cfg->evolve_grid < 1 || (cfg->fuse_threads != 128 && cfg->fuse_threads != 256) ||
+  if (cfg->evolve_grid < 1 || (cfg->fuse_threads != 0 && cfg->fuse_threads != 128 && cfg->fuse_threads != 256) ||
       (cfg->fuse_clones != 1 && cfg->fuse_clones != 2) || (cfg->fuse_threads == 256 && cfg->fuse_clones != 1) ||
       cfg->chains < 1 || cfg->chains > kMaxChains ||
       (cfg->gather_threads != 0 && cfg->gather_threads != 128 && cfg->gather_threads != 256) ||
@@ -1590,7 +1593,6 @@ int pop_set_tuning(pop_t* h, const pop_tuning* cfg) {
     return POP_ERR_ARG;
   if (h->phase != kReady) return POP_ERR_STATE;
   set_evolve_grid(h, cfg->evolve_grid);
-  h->one_wave = false;
   h->fuse_threads = cfg->fuse_threads;
   h->fuse_clones = cfg->fuse_clones;
   h->gather_threads = cfg->gather_threads;

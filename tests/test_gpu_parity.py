@@ -879,3 +879,31 @@ def test_long_intervals_counted_in_64_bits_match_oracle(pg, L, mode):
         assert np.array_equal(g["lattice"], oracle.sites_to_words(o.sites, b.W)), p
         assert np.array_equal(g["K"], o.K) and np.array_equal(g["dK"], o.dK), p
         assert int(events[p]) == int(o.dK.astype(np.int64).sum()), p
+
+
+def test_setting_one_tuned_parameter_leaves_the_others(pg):
+    # the fused kernel's form stays the rule's (fuse_threads 0: 256 threads in a batch within
+    # one wave) until it is set itself, and can be given back to the rule
+    pops = [dict(L=50, N=25, n_clones=5000, seed=31), dict(L=40, N=20, n_clones=3000, seed=32)]
+    s = [0.01, 0.02]
+    a = pg.PopulationBatch(pops)
+    before = a.get_tuning()
+    assert before["fuse_threads"] == 0
+    a.set_tuning()
+    assert a.get_tuning() == before
+    b = pg.PopulationBatch(pops)
+    b.run(0.1, s, 5)
+    for cfg in (dict(chains=1), dict(hist_mode=0), dict(evolve_grid=5), dict(gather_threads=256), dict(fuse_clones=2),
+                dict(fuse_threads=128), dict(fuse_threads=128, fuse_clones=2), dict(fuse_threads=256, fuse_clones=1)):
+        c = pg.PopulationBatch(pops)
+        c.set_tuning(**cfg)
+        got = c.get_tuning()
+        assert got == dict(before, **cfg), cfg
+        c.run(0.1, s, 5)
+        for p in range(2):
+            for key in ("lattice", "K", "anc", "dK"):
+                assert np.array_equal(b.copy_state(p)[key], c.copy_state(p)[key]), (cfg, p, key)
+        c.set_tuning(**{k: before[k] for k in cfg})
+        assert c.get_tuning() == before
+    with pytest.raises(pg.PopError):
+        a.set_tuning(fuse_threads=256, fuse_clones=2)
