@@ -777,6 +777,15 @@ cudaError_t copy_chain_counters(pop_t* h, bool to_chains) {
   return cudaSuccess;
 }
 
+// The density mode's kernel: by sites, by particles, or by what suits each population.
+template <int W>
+auto density_kernel(const pop_t* h) -> void (*)(Batch, const float2*, double*) {
+  int few = 0;
+  for (const PopDesc& d : h->desc) few += density_by_particles(d.N, h->lay.W) ? 1 : 0;
+  if (few == 0) return k_density<W, kBySites>;
+  return few == h->lay.P ? k_density<W, kByParticles> : k_density<W, kByPopulation>;
+}
+
 int check_device_errors(pop_t* h, std::vector<PopState>* out) {
   std::vector<PopState> st((size_t)h->lay.P);
   POP_CUDA(cudaMemcpyAsync(st.data(), h->ws + h->lay.o_st, st.size() * sizeof(PopState),
@@ -1620,9 +1629,9 @@ int pop_density_mode(pop_t* h, int32_t n, double* h_mean) {
                            h->stream));
   const unsigned grid = (unsigned)h->lay.ntiles;
   h->launches[POP_K_OTHER] += 1;
-  if (h->lay.W == 1) k_density<1><<<grid, kThreads, 0, h->stream>>>(h->B, d_cs, d_tacc);
-  else if (h->lay.W == 2) k_density<2><<<grid, kThreads, 0, h->stream>>>(h->B, d_cs, d_tacc);
-  else k_density<0><<<grid, kThreads, 0, h->stream>>>(h->B, d_cs, d_tacc);
+  if (h->lay.W == 1) density_kernel<1>(h)<<<grid, kThreads, 0, h->stream>>>(h->B, d_cs, d_tacc);
+  else if (h->lay.W == 2) density_kernel<2>(h)<<<grid, kThreads, 0, h->stream>>>(h->B, d_cs, d_tacc);
+  else density_kernel<0>(h)<<<grid, kThreads, 0, h->stream>>>(h->B, d_cs, d_tacc);
   POP_CUDA(cudaGetLastError());
   std::vector<double> tacc((size_t)h->lay.ntiles);
   POP_CUDA(cudaMemcpyAsync(tacc.data(), d_tacc, tacc.size() * sizeof(double),

@@ -1961,9 +1961,18 @@ __global__ void __launch_bounds__(kThreads) k_copy_wide(Batch B) {
 // FP64 sum over its clones.
 // Every site in turn, with the additions under the site's bit and its pair of values read
 // from shared memory by all lanes at once: about five instructions a site without
-// divergence, where a loop over each clone's set bits with a table load for each took some
-// 28 per particle (2^21 clones of L = 128: 154 us).
-template <int W>
+// divergence, where a loop over each clone's set bits with a table load for each takes some
+// 28 per particle (2^21 clones of L = 128, N = 64: 32 us, and 151 us by particles).
+// Populations of few particles are summed by particles, in the same order: with N = 4 of
+// 128 sites 23 us (32 by sites), 4 of 256 (2^19 clones) 13 (19), 8 of 4096 (2^15) 83 (94).
+// The line, N <= 4 + words but at most 8: both forms take the same at 6 particles in one
+// word, 8 in two, 10 in four, 11 in eight, 7 in sixteen, 13 in thirty-two.  A batch with
+// populations on both sides of it takes a kernel with both forms, which costs the other
+// populations up to 6 %.
+__host__ __device__ inline bool density_by_particles(int N, int words) { return N <= 4 + (words < 4 ? words : 4); }
+enum DensityForm { kBySites = 0, kByParticles = 1, kByPopulation = 2 };
+
+template <int W, int FORM>
 __global__ void __launch_bounds__(kThreads) k_density(Batch B, const float2* cs, double* tile_acc) {
   __shared__ double s_part[kWarps];
   __shared__ float4 s_cs[32 * (W > 0 ? W : 8)];  // pairs of sites; wide lattices 8 words at a time
@@ -1975,52 +1984,70 @@ __global__ void __launch_bounds__(kThreads) k_density(Batch B, const float2* cs,
   const float2* tab = cs + (size_t)p * kInvStride;
   const int64_t base = (int64_t)tile * kTile;
   const int nw = W > 0 ? W : B.W;
-  float c[kItems], sn[kItems];
-#pragma unroll
-  for (int i = 0; i < kItems; ++i) c[i] = sn[i] = 0.0f;
-  for (int w0 = 0; w0 < nw; w0 += WB) {
-    __syncthreads();
-    for (int e = tid; e < 32 * WB; e += kThreads) {
-      const int x = 64 * w0 + 2 * e;
-      const float2 a = x < d.L ? tab[x] : make_float2(0.0f, 0.0f);
-      const float2 b = x + 1 < d.L ? tab[x + 1] : make_float2(0.0f, 0.0f);
-      s_cs[e] = make_float4(a.x, a.y, b.x, b.y);
-    }
-    __syncthreads();
-    for (int w = 0; w < WB && w0 + w < nw; ++w) {
-      uint32_t v[kItems][2];
-#pragma unroll
-      for (int i = 0; i < kItems; ++i) {
-        const int64_t slot = base + i * kThreads + tid;
-        const unsigned long long x = slot - d.off < d.nc ? B.Y[slot * nw + w0 + w] : 0ull;
-        v[i][0] = (uint32_t)x;
-        v[i][1] = (uint32_t)(x >> 32);
-      }
-#pragma unroll
-      for (int hf = 0; hf < 2; ++hf)
-#pragma unroll 4
-        for (int e = 0; e < 16; ++e) {
-          const float4 q = s_cs[32 * w + 16 * hf + e];
-#pragma unroll
-          for (int i = 0; i < kItems; ++i) {
-            if (v[i][hf] & 1u) {
-              c[i] = __fadd_rn(c[i], q.x);
-              sn[i] = __fadd_rn(sn[i], q.y);
-            }
-            if (v[i][hf] & 2u) {
-              c[i] = __fadd_rn(c[i], q.z);
-              sn[i] = __fadd_rn(sn[i], q.w);
-            }
-            v[i][hf] >>= 2;
-          }
-        }
-    }
-  }
   double acc = 0.0;
+  auto mode = [&](float re, float im) {
+    return (double)__fdiv_rn(__fadd_rn(__fmul_rn(re, re), __fmul_rn(im, im)), (float)d.L);
+  };
+  if (FORM == kByParticles || (FORM == kByPopulation && density_by_particles(d.N, nw))) {
+    for (int64_t slot = base + tid; slot < min(base + kTile, d.off + d.nc); slot += kThreads) {
+      float c = 0.0f, sn = 0.0f;
+      for (int w = 0; w < nw; ++w) {
+        unsigned long long bits = B.Y[slot * nw + w];
+        while (bits) {
+          const float2 v = tab[64 * w + __ffsll((long long)bits) - 1];
+          c = __fadd_rn(c, v.x);
+          sn = __fadd_rn(sn, v.y);
+          bits &= bits - 1ull;
+        }
+      }
+      acc += mode(c, sn);
+    }
+  } else {
+    float c[kItems], sn[kItems];
 #pragma unroll
-  for (int i = 0; i < kItems; ++i)
-    if (base - d.off + i * kThreads + tid < d.nc)
-      acc += (double)__fdiv_rn(__fadd_rn(__fmul_rn(c[i], c[i]), __fmul_rn(sn[i], sn[i])), (float)d.L);
+    for (int i = 0; i < kItems; ++i) c[i] = sn[i] = 0.0f;
+    for (int w0 = 0; w0 < nw; w0 += WB) {
+      __syncthreads();
+      for (int e = tid; e < 32 * WB; e += kThreads) {
+        const int x = 64 * w0 + 2 * e;
+        const float2 a = x < d.L ? tab[x] : make_float2(0.0f, 0.0f);
+        const float2 b = x + 1 < d.L ? tab[x + 1] : make_float2(0.0f, 0.0f);
+        s_cs[e] = make_float4(a.x, a.y, b.x, b.y);
+      }
+      __syncthreads();
+      for (int w = 0; w < WB && w0 + w < nw; ++w) {
+        uint32_t v[kItems][2];
+#pragma unroll
+        for (int i = 0; i < kItems; ++i) {
+          const int64_t slot = base + i * kThreads + tid;
+          const unsigned long long x = slot - d.off < d.nc ? B.Y[slot * nw + w0 + w] : 0ull;
+          v[i][0] = (uint32_t)x;
+          v[i][1] = (uint32_t)(x >> 32);
+        }
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf)
+#pragma unroll 4
+          for (int e = 0; e < 16; ++e) {
+            const float4 q = s_cs[32 * w + 16 * hf + e];
+#pragma unroll
+            for (int i = 0; i < kItems; ++i) {
+              if (v[i][hf] & 1u) {
+                c[i] = __fadd_rn(c[i], q.x);
+                sn[i] = __fadd_rn(sn[i], q.y);
+              }
+              if (v[i][hf] & 2u) {
+                c[i] = __fadd_rn(c[i], q.z);
+                sn[i] = __fadd_rn(sn[i], q.w);
+              }
+              v[i][hf] >>= 2;
+            }
+          }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kItems; ++i)
+      if (base - d.off + i * kThreads + tid < d.nc) acc += mode(c[i], sn[i]);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) s_part[wid] = acc;

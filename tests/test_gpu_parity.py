@@ -907,3 +907,19 @@ def test_setting_one_tuned_parameter_leaves_the_others(pg):
         assert c.get_tuning() == before
     with pytest.raises(pg.PopError):
         a.set_tuning(fuse_threads=256, fuse_clones=2)
+
+
+@pytest.mark.parametrize("rings", [[(50, 0), (64, 1), (64, 5), (64, 6), (20, 20)], [(128, 6), (128, 7), (65, 1), (40, 7)],
+                                   [(256, 8), (256, 9), (30, 8)], [(1025, 8), (1025, 9), (4096, 2), (17, 1)],
+                                   [(64, 5), (30, 0), (64, 1)], [(128, 6), (100, 3)], [(4096, 8), (200, 1)]])
+def test_density_mode_of_few_particles_matches_oracle(pg, rings):
+    # either side of the line between the sums by particles and by sites, rings shorter than
+    # the batch's words among them; a tile and a ragged one.  Both sum a clone in FP32 in the
+    # order of the sites, so only the FP64 sum over the clones may differ
+    pops = [dict(L=L, N=N, n_clones=1025 + 3 * i, seed=500 + i) for i, (L, N) in enumerate(rings)]
+    b = pg.PopulationBatch(pops)
+    orcs = [oracle.Population(q["L"], q["N"], q["n_clones"], q["seed"]) for q in pops]
+    for n in (1, 2):
+        got = b.density_mode(n)
+        for p, o in enumerate(orcs):
+            np.testing.assert_allclose(got[p], oracle.density_mode(o.sites, n), rtol=1e-12, err_msg=str(rings[p]))
