@@ -923,3 +923,113 @@ def test_density_mode_of_few_particles_matches_oracle(pg, rings):
         got = b.density_mode(n)
         for p, o in enumerate(orcs):
             np.testing.assert_allclose(got[p], oracle.density_mode(o.sites, n), rtol=1e-12, err_msg=str(rings[p]))
+
+
+# what the forms of the fused kernel differ in beside RUN_CASES: MODIFIED weights and rings
+# that fill their words in populations of more than 64 tiles, which scan their tile sums
+FORM_CASES = dict({k: v for k, v in RUN_CASES.items() if k != "iid_unfused"},
+                  w1_modified_scan=([dict(L=30, N=15, n_clones=65 * 1024 + 5, seed=27, weight_mode=1),
+                                     dict(L=64, N=32, n_clones=66 * 1024, seed=28)], [0.05, -0.01], [4]),
+                  w1_full_modified=([dict(L=64, N=32, n_clones=3000, seed=29, weight_mode=1)], [0.02], [4]),
+                  w1_full_scan=([dict(L=64, N=32, n_clones=66 * 1024, seed=30)], [0.02], [4]),
+                  w2_full_scan=([dict(L=128, N=64, n_clones=65 * 1024 + 1, seed=31)], [0.01], [4]),
+                  w2_modified_scan=([dict(L=100, N=50, n_clones=65 * 1024 + 1, seed=32, weight_mode=1)], [0.01], [4]),
+                  w2_full_modified_scan=([dict(L=128, N=64, n_clones=65 * 1024 + 1, seed=33, weight_mode=1)], [0.01], [4]))
+
+
+@pytest.mark.parametrize("form", [dict(fuse_threads=128, fuse_clones=1), dict(fuse_threads=128, fuse_clones=2),
+                                  dict(fuse_threads=256, fuse_clones=1)], ids=["128", "128x2", "256"])
+@pytest.mark.parametrize("case", sorted(FORM_CASES))
+def test_every_form_of_the_fused_stage_equals_steps(pg, case, form):
+    pops, s, splits = FORM_CASES[case]
+    a = pg.PopulationBatch(pops)
+    a.set_tuning(**form)
+    b = pg.PopulationBatch(pops)
+    for n in splits:
+        a.run(0.1, s, n)
+    for _ in range(sum(splits)):
+        b.evolve(0.1, s)
+        b.resample()
+    for p in range(len(pops)):
+        ga, gb = a.copy_state(p), b.copy_state(p)
+        for key in ("lattice", "K", "anc", "dK"):
+            assert np.array_equal(ga[key], gb[key]), (p, key)
+    pa, _, ta = a.estimate_psi()
+    pb, _, tb = b.estimate_psi()
+    np.testing.assert_allclose(pa * ta, pb * tb, rtol=1e-15)
+    np.testing.assert_array_equal(a.events(), b.events())
+
+
+def test_step_limit_of_every_stage(pg, tmp_path):
+    # a library whose step limit is 64 steps (32 draws) per interval: intervals within it give
+    # what the ordinary library gives (a lane of the fused stage makes more draws than that, of
+    # several clones), longer ones end and are reported, by every form of every stage
+    import ctypes
+    import subprocess
+    from paper_1711_05095_gb300 import build as b
+    so = str(tmp_path / "libpop_limit.so")
+    subprocess.run([b.nvcc(), "-O3", "-std=c++17", *b.ARCH, "-Xcompiler", "-fPIC", "-shared", "-DPOP_STEP_LIMIT=64u",
+                    "-I", b.ROOT + "/include", *b.SOURCES, "-o", so], check=True)
+    forms = [dict(fuse_threads=128, fuse_clones=1), dict(fuse_threads=128, fuse_clones=2),
+             dict(fuse_threads=256, fuse_clones=1)]
+    batches = [[dict(L=20, N=10, n_clones=9000, seed=95)], [dict(L=20, N=10, n_clones=5000, seed=96, weight_mode=MOD)],
+               [dict(L=20, N=10, n_clones=5000, seed=97), dict(L=100, N=2, n_clones=3000, seed=98)],
+               [dict(L=100, N=2, n_clones=3000, seed=99, weight_mode=MOD)]]
+    small = [[dict(L=20, N=10, n_clones=700, seed=85)], [dict(L=100, N=2, n_clones=1000, seed=86, weight_mode=MOD)]]
+    s = [0.3, 0.1]
+
+    def run(q, dt, n, form):
+        a = pg.PopulationBatch(q)
+        if form:
+            a.set_tuning(**form)
+        a.run(dt, s[:len(q)], n)
+        return a
+
+    # at rate 10.5 (L = 20) or 4 an interval of 1 takes 6 draws, hardly ever 32
+    want = []
+    for q in batches + small:
+        x = run(q, 1.0, 6, None)
+        want.append([x.copy_state(p) for p in range(len(q))])
+        x.close()
+    saved, path = pg._lib, pg.LIB_PATH
+    try:
+        pg._lib, pg.LIB_PATH = None, so
+        for i, q in enumerate(batches + small):
+            for form in forms if i < len(batches) else [None]:
+                x = run(q, 1.0, 6, form)
+                for p in range(len(q)):
+                    g = x.copy_state(p)
+                    for key in ("lattice", "K", "anc", "dK"):
+                        assert np.array_equal(g[key], want[i][p][key]), (i, form, p, key)
+                x.close()
+        # the first interval, by the separate dynamical stage, stays within the limit (61, 62, 62
+        # and 61 hops at most, by the oracle); of the other 39, by the fused stage or the
+        # one-tile launch, several do not
+        for q, dt in (([dict(L=20, N=10, n_clones=9000, seed=81)], 3.4),
+                      ([dict(L=20, N=10, n_clones=9000, seed=82, weight_mode=MOD)], 3.4 / np.e),
+                      ([dict(L=20, N=10, n_clones=9000, seed=83), dict(L=80, N=0, n_clones=3000, seed=84)], 3.2),
+                      ([dict(L=20, N=10, n_clones=1024, seed=85)], 3.4)):
+            sq = [-1.0] * len(q)
+            x = pg.PopulationBatch(q)
+            x.evolve(dt, sq)
+            assert int(x.events()[0]) > 0          # no error
+            x.close()
+            for form in forms:
+                x = pg.PopulationBatch(q)
+                x.set_tuning(**form)
+                x.run(dt, sq, 40)
+                with pytest.raises(pg.PopError) as e:
+                    x.events()
+                assert e.value.status == pg.POP_ERR_RANGE
+                x.close()
+        # the dynamical stages
+        for q in ([dict(L=20, N=10, n_clones=500, seed=87)], [dict(L=200, N=3, n_clones=50, seed=88)],
+                  [dict(L=40, N=20, n_clones=50, seed=89, weight_mode=pg.POP_GUIDED)]):
+            x = pg.PopulationBatch(q)
+            x.evolve(50.0, [0.0])
+            with pytest.raises(pg.PopError) as e:
+                x.events()
+            assert e.value.status == pg.POP_ERR_RANGE
+            x.close()
+    finally:
+        pg._lib, pg.LIB_PATH = saved, path
