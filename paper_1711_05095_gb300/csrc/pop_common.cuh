@@ -213,94 +213,11 @@ __device__ __forceinline__ float neg_ln_u(uint32_t w, const float2* tab) {
 // Lattice helpers.  A clone is W 64-bit words; site i is bit i%64 of word i/64.
 // Bond i joins sites i and (i+1) mod L; it is active (a hop across it is
 // possible) when exactly one end is occupied: a = x XOR rot(x), rot(x)_i = x_{i+1}.
-// ---------------------------------------------------------------------------
-template <int W>
-__device__ __forceinline__ void active_bonds(const unsigned long long (&x)[W], int L,
-                                             unsigned long long (&a)[W]) {
-  if constexpr (W == 1) {
-    const unsigned long long rot = (x[0] >> 1) | ((x[0] & 1ull) << (L - 1));
-    a[0] = x[0] ^ rot;
-  } else {
-    if (L <= 64) {
-      const unsigned long long rot = (x[0] >> 1) | ((x[0] & 1ull) << (L - 1));
-      a[0] = x[0] ^ rot;
-      a[1] = 0ull;
-    } else {
-      const unsigned long long r0 = (x[0] >> 1) | (x[1] << 63);
-      const unsigned long long r1 = (x[1] >> 1) | ((x[0] & 1ull) << (L - 65));
-      a[0] = x[0] ^ r0;
-      a[1] = x[1] ^ r1;
-    }
-  }
-}
-
-template <int W>
-__device__ __forceinline__ int popc_lat(const unsigned long long (&a)[W]) {
-  if constexpr (W == 1) return __popcll(a[0]);
-  else return __popcll(a[0]) + __popcll(a[1]);
-}
-
-// Position of the k-th (0-based) set bit of a, k < popc(a): binary descent on the
-// population counts of halves.
-__device__ __forceinline__ int kth_set_bit64(unsigned long long a, uint32_t k) {
-  uint32_t x = (uint32_t)a;
-  int pos = 0;
-  uint32_t c = (uint32_t)__popc(x);
-  if (k >= c) { k -= c; x = (uint32_t)(a >> 32); pos = 32; }
-  c = (uint32_t)__popc(x & 0xffffu);
-  if (k >= c) { k -= c; x >>= 16; pos += 16; }
-  c = (uint32_t)__popc(x & 0xffu);
-  if (k >= c) { k -= c; x >>= 8; pos += 8; }
-  c = (uint32_t)__popc(x & 0xfu);
-  if (k >= c) { k -= c; x >>= 4; pos += 4; }
-  c = (uint32_t)__popc(x & 0x3u);
-  if (k >= c) { k -= c; x >>= 2; pos += 2; }
-  c = x & 1u;
-  if (k >= c) { pos += 1; }
-  return pos;
-}
-
-template <int W>
-__device__ __forceinline__ int kth_bond(const unsigned long long (&a)[W], uint32_t k) {
-  if constexpr (W == 1) {
-    return kth_set_bit64(a[0], k);
-  } else {
-    const uint32_t c0 = (uint32_t)__popcll(a[0]);
-    const bool lo = k < c0;
-    return kth_set_bit64(lo ? a[0] : a[1], lo ? k : k - c0) + (lo ? 0 : 64);
-  }
-}
-
-// A hop across bond b swaps the occupations of sites b and (b+1) mod L, which
-// differ, so both bits flip: bits b, b+1 (or b and 0 for the closing bond L-1).
-template <int W>
-__device__ __forceinline__ void hop(unsigned long long (&x)[W], int b, int L) {
-  if constexpr (W == 1) {
-    x[0] ^= (b + 1 == L) ? ((1ull << b) | 1ull) : (3ull << b);
-  } else {
-    unsigned long long m0, m1;
-    if (b + 1 == L) {
-      m0 = 1ull | (b < 64 ? (1ull << b) : 0ull);
-      m1 = b >= 64 ? (1ull << (b - 64)) : 0ull;
-    } else if (b < 63) {
-      m0 = 3ull << b;
-      m1 = 0ull;
-    } else if (b == 63) {
-      m0 = 1ull << 63;
-      m1 = 1ull;
-    } else {
-      m0 = 0ull;
-      m1 = 3ull << (b - 64);
-    }
-    x[0] ^= m0;
-    x[1] ^= m1;
-  }
-}
-
-// The same lattice operations on 32-bit words (u[j] holds sites [32j, 32j + 32)),
-// the ALU's native width.  Shifts that may fall outside a word use the clamped
+// In registers a clone is 2W 32-bit words (u[j] holds sites [32j, 32j + 32)), the ALU's
+// native width.  Shifts that may fall outside a word use the clamped
 // funnel shift: __funnelshift_lc(0, v, n) = v << min(n, 32), which is 0 for n >= 32
 // and, with n formed in unsigned arithmetic, for "negative" n too.
+// ---------------------------------------------------------------------------
 template <int W>
 __device__ __forceinline__ void split32(const unsigned long long (&x)[W], uint32_t (&u)[2 * W]) {
 #pragma unroll

@@ -604,9 +604,6 @@ __global__ void __launch_bounds__(kScanThreads, 3) k_tile_scan(Batch B, int pop0
 #ifndef POP_GATHER_THREADS
 #define POP_GATHER_THREADS 128
 #endif
-#ifndef POP_FUSE_THREADS
-#define POP_FUSE_THREADS 128
-#endif
 #ifndef POP_FUSE_MIN_BLOCKS
 #define POP_FUSE_MIN_BLOCKS 8  // 64 registers, no spills; pop_run's chains keep more than one launch resident
 #endif
