@@ -100,6 +100,7 @@ struct PopState {
   unsigned long long T;        // total weight of this interval (k_tile_scan or k_gather)
   unsigned long long pos_m;    // PosScale of T (k_tile_scan)
   int32_t pos_sh;
+  int32_t copy_par;            // wide lattices: parity of the words k_copy_wide copies, -1: none
   uint32_t done;               // k_run_small, population 0: blocks that have ended
   int32_t stuck;               // k_run_small reached the step limit: its later launches run no interval
 };

@@ -1139,6 +1139,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
       if (ovf) st->hovf = 1;
     }
   } else if (iid) {
+    if (W == 0 && lt == 0 && tid == 0) st->copy_par = par;
     int32_t* const guide = B.dKb[par ^ 1];  // the last interval's activities are no longer needed
     for (uint32_t jj = J0 + (uint32_t)tid; jj < J1; jj += NT) guide[d.off + (int64_t)jj] = lt * kTile + source(jj);
   } else if constexpr (W > 0) {
@@ -1154,6 +1155,7 @@ __global__ void __launch_bounds__(NT, FUSE ? (NCL == 1 ? POP_FUSE_MIN_BLOCKS * 1
     }
   } else {
     // wide lattices: the ancestors here, their words by k_copy_wide
+    if (lt == 0 && tid == 0) st->copy_par = s_T == 0ull ? -1 : par;
     for (uint32_t jj = J0 + (uint32_t)tid; jj < J1; jj += NT) {
       const int k = source(jj);
       const int64_t dst = d.off + (int64_t)jj;
@@ -1527,7 +1529,9 @@ __global__ void __launch_bounds__(kThreads) k_select_iid(Batch B) {
       const uint4 r = philox4x32_10(make_uint4(j, beta, 0u, kTagIid), k0, k1);
       const unsigned long long u64 = ((unsigned long long)r.y << 32) | r.x;
       alpha[i] = __umul64hi(u64, T);
-      k[i] = guide[(int)__umul64hi(u64, (unsigned long long)nc)];
+      // without any weight (MODIFIED, e^-s beyond FP32) there are no guide entries, and every
+      // prefix sum is at or before alpha_j = 0: the last clone
+      k[i] = T != 0ull ? guide[(int)__umul64hi(u64, (unsigned long long)nc)] : nc - 1;
     }
 #pragma unroll
     for (int i = 0; i < kItems; ++i) {
@@ -1939,16 +1943,21 @@ __global__ void __launch_bounds__(kThreads) k_copy_wide(Batch B) {
   const int tile = blockIdx.x;
   const int p = B.tile_pop[tile];
   const PopDesc d = B.pops[p];
-  const int par = (int)(B.st[p].beta & 1u);
-  const unsigned long long* const X = B.Xb[par] + d.off * B.W;
+  const int par = B.st[p].copy_par;
   const int64_t base = (int64_t)tile * kTile;
-  const int n = (int)min((int64_t)kTile, d.nc - (base - d.off));
   const uint32_t W = (uint32_t)B.W;
+  int32_t a[kItems];
+#pragma unroll
+  for (int i = 0; i < kItems; ++i)  // the tile's padding included, so that no load waits for the parity
+    a[i] = B.anc[base + (blockIdx.y * kTile + i * kThreads + threadIdx.x) / W];
+  // without weights (par < 0) [eq] has no new clones, and the ancestors are old
+  const int n = par < 0 ? 0 : (int)min((int64_t)kTile, d.nc - (base - d.off));
+  const unsigned long long* const X = B.Xb[par & 1] + d.off * B.W;
 #pragma unroll
   for (int i = 0; i < kItems; ++i) {
     const uint32_t e = blockIdx.y * kTile + i * kThreads + threadIdx.x;  // word of the tile
     const uint32_t j = e / W, q = e - j * W;
-    if ((int)j < n) B.Y[(base + j) * W + q] = X[(int64_t)B.anc[base + j] * W + q];
+    if ((int)j < n) B.Y[(base + j) * W + q] = X[(int64_t)a[i] * W + q];
   }
 }
 

@@ -1033,3 +1033,26 @@ def test_step_limit_of_every_stage(pg, tmp_path):
             x.close()
     finally:
         pg._lib, pg.LIB_PATH = saved, path
+
+
+@pytest.mark.parametrize("L,nc", [(20, 3), (20, 1500), (100, 2100), (300, 70)])
+def test_a_population_without_weights_selects_in_range(pg, L, nc):
+    # MODIFIED weights at e^-s beyond FP32: infinity times the clones' differences, so every
+    # weight is 0 or not a number, which counts as 0.  [iid]: every point lies at the last
+    # clone; [eq]: no point, so the clones stay as they are.  dt = 1e-38 at rates 4.5e38 makes
+    # some 45 hops per clone, more than the smallest population has clones
+    q = dict(L=L, N=L // 2, n_clones=nc, weight_mode=MOD)
+    b = pg.PopulationBatch([dict(q, seed=610, selection=IID), dict(q, seed=611)])
+    for _ in range(3):
+        before = b.copy_state(1)
+        b.evolve(1e-38 if L == 20 else 2e-39, [-89.0, -89.0])
+        x = b.copy_state(0)
+        assert x["dK"].max() > 3
+        b.resample()
+        g = b.copy_state(0)
+        assert (g["anc"] == nc - 1).all()
+        assert np.array_equal(g["lattice"], np.repeat(x["lattice"][-1:], nc, axis=0))
+        assert np.array_equal(g["K"], np.repeat(x["K"][-1:], nc))
+        after = b.copy_state(1)
+        assert np.array_equal(after["lattice"], before["lattice"]) and np.array_equal(after["K"], before["K"])
+    assert not np.isfinite(b.estimate_psi()[0]).any()
