@@ -161,7 +161,8 @@ int pop_run(pop_t* pop, double dt, const double* s, int64_t n_intervals);
  * waves of the fused kernel on this device or has at least 8 populations; up to 2 for a
  * larger one of fewer) for which the
  * population starts nearest k/K of the tiles (k = 1 .. K-1) leave every chain at least
- * half of its equal share.
+ * half of its equal share.  A batch that pop_run advances by whole intervals in one launch
+ * (see there) has no chains; the split it would have otherwise is what is reported.
  */
 int32_t pop_run_chains(pop_t* pop, int32_t* h_first_tiles);
 
@@ -187,7 +188,9 @@ int pop_copy_state(pop_t* pop, int32_t p, uint64_t* h_lattice, int32_t* h_K,
 
 /*
  * Launch configuration of a batch (the paper has none: its codes had fixed thread
- * counts).  Every choice changes only speed, never a result:
+ * counts).  Every choice changes only speed, never a result; of a batch that pop_run
+ * advances by whole intervals in one launch, evolve_grid and gather_threads apply to the
+ * per-step calls and the others to nothing:
  *   evolve_grid     persistent grid of the separate dynamical stage (the first interval
  *                   of a fused run; every interval of a batch that does not fuse)
  *   fuse_threads    threads per block of the fused cloning + dynamical stage: 128, 256, or

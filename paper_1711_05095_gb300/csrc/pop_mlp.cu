@@ -202,14 +202,14 @@ __global__ void __launch_bounds__(256) k_forward(Work w) {
 // number, split into 16 low bits (unsigned) and the rest (signed), one native 32-bit add
 // each.  A chunk has at most kChunkCfg configurations of at most 32 groups, so no bin
 // leaves 32 bits.  The scale takes the largest |d| of the block's chunk into [2^29, 2^30);
-// the terms of its binary order and the six below keep 24 bits or more, as in an FP32 sum,
-// and are added; those below them are left to a pass of their own, scaled by the largest
-// of them, and so on: a network near its start needs one pass, one that is sure of many
-// configurations several (2^18 configurations of L = 128, the initial network's last layer
-// 10 and 30 times as large: 88 and 95 us per gradient, 82 as it is; in one pass, 83 for all
-// of them, small terms beside a large one lost their digits).  So a term's rounding is at most 2^-24 of
-// it, and the sums of a pass are exact.  Non-finite d take a plain FP64 path that gives the
-// same infinities and NaN.
+// the terms of its binary order and the six below are added, with 24 bits or more as in an
+// FP32 sum; those below them are left to a pass of their own, scaled by the largest of
+// them, and so on.  So a term's rounding is at most 2^-24 of it, and the sums of a pass are
+// exact.  A network near its start needs one pass, one that is sure of many configurations
+// several (2^18 configurations of L = 128: 82 us per gradient with the initial network, 88
+// and 95 with its last layer 10 and 30 times as large; in one pass, 83 for all of them,
+// small terms beside a large one lost their digits).  Non-finite d take a plain FP64 path
+// that gives the same infinities and NaN.
 // A gradient of 16384 configurations of L = 128, its read-back included: 151 us with a
 // thread per configuration and FP32 adds per window (55 us of it here) in nine launches,
 // 56 us now; of 2^20: 493 us, now 108.
