@@ -360,7 +360,8 @@ int pop_events(pop_t* pop, uint64_t* h_events);
  * inside the graph).  Any output may be NULL; each is a host array of POP_NKINDS:
  *   h_us    per kind, the time during which at least one of its launches runs (the
  *           union of their start-to-end ranges), divided by the number of intervals
- *           that launch it, microseconds (one chain: the mean launch time; 0 if none)
+ *           that launch it or that it runs (launches of whole intervals), microseconds
+ *           (one chain: the mean launch time; 0 if none)
  *   h_n     number of launches of each kind
  *   h_hops  hops executed by the launches of each kind (nonzero only for the kinds
  *           that run dynamical stages)

@@ -1240,6 +1240,7 @@ int pop_kernel_times(pop_t* h, double dt, const double* s, int64_t n_intervals, 
     if (hi > lo) sum += hi - lo;
     int64_t groups = 0;
     for (char c : seen[k]) groups += c;
+    if (small && k == POP_K_GATHER_EVOLVE) groups = n_intervals;  // whole intervals in a launch
     if (h_us) h_us[k] = groups ? 1e3 * sum / (double)groups : 0.0;
     if (h_n) h_n[k] = cnt[k];
     if (h_hops) h_hops[k] = 0;

@@ -1056,3 +1056,13 @@ def test_a_population_without_weights_selects_in_range(pg, L, nc):
         after = b.copy_state(1)
         assert np.array_equal(after["lattice"], before["lattice"]) and np.array_equal(after["K"], before["K"])
     assert not np.isfinite(b.estimate_psi()[0]).any()
+
+
+def test_kernel_times_of_one_tile_populations_are_per_interval(pg):
+    # a launch of 30 intervals and launches of 3000: both some microseconds per interval
+    us = []
+    for n in (30, 3000):
+        b = pg.PopulationBatch([dict(L=20, N=10, n_clones=1000, seed=77)])
+        b.kernel_times(0.1, [0.05], 30)   # warm
+        us.append(b.kernel_times(0.1, [0.05], n)["gather_evolve"][0])
+    assert 0.2 < us[0] / us[1] < 5.0, us  # a sum over the launch would be a hundredth
