@@ -217,6 +217,7 @@ struct pop_batch {
   bool any_mod = false;
   bool guided = false;       // every population GUIDED
   bool guided_q_stale = true; // GUIDED: the rate tables need (re)building once s is fixed
+  int64_t chunks = 0;         // of clones, for the dynamical stage (PopDesc::chunk0)
   int evolve_grid = 0;
   int evolve_grid_cap = 0;  // persistent grid at full occupancy
   int small_threads = 0;    // pop_run in one launch (k_run_small): threads per block, 0: not
@@ -627,16 +628,17 @@ int size_chains(pop_t* h) {
   return POP_OK;
 }
 
-// Split the slots over a persistent grid of k_evolve: an even share of the chunks of
-// 32 / G slots (what a warp holds at a time) to each warp.
+// Split the clones over a persistent grid of k_evolve: an even share of the chunks of 32 / G
+// clones (what a warp holds at a time) to each warp.  Of clones, not of slots: a population
+// fills its tiles only in part (1024 populations of 300 clones, L = 50, dt = 2, [iid]:
+// 200 us per interval with shares of slots, 132 so).
 void set_evolve_grid(pop_t* h, int grid) {
-  const int64_t chunks = h->lay.nslots / (32 / evolve_lanes(h));
-  const int64_t most = (chunks + kEvolveWarps - 1) / kEvolveWarps;
+  const int64_t most = (h->chunks + kEvolveWarps - 1) / kEvolveWarps;
   if (grid < 1) grid = 1;
   if (grid > most) grid = (int)most;
   h->evolve_grid = grid;
-  h->B.unit_q = chunks / ((int64_t)grid * kEvolveWarps);
-  h->B.unit_r = chunks % ((int64_t)grid * kEvolveWarps);
+  h->B.unit_q = h->chunks / ((int64_t)grid * kEvolveWarps);
+  h->B.unit_r = h->chunks % ((int64_t)grid * kEvolveWarps);
 }
 
 // As many blocks as fit on the device at once (or as there are chunks for).
@@ -862,6 +864,8 @@ int pop_init(pop_t** out, const pop_params* params, int32_t n_pops, void* d_work
     h->guided = d.guided != 0;
     h->any_mod = h->any_mod || d.modified;
     h->B.any_iid = h->B.any_iid || d.iid;
+    d.chunk0 = h->chunks;
+    h->chunks += (d.nc + 32 / evolve_lanes(h) - 1) / (32 / evolve_lanes(h));
     for (int32_t t = 0; t < d.ntiles; ++t) tile_pop[(size_t)tile + t] = p;
     tile += d.ntiles;
   }
@@ -951,6 +955,7 @@ int pop_init(pop_t** out, const pop_params* params, int32_t n_pops, void* d_work
   B.dKb[0] = (int32_t*)(ws + lay.o_dK);
   B.dKb[1] = B.dKb[0] + lay.nslots;
   B.anc = (int32_t*)(ws + lay.o_anc);
+  B.P = lay.P;
   B.ntiles = lay.ntiles;
   B.nslots = lay.nslots;
   B.W = lay.W;

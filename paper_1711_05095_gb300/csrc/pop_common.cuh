@@ -76,6 +76,7 @@ struct PopDesc {
   double abs_s;
   int32_t s_q;       // GUIDED: s in units of 2^-17 (nearest integer)
   float c_s;         // GUIDED: float(s_q 2^-17 - s)
+  int64_t chunk0;    // chunks of clones (k_evolve: 32 / G each) in the populations before
 };
 
 // Mutable per population.
@@ -141,7 +142,8 @@ struct Batch {
   int32_t ntiles;
   int64_t nslots;
   int32_t W;                            // lattice words per clone
-  int64_t unit_q, unit_r;               // k_evolve: chunks of 32 / G slots = unit_q * warps + unit_r
+  int64_t unit_q, unit_r;               // k_evolve: chunks of 32 / G clones = unit_q * warps + unit_r
+  int32_t P;                            // populations
   int32_t any_iid;                      // some population selects [iid]: k_select_iid runs last
 };
 

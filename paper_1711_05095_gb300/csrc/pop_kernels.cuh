@@ -115,7 +115,7 @@ __device__ __forceinline__ bool bkl_step_pred(uint32_t (&u)[2 * W], float& t, fl
 // bond lies in the lane whose range of an exclusive prefix of the lanes' counts holds k,
 // and the draw, the waiting time and the bond are the same on every lane of the group
 // (the same arithmetic as with one lane, so the same results).
-// A persistent grid: each warp has an even share of the slots and walks it population by
+// A persistent grid: each warp has an even share of the clones and walks it population by
 // population (it drains at the end of each: by tiles, 395 us per interval of the [iid] study);
 // a group whose clone ended takes the share's next clone, so a warp needs no barrier and
 // no shared counter.  Clones go from global memory to registers and back.
@@ -213,6 +213,20 @@ __device__ __forceinline__ bool wide_step_pred(uint32_t (&u)[8], float& t, float
   return hopped;
 }
 
+// The population that holds a chunk of the batch's clones (PopDesc::chunk0, ascending; every
+// population has one at least), searched by 32 pivots at a time.
+__device__ __forceinline__ int population_of_chunk(const Batch& B, int64_t chunk, int lane) {
+  int p = 0, n = B.P;
+  while (n > 1) {
+    const int step = (n + 31) / 32, at = lane * step;
+    const bool le = at < n && B.pops[p + min(at, n - 1)].chunk0 <= chunk;
+    const int k = (31 - __clz((int)__ballot_sync(0xffffffffu, le))) * step;
+    p += k;
+    n = min(step, n - k);
+  }
+  return p;
+}
+
 // FULL: every ring fills the words (L = 32 NW), so there is no padding to keep.
 // COUNT64: the hops of a lane's share are counted in 64 bits, where they may not fit 32 (the
 // host's rule; beside the steps that costs a register, 2.5 % of the [iid] study's time, and
@@ -241,17 +255,14 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
   for (int i = 0; i < 32; i += G) leaders |= 1u << i;
   const unsigned int before = leaders & ((1u << lead) - 1u);
   const int W = NW == 8 ? B.W : W64;
-  // the warp's share of the slots: B.unit_q chunks of 32 / G slots each and one more for
-  // the first B.unit_r warps
+  // the warp's share: B.unit_q chunks of 32 / G clones and one more for the first B.unit_r warps
   const int64_t wi = (int64_t)blockIdx.x * kEvolveWarps + wid;
-  int64_t slot0 = (wi * B.unit_q + min(wi, B.unit_r)) * (32 / G);
-  const int64_t slot_end = slot0 + (B.unit_q + (wi < B.unit_r ? 1 : 0)) * (32 / G);
-  while (slot0 < slot_end) {
-    const int p = B.tile_pop[slot0 / kTile];
+  int64_t chunk = wi * B.unit_q + min(wi, B.unit_r);
+  const int64_t chunk_end = chunk + B.unit_q + (wi < B.unit_r ? 1 : 0);
+  for (int p = population_of_chunk(B, chunk, lane); chunk < chunk_end; ++p) {
     const PopDesc d = B.pops[p];
-    const int64_t seg_end = min(slot_end, d.off + (int64_t)d.ntiles * kTile);  // within one population
-    const int64_t j0 = slot0 - d.off;
-    const int n = (int)max((int64_t)0, min(seg_end - slot0, d.nc - j0));  // warp-uniform
+    const int64_t j0 = (chunk - d.chunk0) * (32 / G), slot0 = d.off + j0;
+    const int n = (int)min((chunk_end - chunk) * (32 / G), d.nc - j0);  // warp-uniform, at least 1
     const float* inv = B.inv_rate + (size_t)p * kInvStride;
     if (lane < 10)
       s_key[wid][lane] = make_uint2((uint32_t)d.seed + (uint32_t)lane * 0x9E3779B9u,
@@ -368,7 +379,7 @@ __global__ void __launch_bounds__(kEvolveThreads, NW == 8 ? 1 : POP_EVOLVE_MIN_B
       }
     }
     __syncwarp();  // the segment's key and factors have been read
-    slot0 = seg_end;
+    chunk += (n + 32 / G - 1) / (32 / G);
   }
 }
 
@@ -1667,7 +1678,7 @@ __device__ __forceinline__ float i64_to_float_rn(long long v) {
 }
 
 // One lane per clone.  A persistent grid as k_evolve's: each warp has an even share of the
-// slots and walks it population by population, a lane whose clone ended takes the share's
+// clones and walks it population by population, a lane whose clone ended takes the share's
 // next one.
 // Per lane in shared memory: the rate sums of the clone's groups of eight bonds and its
 // sites as a bit string that starts eight sites before site 0 and goes on past the closing
@@ -1712,14 +1723,12 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
   const unsigned long long* const gin = B.gcar[par ^ 1];
   unsigned long long* const gout = B.gcar[par];
   const int64_t wi = (int64_t)blockIdx.x * kWarpsG + wid;
-  int64_t slot0 = (wi * B.unit_q + min(wi, B.unit_r)) * 32;
-  const int64_t slot_end = slot0 + (B.unit_q + (wi < B.unit_r ? 1 : 0)) * 32;
-  while (slot0 < slot_end) {
-    const int p = B.tile_pop[slot0 / kTile];
+  int64_t chunk = wi * B.unit_q + min(wi, B.unit_r);
+  const int64_t chunk_end = chunk + B.unit_q + (wi < B.unit_r ? 1 : 0);
+  for (int p = population_of_chunk(B, chunk, lane); chunk < chunk_end; ++p) {
     const PopDesc d = B.pops[p];
-    const int64_t seg_end = min(slot_end, d.off + (int64_t)d.ntiles * kTile);  // within one population
-    const int64_t j0 = slot0 - d.off;
-    const int n = (int)max((int64_t)0, min(seg_end - slot0, d.nc - j0));  // warp-uniform
+    const int64_t j0 = (chunk - d.chunk0) * 32, slot0 = d.off + j0;
+    const int n = (int)min((chunk_end - chunk) * 32, d.nc - j0);  // warp-uniform, at least 1
     const int L = d.L;
     const uint32_t lm1 = (uint32_t)L - 1u;
     const LatWords<NW> pad = pad_mask<NW>((uint32_t)L);
@@ -1928,7 +1937,7 @@ __global__ void __launch_bounds__(kGuideThreads, POP_GUIDE_MIN_BLOCKS) k_evolve_
       atomicMax(&st->a_max[par], xmax);
     }
     __syncwarp();
-    slot0 = seg_end;
+    chunk += (n + 31) / 32;
   }
 }
 

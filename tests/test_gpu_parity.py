@@ -1066,3 +1066,39 @@ def test_kernel_times_of_one_tile_populations_are_per_interval(pg):
         b.kernel_times(0.1, [0.05], 30)   # warm
         us.append(b.kernel_times(0.1, [0.05], n)["gather_evolve"][0])
     assert 0.2 < us[0] / us[1] < 5.0, us  # a sum over the launch would be a hundredth
+
+
+@pytest.mark.parametrize("kind", ["plain", "modified", "wide", "guided"])
+def test_even_shares_of_many_part_filled_populations(pg, kind):
+    # 70 populations (the search for a warp's first one takes two rounds) of 1 to 2051 clones:
+    # shares that begin and end anywhere in them, empty ones included, against the oracle
+    g = np.random.default_rng(7)
+    sizes = [1, 32, 33, 1024, 1025, 2051] + [int(v) for v in np.floor(2.0 ** g.uniform(0, 8, 64))]
+    L = [20 if kind == "guided" else int(v) for v in g.integers(5, 60, 70)]
+    if kind == "wide":
+        L[3] = 300
+    mode = {"modified": MOD, "guided": pg.POP_GUIDED}.get(kind, 0)
+    pops = [dict(L=L[i], N=L[i] // 2, n_clones=sizes[i], seed=700 + i, weight_mode=mode) for i in range(70)]
+    s = [float(v) for v in g.uniform(-0.1, 0.1, 70)]
+    phi = g.normal(0.0, 0.3, 512).astype(np.float32)
+    orcs = []
+    for p, q in enumerate(pops):
+        o = oracle.Population(q["L"], q["N"], q["n_clones"], q["seed"], modified=mode == MOD,
+                              phi=phi if kind == "guided" else None)
+        o.evolve(0.3, s[p])
+        orcs.append(o)
+    for grid in (None, 1, 3, 50):
+        b = pg.PopulationBatch(pops)
+        if kind == "guided":
+            for p in range(70):
+                b.set_potential(p, phi)
+        if grid is not None:
+            b.set_tuning(evolve_grid=grid)
+        b.evolve(0.3, s)
+        events = b.events()
+        for p, o in enumerate(orcs):
+            c = b.copy_state(p)
+            assert np.array_equal(c["lattice"], oracle.sites_to_words(o.sites, b.W)), (grid, p)
+            assert np.array_equal(c["dK"], o.dK) and np.array_equal(c["K"], o.K), (grid, p)
+            assert int(events[p]) == int(o.dK.astype(np.int64).sum())
+        b.close()
