@@ -223,6 +223,7 @@ struct pop_batch {
   int small_threads = 0;    // pop_run in one launch (k_run_small): threads per block, 0: not
   bool s_fixed = false;
   std::vector<double> s;
+  double largest_rate = 0.0;  // of a clone, once s is fixed
   Phase phase = kReady;
   int64_t intervals = 0;
   double t_obs = 0.0;
@@ -317,6 +318,12 @@ int fix_biases(pop_t* h, const double* s) {
   POP_CUDA(cudaStreamSynchronize(h->stream));
   h->s.assign(s, s + h->lay.P);
   h->s_fixed = true;
+  // a ring of N particles on L sites has at most 2 min(N, L - N) active bonds, each with hops
+  // of rate 1 (MODIFIED: e^-s)
+  for (const PopDesc& d : h->desc) {
+    const double r = 2.0 * (double)std::min(d.N, d.L - d.N);
+    h->largest_rate = std::max(h->largest_rate, d.modified ? r * std::exp(-d.s) : r);
+  }
   return guided_rate_tables(h);
 }
 
@@ -378,24 +385,13 @@ EvolveKernel evolve_kernel_of(const pop_t* h) {
   }
 }
 
-// The largest rate of a clone: a ring of N particles on L sites has at most 2 min(N, L - N)
-// active bonds, each with hops of rate 1 (MODIFIED: e^-s).
-double largest_rate(const pop_t* h) {
-  double rate = 0.0;
-  for (const PopDesc& d : h->desc) {
-    const double r = 2.0 * (double)std::min(d.N, d.L - d.N);
-    rate = std::max(rate, d.modified ? r * std::exp(-d.s) : r);
-  }
-  return rate;
-}
-
 // Whether the hops of a warp's share may not fit 32 bits: they are at most a Poisson number
 // of mean share * rate * dt, which does not reach 2^32 from a mean below 2^30 (the exponent
 // of its probability is -2^30 (4 ln 4 - 3)).  From about 2^23 hops per clone on, time in FP32
 // may stand still and hops no longer follow that law.
 bool many_hops(const pop_t* h, float dt_f) {
   const double share = (double)(h->B.unit_q + 1) * (32 / evolve_lanes(h));
-  const double hops = largest_rate(h) * (double)dt_f;
+  const double hops = h->largest_rate * (double)dt_f;
   return !(hops < 1048576.0 && share * hops < 1073741824.0);
 }
 
@@ -696,7 +692,7 @@ int launch_small_form(pop_t* h, cudaStream_t st, float dt_f, int n) {
 constexpr int kSmallIntervals = 1024;
 constexpr double kSmallDraws = 32768.0;
 int small_intervals(const pop_t* h, float dt_f) {
-  const double n = kSmallDraws / (0.5 * largest_rate(h) * (double)dt_f + 1.0);
+  const double n = kSmallDraws / (0.5 * h->largest_rate * (double)dt_f + 1.0);
   return n >= kSmallIntervals ? kSmallIntervals : (n >= 1.0 ? (int)n : 1);
 }
 
